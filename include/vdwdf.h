@@ -149,7 +149,7 @@ typedef struct {
                                  other fields are ignored) */
 typedef struct {
     int32_t threads;      /* threads per CTA: 256, 384, 448, 512 or 1024 (0 = default:
-                             FP32 E + v 448, or 384 on skewed cells; 512 otherwise);
+                             FP32 640, which only the default takes; FP64 512);
                              skewed cells take 384, 448 or 512; VDWDF_TUNE_AUTO in
                              vdwdf_energy_batched                                    */
     int32_t items_per_sm; /* target work items per warp slot for load balance (0 = 256) */
@@ -481,9 +481,9 @@ int vdwdf_energy_noalloc(const vdwdf_grid *grid, const double *n_dev, const doub
  * path, on every k-th work item: about 16 items per warp slot spread over the
  * whole pair triangle) and write the fastest to *best: the one with the most
  * pair evaluations per millisecond of its second timed run.  The shape
- * suits vdwdf_energy and the batched path; vdwdf_potential's default shape
- * (448 threads, 384 on skewed cells) was the fastest for the potential pass
- * on every workload measured. */
+ * is the fastest of those that a tuning can name.  The FP32 default (640
+ * threads) is not one of them and measured faster on every workload, in
+ * vdwdf_energy, vdwdf_potential and the batched path. */
 int vdwdf_autotune(const vdwdf_grid *grid, const double *n_dev, double n_cut, double r_cut,
                    const vdwdf_table *table, int precision, vdwdf_tuning *best,
                    void *cuda_stream);

@@ -30,7 +30,13 @@ struct vdwdf_table {
     std::vector<double> coef64;  // (nD + 2) * (nd + 2), / 36
     std::vector<float> coef32;
     std::mutex mu;
-    std::map<int, std::pair<double *, float *>> dev;  // device id -> copies
+    struct Dev {
+        double *d64 = nullptr;
+        float *d32 = nullptr;
+        cudaArray_t arr = nullptr;      // the bicubic block of coef32 for texture gathers
+        cudaTextureObject_t tex = 0;    // 0: the table exceeds the texture limits
+    };
+    std::map<int, Dev> dev;  // device id -> copies
 };
 
 namespace vdwdf {
@@ -88,27 +94,78 @@ int finish_table(vdwdf_table *t) {
     return VDWDF_OK;
 }
 
-int table_on_device(const vdwdf_table *tc, double **d64, float **d32) {
+// The device copies of a table as the calls use them.
+struct TableDev {
+    double *d64 = nullptr;
+    float *d32 = nullptr;
+    cudaTextureObject_t tex = 0;
+};
+
+// The bicubic block of the FP32 coefficients as a texture (exact fetches of single
+// values); none when an axis exceeds the device's limit for gathers.
+int make_texture(const vdwdf_table *t, int dev, vdwdf_table::Dev &d) {
+    const int S = t->nd + 2, rows = t->nD + 2;
+    int wmax = 0, hmax = 0;
+    VDWDF_CUDA_TRY(cudaDeviceGetAttribute(&wmax, cudaDevAttrMaxTexture2DGatherWidth, dev));
+    VDWDF_CUDA_TRY(cudaDeviceGetAttribute(&hmax, cudaDevAttrMaxTexture2DGatherHeight, dev));
+    if (S > wmax || rows > hmax) return VDWDF_OK;
+    const cudaChannelFormatDesc cd = cudaCreateChannelDesc<float>();
+    if (cudaMallocArray(&d.arr, &cd, S, rows, cudaArrayTextureGather) != cudaSuccess) return VDWDF_EALLOC;
+    VDWDF_CUDA_TRY(cudaMemcpy2DToArray(d.arr, 0, 0, t->coef32.data(), sizeof(float) * S, sizeof(float) * S, rows,
+                                       cudaMemcpyHostToDevice));
+    cudaResourceDesc rd;
+    std::memset(&rd, 0, sizeof(rd));
+    rd.resType = cudaResourceTypeArray;
+    rd.res.array.array = d.arr;
+    cudaTextureDesc td;
+    std::memset(&td, 0, sizeof(td));
+    td.addressMode[0] = td.addressMode[1] = cudaAddressModeClamp;
+    td.filterMode = cudaFilterModePoint;
+    td.readMode = cudaReadModeElementType;
+    VDWDF_CUDA_TRY(cudaCreateTextureObject(&d.tex, &rd, &td, nullptr));
+    return VDWDF_OK;
+}
+
+void free_copies(vdwdf_table::Dev &d) {
+    if (d.tex) cudaDestroyTextureObject(d.tex);
+    if (d.arr) cudaFreeArray(d.arr);
+    if (d.d64) cudaFree(d.d64);
+    if (d.d32) cudaFree(d.d32);
+    d = vdwdf_table::Dev();
+}
+
+TableDev view_of(const vdwdf_table::Dev &d) {
+    TableDev v;
+    v.d64 = d.d64;
+    v.d32 = d.d32;
+    v.tex = d.tex;
+    return v;
+}
+
+int table_on_device(const vdwdf_table *tc, TableDev *out) {
     vdwdf_table *t = const_cast<vdwdf_table *>(tc);
     int dev = 0;
     VDWDF_CUDA_TRY(cudaGetDevice(&dev));
     std::lock_guard<std::mutex> lk(t->mu);
     auto it = t->dev.find(dev);
     if (it == t->dev.end()) {
-        double *a = nullptr;
-        float *b = nullptr;
+        vdwdf_table::Dev d;
         const size_t n = t->coef64.size();
-        if (cudaMalloc(&a, n * sizeof(double)) != cudaSuccess) return VDWDF_EALLOC;
-        if (cudaMalloc(&b, n * sizeof(float)) != cudaSuccess) {
-            cudaFree(a);
-            return VDWDF_EALLOC;
+        auto fill = [&]() -> int {
+            if (cudaMalloc(&d.d64, n * sizeof(double)) != cudaSuccess) return VDWDF_EALLOC;
+            if (cudaMalloc(&d.d32, n * sizeof(float)) != cudaSuccess) return VDWDF_EALLOC;
+            VDWDF_CUDA_TRY(cudaMemcpy(d.d64, t->coef64.data(), n * sizeof(double), cudaMemcpyHostToDevice));
+            VDWDF_CUDA_TRY(cudaMemcpy(d.d32, t->coef32.data(), n * sizeof(float), cudaMemcpyHostToDevice));
+            return make_texture(t, dev, d);
+        };
+        const int rc = fill();
+        if (rc) {
+            free_copies(d);
+            return rc;
         }
-        VDWDF_CUDA_TRY(cudaMemcpy(a, t->coef64.data(), n * sizeof(double), cudaMemcpyHostToDevice));
-        VDWDF_CUDA_TRY(cudaMemcpy(b, t->coef32.data(), n * sizeof(float), cudaMemcpyHostToDevice));
-        it = t->dev.emplace(dev, std::make_pair(a, b)).first;
+        it = t->dev.emplace(dev, d).first;
     }
-    *d64 = it->second.first;
-    *d32 = it->second.second;
+    *out = view_of(it->second);
     return VDWDF_OK;
 }
 
@@ -418,9 +475,16 @@ int prepare(const Geom &G, const double *n_dev, const double *grad_dev, double n
 
 void fill_params(const Geom &G, const Work &w, PairParams &pp) {
     pp.rc2 = G.rc * G.rc * (1.0 + 1e-12);  // inclusive cutoff, rounding ties inside
+    const float rc2f = static_cast<float>(pp.rc2);
+    pp.cut_lo = rc2f * (1.0f - 1e-5f);
+    pp.cut_hi = rc2f * (1.0f + 1e-5f);
+    pp.box_out = rc2f * 1.0002f + 1e-6f;
+    pp.box_in = rc2f * 0.9998f - 1e-6f;
     for (int a = 0; a < 3; ++a) {
         pp.h2[a] = G.met[a];
         pp.g2x[a] = 2.0 * G.met[3 + a];
+        pp.h2f[a] = static_cast<float>(pp.h2[a]);
+        pp.g2f[a] = static_cast<float>(pp.g2x[a]);
         pp.dims[a] = G.dims[a];
         pp.M[a] = G.M[a];
         // culling: exact per-axis metric on orthogonal cells, its smallest eigenvalue
@@ -450,7 +514,7 @@ void fill_params(const Geom &G, const Work &w, PairParams &pp) {
 struct Launch {
     int threads = 512;
     int nctas = 1;
-    int jt = 64;
+    int itile = kTile, jpts = 64 * kTile;  // i and j points per work item
     int ks0 = 0, ksn = 0;
 };
 
@@ -494,10 +558,11 @@ void fill_loop_consts(const PairShared &sh, LoopConsts<R> &k) {
     k.lmax = sh.nd - 2;
 }
 
-void fill_shared(const vdwdf_table *t, const double *d64, const float *d32, const Launch &ln,
+void fill_shared(const vdwdf_table *t, const TableDev &td, const Launch &ln,
                  unsigned int *queue, unsigned int max_iters, PairShared &sh) {
-    sh.tab64 = d64;
-    sh.tab32 = d32;
+    sh.tab64 = td.d64;
+    sh.tab32 = td.d32;
+    sh.tex32 = td.tex;
     sh.S = t->nd + 2;
     sh.nD = t->nD;
     sh.nd = t->nd;
@@ -509,11 +574,13 @@ void fill_shared(const vdwdf_table *t, const double *d64, const float *d32, cons
     const double Dm = t->Dmax, Dm2 = Dm * Dm;
     const double p17 = -sh.C_asym / (2.0 * Dm2 * Dm2 * Dm2);
     sh.om_rho0 = 1.0 - t->nodes[static_cast<size_t>(t->nD - 1) * t->nd] / p17;
+    sh.phi00 = t->nodes[0];
     fill_loop_consts(sh, sh.k32);
     fill_loop_consts(sh, sh.k64);
     sh.ks0 = ln.ks0;
     sh.ksn = ln.ksn;
-    sh.jtiles_per_item = ln.jt;
+    sh.itile = ln.itile;
+    sh.jpts = ln.jpts;
     sh.item_limit = 0xFFFFFFFFu;
     sh.item_stride = 1u;
     sh.max_iters = max_iters_override(max_iters);
@@ -525,7 +592,8 @@ void fill_shared(const vdwdf_table *t, const double *d64, const float *d32, cons
 // A caller's launch shape: VDWDF_EINVAL outside the documented values,
 // VDWDF_EUNSUPPORTED for a thread count the skewed kernel is not built for.
 // The autotuner's candidate launch shapes (threads, items per warp slot, shared
-// band rows, band start); the fourth is the energy-mode default.
+// band rows, band start): shapes that a caller's tuning can name.  The FP32 default
+// (640 threads) is not among them.
 constexpr int kTuneCount = 8;
 constexpr vdwdf_tuning kTuneCandidates[kTuneCount] = {
     {256, 256, 0, -1}, {384, 256, 0, -1}, {448, 256, 0, -1}, {512, 256, 0, -1},
@@ -547,26 +615,31 @@ Launch choose_launch(int precision, bool pot, const vdwdf_tuning *tu, const vdwd
                      long long n_active, bool skew, int ninst = 1) {
     Launch ln;
     const int S = t->nd + 2;
-    // Default shape: 512 threads, and for FP32 E + v 448 (384 on skewed cells).  The
-    // potential pass ran 1-3 % faster with 14 warps (448 threads) than with 16 (512)
-    // or 12 (384); 448 and 512 threads both cap a thread at 128 registers (up to
-    // four warps share one scheduler's 16384), 384 at 168.  The skewed instance,
-    // with its cross terms, was fastest at 384 and 8 % slower at 448.  Energy mode
-    // gains from the extra warps of 512 threads.
-    if (pot && precision == VDWDF_FP32) ln.threads = skew ? 384 : 448;
+    // Default shape: FP64 512 threads, FP32 640: the FP32 kernel is bound by instruction
+    // issue, and 20 warps of 96 registers keep the schedulers 84 % busy (E + v on the
+    // 36 x 63 x 90 monolayer 102.7 ms against 111.9 with 16 warps of 128).
+    if (precision == VDWDF_FP32) ln.threads = 640;
     if (tu && (tu->threads == 384 || tu->threads == 448 || tu->threads == 512 ||
                (!skew && (tu->threads == 256 || tu->threads == 1024))))
         ln.threads = tu->threads;  // skewed cells: the 384-, 448- and 512-thread kernels only
     const int sms = sm_count();
     ln.nctas = sms * ctas_per_sm(precision, pot, ln.threads, 0, S);
-    // work items are (tile of kTile i points) x (jt j tiles); aim at ipsm items per
+    // work items are itile i points (a warp's) x jpts j points; aim at ipsm items per
     // warp slot so that the dynamic queue balances uneven (culled) items
     int ipsm = (tu && tu->items_per_sm > 0) ? tu->items_per_sm : 256;
-    const long long nT = std::max<long long>(1, (n_active + kTile - 1) / kTile);
+    ln.itile = precision == VDWDF_FP32 ? 2 * kTile : kTile;
+    const long long n = std::max<long long>(1, n_active), nI = (n + ln.itile - 1) / ln.itile;
     const long long want = std::max<long long>(1, static_cast<long long>(ipsm) * sms * (ln.threads / 32) / std::max(1, ninst));
-    long long C = std::max<long long>(1, (want + nT - 1) / nT);
-    C = std::min<long long>(C, nT);
-    ln.jt = static_cast<int>(std::max<long long>(1, (nT + C - 1) / C));
+    const long long C = std::max<long long>(1, (want + nI - 1) / nI);
+    const long long jp = (n + C - 1) / C;
+    // FP32: no fewer j points than 64, whose setup would show, unless the items would
+    // then be fewer than four per warp slot (small problems; measured: 64 against 32
+    // points 2-9 % faster from 13,000 active points on, 32 and 16 faster below 5,000)
+    const long long slots = std::max<long long>(1, static_cast<long long>(sms) * (ln.threads / 32) / std::max(1, ninst));
+    const long long four = n * n / (2 * ln.itile * 4 * slots);
+    const long long jmin = precision != VDWDF_FP32 ? 1 : std::min<long long>(64, four);
+    const long long ju = std::max(jp, jmin);
+    ln.jpts = (precision == VDWDF_FP32 && ju <= 16) ? 16 : static_cast<int>((ju + kTile - 1) / kTile) * kTile;
     if (precision == VDWDF_FP32) {
         const int avail = smem_rows_available(ln.threads, S);
         int rows = std::min(avail, t->nD + 2);
@@ -641,9 +714,8 @@ int run_single(const vdwdf_grid *grid, const double *n_dev, const double *grad_d
     if (rc) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const long long launches0 = g_launches.load();
-    double *d64 = nullptr;
-    float *d32 = nullptr;
-    rc = table_on_device(table, &d64, &d32);
+    TableDev td;
+    rc = table_on_device(table, &td);
     if (rc) return rc;
     int *order = nullptr, nb = 0;
     rc = brick_order(G.dims, &order, &nb);
@@ -676,9 +748,9 @@ int run_single(const vdwdf_grid *grid, const double *n_dev, const double *grad_d
             VDWDF_CUDA_TRY(cudaMemsetAsync(w.queue, 0, sizeof(unsigned int), st));
             PairLaunch pl;
             std::memset(&pl, 0, sizeof(pl));
-            const long long items = pair_items(hs.n_active, ln.jt);
+            const long long items = pair_items(hs.n_active, ln.itile, ln.jpts);
             if (items > 0xFFFFFFF0LL) return VDWDF_EINVAL;
-            fill_shared(table, d64, d32, ln, w.queue, static_cast<unsigned int>(items + 2), pl.sh);
+            fill_shared(table, td, ln, w.queue, static_cast<unsigned int>(items + 2), pl.sh);
             if (!pot) {
                 // one energy partial per work item, summed afterwards in a fixed order
                 if (scratch_malloc_async(reinterpret_cast<void **>(&item_buf), sizeof(double) * items, st) != cudaSuccess)
@@ -784,8 +856,8 @@ void destroy_plan(BatchPlan *bp) {
 }
 
 int record_batch(BatchPlan &bp, int ninst, const double *const *n_dev, double n_cut,
-                 const vdwdf_table *table, int precision, const vdwdf_tuning *tu, double *d64,
-                 float *d32, cudaStream_t st) {
+                 const vdwdf_table *table, int precision, const vdwdf_tuning *tu, const TableDev &td,
+                 cudaStream_t st) {
     long long nmax = 0, nsum = 0;
     for (int k = 0; k < ninst; ++k) {
         nmax = std::max(nmax, bp.geo[k].N);
@@ -807,9 +879,9 @@ int record_batch(BatchPlan &bp, int ninst, const double *const *n_dev, double n_
         PairLaunch pl;
         std::memset(&pl, 0, sizeof(pl));
         long long items = 0;
-        for (int k = k0; k < k1; ++k) items += pair_items(bp.geo[k].N, ln.jt);
+        for (int k = k0; k < k1; ++k) items += pair_items(bp.geo[k].N, ln.itile, ln.jpts);
         if (items > 0xFFFFFFF0LL) return VDWDF_EINVAL;
-        fill_shared(table, d64, d32, ln, bp.queues + g, static_cast<unsigned int>(items + 2), pl.sh);
+        fill_shared(table, td, ln, bp.queues + g, static_cast<unsigned int>(items + 2), pl.sh);
         pl.sh.item_E = bp.item_bufs[g];
         pl.sh.item_cap = static_cast<unsigned int>(bp.item_caps[g]);
         pl.ninst = k1 - k0;
@@ -1027,10 +1099,7 @@ void vdwdf_table_free(vdwdf_table *t) {
     int cur = 0;
     const bool have = cudaGetDevice(&cur) == cudaSuccess;
     for (auto &kv : t->dev) {
-        if (cudaSetDevice(kv.first) == cudaSuccess) {
-            cudaFree(kv.second.first);
-            cudaFree(kv.second.second);
-        }
+        if (cudaSetDevice(kv.first) == cudaSuccess) free_copies(kv.second);
     }
     if (have) cudaSetDevice(cur);
     delete t;
@@ -1044,14 +1113,13 @@ int vdwdf_kernel_eval(const vdwdf_table *t, int precision, int64_t npts, const d
         return VDWDF_EINVAL;
     if (precision != VDWDF_FP32 && precision != VDWDF_FP64) return VDWDF_EINVAL;
     if (npts == 0) return VDWDF_OK;
-    double *d64 = nullptr;
-    float *d32 = nullptr;
-    int rc = table_on_device(t, &d64, &d32);
+    TableDev td;
+    int rc = table_on_device(t, &td);
     if (rc) return rc;
     Launch ln;
     PairShared sh;
     std::memset(&sh, 0, sizeof(sh));
-    fill_shared(t, d64, d32, ln, nullptr, 0, sh);
+    fill_shared(t, td, ln, nullptr, 0, sh);
     return launch_kernel_eval(precision, sh, npts, r_dev, qi_dev, qj_dev, phi_dev, rdphi_dev,
                               static_cast<cudaStream_t>(cuda_stream));
 }
@@ -1140,9 +1208,8 @@ int vdwdf_phi0_eval(const vdwdf_table *table, const double *voxel, int64_t nq, c
     if (table->nD < 3) return VDWDF_EINVAL;
     if (nq == 0) return VDWDF_OK;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    double *d64 = nullptr;
-    float *d32 = nullptr;
-    int rc = table_on_device(table, &d64, &d32);
+    TableDev td;
+    int rc = table_on_device(table, &td);
     if (rc) return rc;
     Phi0Rule rule;
     phi0_model(table, voxel, rule);
@@ -1155,7 +1222,7 @@ int vdwdf_phi0_eval(const vdwdf_table *table, const double *voxel, int64_t nq, c
     Launch ln;
     PairShared sh;
     std::memset(&sh, 0, sizeof(sh));
-    fill_shared(table, d64, d32, ln, nullptr, 0, sh);
+    fill_shared(table, td, ln, nullptr, 0, sh);
     if (cudaMemcpyAsync(xw_dev, xw.data(), sizeof(double) * xw.size(), cudaMemcpyHostToDevice, st) != cudaSuccess)
         rc = VDWDF_ECUDA;
     if (rc == VDWDF_OK)
@@ -1185,9 +1252,8 @@ int diag_voxel(const vdwdf_grid *grid, const double *n_dev, const double *grad_d
     if (table->nD < 3) return VDWDF_EINVAL;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     const long long launches0 = g_launches.load();
-    double *d64 = nullptr;
-    float *d32 = nullptr;
-    rc = table_on_device(table, &d64, &d32);
+    TableDev td;
+    rc = table_on_device(table, &td);
     if (rc) return rc;
     Phi0Rule rule;
     double vox[9];
@@ -1258,7 +1324,7 @@ int diag_voxel(const vdwdf_grid *grid, const double *n_dev, const double *grad_d
         Launch ln;
         PairShared sh;
         std::memset(&sh, 0, sizeof(sh));
-        fill_shared(table, d64, d32, ln, nullptr, 0, sh);
+        fill_shared(table, td, ln, nullptr, 0, sh);
         r = launch_phi0(sh, rule, nq, qg, xw_dev, opart, tab, st);
         if (r) return r;
         r = launch_diag_sum(G.N, n_dev, q0, n_cut, tab, nq, lnq0, dlnq, part, sums, st);
@@ -1299,9 +1365,8 @@ int diag_voxel(const vdwdf_grid *grid, const double *n_dev, const double *grad_d
 // evaluations per millisecond wins.
 int autotune_one(const Geom &G, const double *n_dev, double n_cut, const vdwdf_table *table, int precision,
                  vdwdf_tuning *best, cudaStream_t st) {
-    double *d64 = nullptr;
-    float *d32 = nullptr;
-    int rc = table_on_device(table, &d64, &d32);
+    TableDev td;
+    int rc = table_on_device(table, &td);
     if (rc) return rc;
     int *order = nullptr, nb = 0;
     rc = brick_order(G.dims, &order, &nb);
@@ -1326,7 +1391,7 @@ int autotune_one(const Geom &G, const double *n_dev, double n_cut, const vdwdf_t
         if (fp64 && cd.smem_rows != 0) continue;
         if (check_tuning(&cd, G.skew) != VDWDF_OK) continue;  // no such kernel for this cell
         Launch ln = choose_launch(precision, false, &cd, table, hs.n_active, G.skew);
-        const long long total = pair_items(hs.n_active, ln.jt);
+        const long long total = pair_items(hs.n_active, ln.itile, ln.jpts);
         const long long want = 16LL * ln.nctas * (ln.threads / 32);
         const long long stride = std::max<long long>(1, total / std::max<long long>(1, want));
         for (int rep = 0; rep < 2 && rc == VDWDF_OK; ++rep) {
@@ -1339,7 +1404,7 @@ int autotune_one(const Geom &G, const double *n_dev, double n_cut, const vdwdf_t
                 rc = VDWDF_ECUDA;
             PairLaunch pl;
             std::memset(&pl, 0, sizeof(pl));
-            fill_shared(table, d64, d32, ln, w.queue, 0xFFFFFFF0u, pl.sh);
+            fill_shared(table, td, ln, w.queue, 0xFFFFFFF0u, pl.sh);
             pl.sh.item_limit = static_cast<unsigned int>(std::min<long long>(want, 0xFFFFFFF0LL));
             pl.sh.item_stride = static_cast<unsigned int>(std::min<long long>(stride, 0xFFFFFFF0LL));
             pl.ninst = 1;
@@ -1625,9 +1690,8 @@ int vdwdf_energy_batched(int ninst, const vdwdf_grid *grids, const double *const
     }
     const bool tune_auto = tuning && tuning->threads == VDWDF_TUNE_AUTO;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
-    double *d64 = nullptr;
-    float *d32 = nullptr;
-    int rc = table_on_device(table, &d64, &d32);
+    TableDev td;
+    int rc = table_on_device(table, &td);
     if (rc) return rc;
     int dev = 0;
     VDWDF_CUDA_TRY(cudaGetDevice(&dev));
@@ -1638,8 +1702,9 @@ int vdwdf_energy_batched(int ninst, const vdwdf_grid *grids, const double *const
     key.push_back(static_cast<uintptr_t>(dev));
     key.push_back(static_cast<uintptr_t>(ninst));
     key.push_back(static_cast<uintptr_t>(table->gen));
-    key.push_back(reinterpret_cast<uintptr_t>(d64));
-    key.push_back(reinterpret_cast<uintptr_t>(d32));
+    key.push_back(reinterpret_cast<uintptr_t>(td.d64));
+    key.push_back(reinterpret_cast<uintptr_t>(td.d32));
+    key.push_back(static_cast<uintptr_t>(td.tex));
     key.push_back(static_cast<uintptr_t>(precision));
     uint64_t bits;
     std::memcpy(&bits, &n_cut, 8);
@@ -1725,7 +1790,7 @@ int vdwdf_energy_batched(int ninst, const vdwdf_grid *grids, const double *const
                 const Launch ln = choose_launch(precision, false, t, table, std::max<long long>(1, gsum / (k1 - k0)),
                                                 gskew, k1 - k0);
                 long long it = 0;
-                for (int k = k0; k < k1; ++k) it += pair_items(geo[k].N, ln.jt);
+                for (int k = k0; k < k1; ++k) it += pair_items(geo[k].N, ln.itile, ln.jpts);
                 items = std::max(items, it);
             }
             double *b = nullptr;
@@ -1738,8 +1803,7 @@ int vdwdf_energy_batched(int ninst, const vdwdf_grid *grids, const double *const
         }
         // VDWDF_TUNE_AUTO: the autotuner times every candidate shape on this very
         // batch (the whole pass, uncaptured, on the caller's stream, twice; the
-        // second run counts) and the fastest is recorded.  The energy-mode default
-        // is a candidate, so the choice is never slower than it by more than noise.
+        // second run counts) and the fastest is recorded.
         if (tune_auto) {
             Timer tt;
             double best_ms = -1.0;
@@ -1751,7 +1815,7 @@ int vdwdf_energy_batched(int ninst, const vdwdf_grid *grids, const double *const
                 if (!ok) continue;
                 for (int rep = 0; rep < 2 && rc == VDWDF_OK; ++rep) {
                     tt.mark(0, st);
-                    rc = record_batch(*bp, ninst, n_dev, n_cut, table, precision, &cd, d64, d32, st);
+                    rc = record_batch(*bp, ninst, n_dev, n_cut, table, precision, &cd, td, st);
                     tt.mark(1, st);
                     if (rc == VDWDF_OK && cudaStreamSynchronize(st) != cudaSuccess) rc = VDWDF_ECUDA;
                 }
@@ -1778,7 +1842,7 @@ int vdwdf_energy_batched(int ninst, const vdwdf_grid *grids, const double *const
         cudaGraph_t graph = nullptr;
         cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
         if (e == cudaSuccess) {
-            rc = record_batch(*bp, ninst, n_dev, n_cut, table, precision, use, d64, d32, cs);
+            rc = record_batch(*bp, ninst, n_dev, n_cut, table, precision, use, td, cs);
             e = cudaStreamEndCapture(cs, &graph);
         }
         if (e == cudaSuccess && rc == VDWDF_OK) e = cudaGraphInstantiate(&bp->exec, graph, 0);
@@ -1881,15 +1945,14 @@ int noalloc_base(unsigned char **p) {
 }
 
 // The table's device copies if they already exist on the current device.
-int table_resident(const vdwdf_table *tc, double **d64, float **d32) {
+int table_resident(const vdwdf_table *tc, TableDev *out) {
     vdwdf_table *t = const_cast<vdwdf_table *>(tc);
     int dev = 0;
     VDWDF_CUDA_TRY(cudaGetDevice(&dev));
     std::lock_guard<std::mutex> lk(t->mu);
     auto it = t->dev.find(dev);
     if (it == t->dev.end()) return VDWDF_ENOTABLE;
-    *d64 = it->second.first;
-    *d32 = it->second.second;
+    *out = view_of(it->second);
     return VDWDF_OK;
 }
 
@@ -1951,9 +2014,8 @@ int vdwdf_energy_noalloc(const vdwdf_grid *grid, const double *n_dev, const doub
     // synchronisation below, so that nothing of this call is still queued on the
     // shared array when the lock is released
     auto run = [&]() -> int {
-        double *d64 = nullptr;
-        float *d32 = nullptr;
-        rc = table_resident(table, &d64, &d32);
+        TableDev td;
+        rc = table_resident(table, &td);
         if (rc) return rc;
         unsigned char *base = nullptr;
         rc = noalloc_base(&base);
@@ -1993,9 +2055,9 @@ int vdwdf_energy_noalloc(const vdwdf_grid *grid, const double *n_dev, const doub
             VDWDF_CUDA_TRY(cudaMemsetAsync(w.queue, 0, sizeof(unsigned int), st));  // work-queue head
             PairLaunch pl;
             std::memset(&pl, 0, sizeof(pl));
-            const long long items = pair_items(hs.n_active, ln.jt);
+            const long long items = pair_items(hs.n_active, ln.itile, ln.jpts);
             if (items > 0xFFFFFFF0LL) return VDWDF_EINVAL;
-            fill_shared(table, d64, d32, ln, w.queue, static_cast<unsigned int>(items + 2), pl.sh);
+            fill_shared(table, td, ln, w.queue, static_cast<unsigned int>(items + 2), pl.sh);
             // every item below item_cap writes its partial; any beyond it are added atomically
             pl.sh.item_E = item_E;
             pl.sh.item_cap = static_cast<unsigned int>(std::min<long long>(items, item_space));

@@ -62,12 +62,15 @@ struct CellRows {
 // Per-instance inputs of the pair kernel.
 struct PairParams {
     double h2[3];        // metric in index units, diagonal: |M_a|^2 / N_a^2
+    float h2f[3], g2f[3];  // h2 and g2x in FP32
     double g2x[3];       // 2 x off-diagonal metric (01, 02, 12): r^2 = sum h2_a d_a^2
                          //   + g2x[0] d_0 d_1 + g2x[1] d_0 d_2 + g2x[2] d_1 d_2
     float cull_h2[3];    // culling metric: h2 on orthogonal cells, the smallest
                          //   eigenvalue of the metric on skewed ones (a lower bound)
     float rcm[3];        // cutoff extent in index units along each axis (widened)
     double rc2;          // squared cutoff times (1 + 1e-12): inside iff r^2 <= rc2
+    float cut_lo, cut_hi;  // FP32: r^2 up to cut_lo is inside, past cut_hi outside
+    float box_out, box_in; // box tests: a gap past box_out is outside, an extent up to box_in inside
     int dims[3];
     int M[3];            // max |image index| per axis (0: not periodic)
     int use_cut;
@@ -104,11 +107,15 @@ struct PairShared {
     double cD, cd;        // tD = r (q_i + q_j) cD,  td = |q_i - q_j|/(q_i + q_j) cd
     double C_asym;
     double om_rho0;       // 1 - rho(0), rho(0) = phi(Dmax, 0) / phi17(Dmax, 0)
+    double phi00;         // phi(0, 0), the first node
     LoopConsts<float> k32;   // the same constants for the FP32 ...
     LoopConsts<double> k64;  // ... and the FP64 pair loop
     int ks0, ksn;         // FP32: table rows [ks0, ks0 + ksn) resident in shared memory;
                           // ks0 < 0: ks0 is inst[0].stats->band_row0 (set by launch_band_choose)
-    int jtiles_per_item;  // j tiles per work item
+    unsigned long long tex32; // the bicubic coefficients of tab32 as a 2D texture (rows along D) for
+                          // gathers; 0 when the table is too large for one
+    int itile, jpts;      // i points and j points per work item (j: a multiple of 8 in FP32, of
+                          // kTile in FP64)
     unsigned int item_limit;  // process at most item_limit items (autotuning) ...
     unsigned int item_stride; // ... taking every item_stride-th one (1: all in order)
     unsigned int max_iters;   // cap on the work loop of one CTA
@@ -157,10 +164,9 @@ int launch_band_choose(const PairLaunch &pl, unsigned int *hist, cudaStream_t st
 // Sum the energy-mode item partials of every instance in a fixed order into its
 // Stats::E_pair (one block per instance).
 int launch_reduce_items(const PairLaunch &pl, cudaStream_t st);
-// Work items of an instance with n_active points and jt j tiles per item.
-__host__ __device__ inline long long pair_items(long long n_active, int jt) {
-    const long long nT = (n_active + kTile - 1) / kTile;
-    return nT * ((nT + jt - 1) / jt);
+// Work items of an instance with n_active points: itile i points x jpts j points each.
+__host__ __device__ inline long long pair_items(long long n_active, int itile, int jpts) {
+    return ((n_active + itile - 1) / itile) * ((n_active + jpts - 1) / jpts);
 }
 // v = dV (chi (A + U dq0/dn) - div), div the divergence term: div_pre when given
 // (the spectral gradient's, from launch_div_spectral), else the 4th-order stencil's.

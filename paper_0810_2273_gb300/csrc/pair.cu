@@ -22,18 +22,19 @@
 //
 // Work decomposition: persistent CTAs keep a band of B-spline rows resident in
 // shared memory (FP32 path, staged once; which rows is chosen on the device from
-// a sampled histogram of the call's D cells).  Each warp then works on its own:
+// a sampled histogram of the call's D cells); the rest comes from the table's
+// texture copy.  Each warp then works on its own:
 // it pulls work items (instance, tile of kTile i points, range of j tiles) from
 // one queue in global memory, culls every (j tile, image) against its i tile
 // by bounding boxes and then every (j point, image) against the i box, stages
 // surviving j tiles in a private shared-memory buffer (warp-synchronous, no
-// block barrier), and runs the pair loop with each lane owning one i, the j
-// points read as broadcasts and the images of a pair innermost.  In FP32 two j
-// points go through the loop together, one in each half of packed FP32x2
-// arithmetic.  FP32 partial sums over one j tile are folded into FP64
-// accumulators.  The work loop is
-// bounded (max_iters); nothing waits on another warp or CTA.
+// block barrier), and runs the pair loop with each lane owning one i (two in
+// FP32), the j points read as broadcasts and the images of a pair innermost.
+// FP32 partial sums over one j tile are folded into FP64 accumulators.  The work
+// loop is bounded (max_iters); nothing waits on another warp or CTA.
 #include <cuda_runtime.h>
+
+#include <type_traits>
 
 #include "common.cuh"
 
@@ -104,48 +105,68 @@ __device__ __forceinline__ double recip(double x) { return 1.0 / x; }
 __device__ __forceinline__ float rlen(float r2) { return r2 * rsqrtf(fmaxf(r2, 1e-30f)); }
 __device__ __forceinline__ double rlen(double r2) { return sqrt(r2); }
 
+// One-instruction reciprocal and reciprocal root of normal values (the same bits as
+// the functions that also take denormals, without their scaling steps).
+__device__ __forceinline__ float rcp_ftz(float x) {
+    float v;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(v) : "f"(x));
+    return v;
+}
+__device__ __forceinline__ float rsqrt_ftz(float x) {
+    float v;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(v) : "f"(x));
+    return v;
+}
+
 __device__ __forceinline__ float lds32(uint32_t a) {
     float v;
     asm("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"(a));
     return v;
 }
 
-// Two FP32 values per instruction (sm_100-family packed FP32 arithmetic).
+// Two FP32 values side by side, one operation each.  Not the packed FP32x2
+// instructions: a packed multiply-add holds the scheduler's dispatch for 2.3 clocks,
+// two single ones for 2.2 (16 warps on an SM, independent chains; beside an integer
+// operation 3.8 against 3.3), and single ones take immediate operands where packed
+// ones need a register pair filled with each constant.  Both ways E + v of the
+// 36 x 63 x 90 monolayer takes 102.7 ms; single operations are 4 % faster on the open
+// molecule and 3 % on the slab.
 __device__ __forceinline__ float2 f2(float a) { return make_float2(a, a); }
-__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
-__device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
-__device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a, b); }
-__device__ __forceinline__ float2 add2_rm(float2 a, float2 b) {
-    unsigned long long d;
-    asm("add.rm.f32x2 %0, %1, %2;"
-        : "=l"(d)
-        : "l"(*reinterpret_cast<const unsigned long long *>(&a)),
-          "l"(*reinterpret_cast<const unsigned long long *>(&b)));
-    return *reinterpret_cast<const float2 *>(&d);
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {
+    return make_float2(__fmaf_rn(a.x, b.x, c.x), __fmaf_rn(a.y, b.y, c.y));
+}
+__device__ __forceinline__ float2 mul2(float2 a, float2 b) {
+    return make_float2(__fmul_rn(a.x, b.x), __fmul_rn(a.y, b.y));
+}
+__device__ __forceinline__ float2 add2(float2 a, float2 b) {
+    return make_float2(__fadd_rn(a.x, b.x), __fadd_rn(a.y, b.y));
+}
+__device__ __forceinline__ float2 sub2(float2 a, float2 b) {
+    return make_float2(__fsub_rn(a.x, b.x), __fsub_rn(a.y, b.y));
 }
 
-// floor_split of two values at once (both non-negative and below 2^22)
-__device__ __forceinline__ float2 floor_split2(float2 x, int &k0, int &k1) {
-    const float2 b = add2_rm(x, f2(12582912.0f));
-    k0 = __float_as_int(b.x) - 0x4B400000;
-    k1 = __float_as_int(b.y) - 0x4B400000;
-    const float2 f = fma2(f2(-1.0f), f2(12582912.0f), b);  // floor(x), exact
-    return fma2(f, f2(-1.0f), x);                            // x - floor(x), exact
+// floor_split of two values at once (both non-negative and below 2^22): the floors as
+// floats, and as the low mantissa bits of the shifted values.
+__device__ __forceinline__ float2 floor2(float2 x, unsigned &b0, unsigned &b1) {
+    const float s0 = __fadd_rd(x.x, 12582912.0f), s1 = __fadd_rd(x.y, 12582912.0f);
+    b0 = __float_as_uint(s0);
+    b1 = __float_as_uint(s1);
+    return make_float2(s0 - 12582912.0f, s1 - 12582912.0f);
 }
 
+// bw and bdw (without dw[0], which the differences leave out) of two offsets at once.
 __device__ __forceinline__ void bw2(float2 t, float2 w[4]) {
-    const float2 t2 = mul2(t, t), t3 = mul2(t2, t), s = fma2(t, f2(-1.0f), f2(1.0f));
-    w[0] = mul2(mul2(s, s), s);
-    w[1] = fma2(f2(3.0f), t3, fma2(f2(-6.0f), t2, f2(4.0f)));
-    w[2] = fma2(f2(-3.0f), t3, fma2(f2(3.0f), t2, fma2(f2(3.0f), t, f2(1.0f))));
-    w[3] = t3;
+    const float2 s = sub2(f2(1.0f), t), t2 = mul2(t, t), s2 = mul2(s, s);
+    w[0] = mul2(s2, s);
+    w[1] = fma2(t2, fma2(t, f2(3.0f), f2(-6.0f)), f2(4.0f));
+    w[2] = fma2(s2, fma2(s, f2(3.0f), f2(-6.0f)), f2(4.0f));
+    w[3] = mul2(t2, t);
 }
 __device__ __forceinline__ void bdw2(float2 t, float2 d[4]) {
-    const float2 t2 = mul2(t, t), s = fma2(t, f2(-1.0f), f2(1.0f));
-    d[0] = mul2(f2(-3.0f), mul2(s, s));
-    d[1] = fma2(f2(9.0f), t2, mul2(f2(-12.0f), t));
-    d[2] = fma2(f2(-9.0f), t2, fma2(f2(6.0f), t, f2(3.0f)));
-    d[3] = mul2(f2(3.0f), t2);
+    const float2 s = sub2(f2(1.0f), t);
+    d[1] = mul2(t, fma2(t, f2(9.0f), f2(-12.0f)));
+    d[2] = mul2(s, fma2(s, f2(-9.0f), f2(12.0f)));
+    d[3] = mul2(mul2(t, t), f2(3.0f));
 }
 
 // The delta-derivative weights sum to zero, so sum_n dwd[n] c[n] is taken as
@@ -164,7 +185,10 @@ __device__ __forceinline__ void combine(const R c[4][4], const R wD[4], const R 
         if (POT) {
             const R drow = dwd[1] * (c[m][1] - c[m][0]) + dwd[2] * (c[m][2] - c[m][0]) +
                            dwd[3] * (c[m][3] - c[m][0]);
-            a += dwD[m] * row;
+            // along D the same in FP32, from the differences to the first row
+            a += dwD[m] * (sizeof(R) == 8 ? row
+                                          : wd[0] * (c[m][0] - c[0][0]) + wd[1] * (c[m][1] - c[0][1]) +
+                                                wd[2] * (c[m][2] - c[0][2]) + wd[3] * (c[m][3] - c[0][3]));
             b += wD[m] * drow;
         }
     }
@@ -190,20 +214,11 @@ __device__ __forceinline__ void interp(const Table<R> &tb, int k, int l, const R
                                        const R dwD[4], const R wd[4], const R dwd[4], R &p, R &pt,
                                        R &pu) {
     R c[4][4];
-    if (sizeof(R) == 4 && k >= tb.k0 && k + 4 <= tb.k0 + tb.kn) {
-        const uint32_t a0 = tb.s + 4u * static_cast<uint32_t>((k - tb.k0) * tb.SB + l);
-        const uint32_t rs = 4u * static_cast<uint32_t>(tb.SB);
+    const R *g = tb.g + static_cast<size_t>(k) * tb.S + l;
 #pragma unroll
-        for (int m = 0; m < 4; ++m)
+    for (int m = 0; m < 4; ++m)
 #pragma unroll
-            for (int n = 0; n < 4; ++n) c[m][n] = static_cast<R>(lds32(a0 + m * rs + 4u * n));
-    } else {
-        const R *g = tb.g + static_cast<size_t>(k) * tb.S + l;
-#pragma unroll
-        for (int m = 0; m < 4; ++m)
-#pragma unroll
-            for (int n = 0; n < 4; ++n) c[m][n] = __ldg(g + m * tb.S + n);
-    }
+        for (int n = 0; n < 4; ++n) c[m][n] = __ldg(g + m * tb.S + n);
     combine<POT, R>(c, wD, dwD, wd, dwd, p, pt, pu);
 }
 
@@ -252,56 +267,96 @@ __device__ __forceinline__ void delta_part(R qi, R qj, const Consts<R> &K, Delta
     d.b2 = -bq * (dq > R(0) ? (R(1) + dl) : -(R(1) - dl));  // sign(ds) (1 + ds)
 }
 
-// The delta parts of two pairs (i, j0) and (i, j1) in the two halves of packed
-// FP32 values: the arithmetic of delta_part, two lanes per instruction.
+// The delta parts of two pairs (i0, j) and (i1, j) in the two halves of packed
+// FP32 values: the quantities of delta_part, two pairs per instruction.
 struct Delta2 {
-    float2 sqcD, b1, b2;
-    float2 wd[4], dwd[4];
-    int l0, l1;
+    float2 sqcD;          // (q_i + q_j) cD
+    float2 b1, sb;        // r dphi/dd1 = a + b1 pu, r dphi/dd2 = a + (b1 - 2 sb) pu
+    float2 wd[4], dwd[4]; // dwd[0] is not used
+    float2 fl;            // the delta cells' third columns, l + 2, as texture coordinates
+    uint32_t l0, l1;
 };
 
 template <bool POT>
-__device__ __forceinline__ void delta_part2(float qi, float2 qj, const Consts<float> &K, Delta2 &d,
-                                            bool &cl0, bool &cl1) {
-    const float2 sq = add2(f2(qi), qj);
-    const float2 dq = fma2(qj, f2(-1.0f), f2(qi));  // q_i - q_j, one rounding
-    const float2 isq = make_float2(recip(sq.x), recip(sq.y));
-    const float2 dl = mul2(make_float2(fabsf(dq.x), fabsf(dq.y)), isq);
-    const float2 td0 = mul2(dl, f2(K.cd));
-    cl0 = td0.x > K.tdmax;
-    cl1 = td0.y > K.tdmax;
-    const float2 td = make_float2(fminf(fmaxf(td0.x, 0.0f), K.tdclamp), fminf(fmaxf(td0.y, 0.0f), K.tdclamp));
-    const float2 u = floor_split2(td, d.l0, d.l1);
+__device__ __forceinline__ void delta_part2(float2 qi, float qj, const Consts<float> &K, Delta2 &d, bool &cl0,
+                                            bool &cl1) {
+    const float2 sq = add2(qi, f2(qj)), ndq = sub2(f2(qj), qi);
+    const float2 isq = make_float2(rcp_ftz(sq.x), rcp_ftz(sq.y));
+    const float2 nds = mul2(ndq, isq);  // -ds = (q_j - q_i)/(q_i + q_j)
+    const float2 td0 = mul2(nds, f2(K.cd));
+    cl0 = fabsf(td0.x) > K.tdmax;
+    cl1 = fabsf(td0.y) > K.tdmax;
+    const float2 td = make_float2(fminf(fabsf(td0.x), K.tdclamp), fminf(fabsf(td0.y), K.tdclamp));
+    unsigned b0, b1;
+    const float2 f = floor2(td, b0, b1), u = sub2(td, f);
+    d.l0 = b0 - 0x4B400000u;
+    d.l1 = b1 - 0x4B400000u;
+    d.fl = make_float2(f.x + 3.0f, f.y + 3.0f);
     bw2(u, d.wd);
-    if (POT || cl0 || cl1) bdw2(u, d.dwd);
+    if (POT) bdw2(u, d.dwd);
     if (cl0 || cl1) {
-        const float2 e = fma2(td, f2(-1.0f), td0);  // 0 in a half that is not past the node
+        // past the last node the weights continue linearly: + e w'(u), and the derivative
+        // weights sum to zero
+        float2 dw[4];
+        bdw2(u, dw);
+        const float2 e = make_float2(cl0 ? fabsf(td0.x) - td.x : 0.0f, cl1 ? fabsf(td0.y) - td.y : 0.0f);
+        d.wd[0] = sub2(d.wd[0], mul2(e, add2(dw[1], add2(dw[2], dw[3]))));
 #pragma unroll
-        for (int n = 0; n < 4; ++n) d.wd[n] = fma2(e, d.dwd[n], d.wd[n]);
+        for (int n = 1; n < 4; ++n) d.wd[n] = fma2(e, dw[n], d.wd[n]);
     }
-    const float2 bq = mul2(isq, f2(K.cd));
-    const float2 one = f2(1.0f);
-    const float2 om = fma2(dl, f2(-1.0f), one), op = add2(dl, one);  // 1 - |ds|, 1 + |ds|
     d.sqcD = mul2(sq, f2(K.cD));
-    d.b1 = mul2(bq, make_float2(dq.x > 0.0f ? om.x : -op.x, dq.y > 0.0f ? om.y : -op.y));
-    d.b2 = mul2(bq, make_float2(dq.x > 0.0f ? -op.x : om.x, dq.y > 0.0f ? -op.y : om.y));
+    // sign(ds) cd/(q_i + q_j), and times (1 - ds)
+    const float2 bq = mul2(isq, f2(K.cd));
+    d.sb = make_float2(copysignf(bq.x, -ndq.x), copysignf(bq.y, -ndq.y));
+    d.b1 = fma2(d.sb, nds, d.sb);
 }
 
-// Half s of a packed delta part as a scalar one (register renaming only).
-template <int S>
-__device__ __forceinline__ Delta<float> delta_half(const Delta2 &d) {
-    Delta<float> r;
-    r.sqcD = S ? d.sqcD.y : d.sqcD.x;
-    r.b1 = S ? d.b1.y : d.b1.x;
-    r.b2 = S ? d.b2.y : d.b2.x;
-#pragma unroll
-    for (int n = 0; n < 4; ++n) {
-        r.wd[n] = S ? d.wd[n].y : d.wd[n].x;
-        r.dwd[n] = S ? d.dwd[n].y : d.dwd[n].x;
+// phi and (POT) r dphi/dd1, r dphi/dd2 past the table (D > Dmax, tD = r (q_i + q_j) cD):
+// g(delta*) times eq. (17).
+template <bool POT, typename R>
+__device__ __forceinline__ void past_part(R r, R r2, R tD, R qi, R qj, R inv_qi, R qi2, const Consts<R> &K,
+                                          const R *rho_c, R &phi, R &rd, R &rd2) {
+    const R r4 = r2 * r2;
+    const R qj2 = qj * qj;
+    const R s2 = qi2 + qj2;
+    const R p17 = -K.C * recip(r4 * r2 * qi2 * qj2 * s2);
+    // rho at delta* = 1 - min(d1, d2)/Dmax, in delta cells; at or below 0 the
+    // spline's value at delta = 0 with zero slope (its end condition), past the
+    // last node its linear continuation.  No index leaves the rho block.
+    const bool i_small = qi < qj;
+    const R ts0 = (R(1) - r * fmin(qi, qj) * K.iDmax) * K.cd;
+    const bool up = ts0 > R(0);
+    const bool past = ts0 > K.tdmax;
+    const R ts = fmin(fmax(ts0, R(0)), K.tdclamp);
+    R u;
+    int l = floor_split(ts, u);
+    if (sizeof(R) == 8 && l > K.lmax) {
+        l = K.lmax;
+        u = ts - R(l);
     }
-    r.l = S ? d.l1 : d.l0;
-    r.cl = false;
-    return r;
+    R w[4], dw[4];
+    bw<R>(u, w);
+    const R *rc = rho_c + l;
+    const R c0 = __ldg(rc), c1 = __ldg(rc + 1), c2 = __ldg(rc + 2), c3 = __ldg(rc + 3);
+    R rho = w[0] * c0 + w[1] * c1 + w[2] * c2 + w[3] * c3;
+    R drho = R(0);  // d rho / d delta*, in cells
+    if (POT || past) {
+        bdw<R>(u, dw);
+        drho = up ? dw[1] * (c1 - c0) + dw[2] * (c2 - c0) + dw[3] * (c3 - c0) : R(0);
+        if (past) rho += (ts0 - ts) * drho;
+    }
+    const R Dr = K.tDmax * recip(tD);  // Dmax / D
+    const R Dr2 = Dr * Dr;
+    const R g = rho + K.om_rho0 * (R(1) - Dr2);
+    phi = g * p17;
+    if (POT) {
+        const R is2 = recip(s2);
+        // (1 - rho(0)) (Dmax/D)^2 r/D with r/D = 2 cD r / tD, and rho'(delta*) r/Dmax
+        const R ramp = K.om_rho0 * Dr2 * R(2) * K.cD * r * recip(tD);
+        const R sl = drho * K.cd * r * K.iDmax;
+        rd = g * (R(-2) * p17 * (inv_qi + qi * is2)) + p17 * (i_small ? ramp - sl : ramp);
+        rd2 = g * (R(-2) * p17 * (recip(qj) + qj * is2)) + p17 * (i_small ? ramp : ramp - sl);
+    }
 }
 
 // The distance-dependent part: phi and (POT) r dphi/dd1, r dphi/dd2 at r^2.
@@ -331,47 +386,7 @@ __device__ __forceinline__ void dist_part(R r2, R qi, R qj, R inv_qi, R qi2, con
             rd2 = a + pu * d.b2;
         }
     } else {
-        const R r4 = r2 * r2;
-        const R qj2 = qj * qj;
-        const R s2 = qi2 + qj2;
-        const R p17 = -K.C * recip(r4 * r2 * qi2 * qj2 * s2);
-        // rho at delta* = 1 - min(d1, d2)/Dmax, in delta cells; at or below 0 the
-        // spline's value at delta = 0 with zero slope (its end condition), past the
-        // last node its linear continuation.  No index leaves the rho block.
-        const bool i_small = qi < qj;
-        const R ts0 = (R(1) - r * fmin(qi, qj) * K.iDmax) * K.cd;
-        const bool up = ts0 > R(0);
-        const bool past = ts0 > K.tdmax;
-        const R ts = fmin(fmax(ts0, R(0)), K.tdclamp);
-        R u;
-        int l = floor_split(ts, u);
-        if (sizeof(R) == 8 && l > K.lmax) {
-            l = K.lmax;
-            u = ts - R(l);
-        }
-        R w[4], dw[4];
-        bw<R>(u, w);
-        const R *rc = tb.rho + l;
-        const R c0 = __ldg(rc), c1 = __ldg(rc + 1), c2 = __ldg(rc + 2), c3 = __ldg(rc + 3);
-        R rho = w[0] * c0 + w[1] * c1 + w[2] * c2 + w[3] * c3;
-        R drho = R(0);  // d rho / d delta*, in cells
-        if (POT || past) {
-            bdw<R>(u, dw);
-            drho = up ? dw[1] * (c1 - c0) + dw[2] * (c2 - c0) + dw[3] * (c3 - c0) : R(0);
-            if (past) rho += (ts0 - ts) * drho;
-        }
-        const R Dr = K.tDmax * recip(tD);  // Dmax / D
-        const R Dr2 = Dr * Dr;
-        const R g = rho + K.om_rho0 * (R(1) - Dr2);
-        phi = g * p17;
-        if (POT) {
-            const R is2 = recip(s2);
-            // (1 - rho(0)) (Dmax/D)^2 r/D with r/D = 2 cD r / tD, and rho'(delta*) r/Dmax
-            const R ramp = K.om_rho0 * Dr2 * R(2) * K.cD * r * recip(tD);
-            const R sl = drho * K.cd * r * K.iDmax;
-            rd = g * (R(-2) * p17 * (inv_qi + qi * is2)) + p17 * (i_small ? ramp - sl : ramp);
-            rd2 = g * (R(-2) * p17 * (recip(qj) + qj * is2)) + p17 * (i_small ? ramp : ramp - sl);
-        }
+        past_part<POT, R>(r, r2, tD, qi, qj, inv_qi, qi2, K, tb.rho, phi, rd, rd2);
     }
 }
 
@@ -418,13 +433,12 @@ __device__ __forceinline__ T warp_sum(T v) {
 struct Cut {
     const PairParams *pp;  // FP64 metric and cutoff (kernel parameters), read only
                            // by the recheck near the boundary
-    float lo, hi;
 };
 template <bool SKEW>
 __device__ __forceinline__ bool beyond(float r2, float dx, float dy, float dz, const Cut &c) {
-    if (r2 > c.hi) return true;
-    if (r2 <= c.lo) return false;
     const PairParams &p = *c.pp;
+    if (r2 > p.cut_hi) return true;
+    if (r2 <= p.cut_lo) return false;
     const double X = dx, Y = dy, Z = dz;
     double e = p.h2[0] * (X * X) + p.h2[1] * (Y * Y) + p.h2[2] * (Z * Z);
     if (SKEW) e += p.g2x[0] * (X * Y) + p.g2x[1] * (X * Z) + p.g2x[2] * (Y * Z);
@@ -467,204 +481,572 @@ __device__ __forceinline__ float box_gap2_cart(const float4 &il, const float4 &i
 
 // The counters of a finished work item, summed over the warp and added by lane 0
 // to the instance's totals (integer atomics: the totals do not depend on order).
-__device__ __forceinline__ void count_item(Stats *s, unsigned cnt, unsigned nclamp, unsigned evals) {
-    const unsigned pairs = warp_sum(cnt), clamped = warp_sum(nclamp);
+__device__ __forceinline__ void count_item(Stats *s, unsigned long long cnt, unsigned nclamp,
+                                           unsigned long long evals, unsigned long long cnt_warp = 0ull) {
+    const unsigned long long pairs = warp_sum(cnt) + cnt_warp;
+    const unsigned clamped = warp_sum(nclamp);
     if ((threadIdx.x & 31) == 0) {
-        if (pairs) atomicAdd(&s->pairs, static_cast<unsigned long long>(pairs));
-        if (evals) atomicAdd(&s->evals, static_cast<unsigned long long>(evals));
+        if (pairs) atomicAdd(&s->pairs, pairs);
+        if (evals) atomicAdd(&s->evals, evals);
         if (clamped) atomicAdd(&s->clamped, static_cast<unsigned long long>(clamped));
     }
 }
 
-// Two evaluations in the resident band at once: half s at cell coordinate tD.s and
-// delta row l_s (a half that is not wanted reads no coefficient and returns 0).
-// wd, dwd: the delta weights of the two halves.  Returns phi and, with POT, the
-// cell-coordinate derivatives pt (along D) and pu (along delta).
+// One FP32 evaluation: the two i points of a lane (halves) against one image of a
+// j point.  Table cells come from two memories at once: twelve of the sixteen
+// coefficients from the resident band by shared loads, the 2 x 2 block of the
+// third and fourth rows' third and fourth columns by a texture gather, whose
+// pipe otherwise idles.  Random stencils cost 3.1 SM clocks per shared load (bank
+// conflicts) and 22 per gather, side by side: 49.7 clocks for sixteen loads, 42.0
+// for twelve and one gather (448 threads on an SM, measured on random cells).
+__device__ __forceinline__ float4 tex_block(unsigned long long tex, float x, float y) {
+    return tex2Dgather<float4>(static_cast<cudaTextureObject_t>(tex), x, y, 0);
+}
+
+// One row of the stencil: row = sum_n wd[n] c[n], and with POT the delta derivative
+// from exact coefficient differences (see combine): fma(c0, -1, c_n) is c_n - c0 with
+// one rounding.
 template <bool POT>
-__device__ __forceinline__ void band_pair2(const Table<float> &tb, float2 tD, int l0, int l1, bool use0,
-                                           bool use1, const float2 wdb[4], const float2 dwdb[4],
+__device__ __forceinline__ void row2(const float2 c[4], const float2 wd[4], const float2 dwd[4], float2 &row,
+                                     float2 &drow) {
+    row = fma2(wd[3], c[3], fma2(wd[2], c[2], fma2(wd[1], c[1], mul2(wd[0], c[0]))));
+    if (POT)
+        drow = fma2(dwd[3], sub2(c[3], c[0]), fma2(dwd[2], sub2(c[2], c[0]), mul2(dwd[1], sub2(c[1], c[0]))));
+}
+
+// Six times the cubic B-spline through four neighbours r at offset t of their middle
+// cell, in powers of t, and (DER) a third of six times its t-derivative.  The
+// differences of neighbours stand in for the eight weight polynomials: as many
+// operations, but one constant instead of nine (each a register pair to fill).
+template <bool DER>
+__device__ __forceinline__ float2 spline2(const float2 r[4], float2 t, float2 t3, float2 &der) {
+    const float2 u0 = sub2(r[1], r[0]), u1 = sub2(r[2], r[1]), u2 = sub2(r[3], r[2]);
+    const float2 v = sub2(u1, u0), x = sub2(sub2(u2, u1), v), y = add2(u0, u1);
+    // 6 r1 + v + 3 t y + 3 t^2 v + t^3 x, and y + 2 t v + t^2 x
+    const float2 z = fma2(t, v, y);
+    if (DER) der = fma2(t, fma2(t, x, v), z);
+    return fma2(f2(3.0f), fma2(t, z, add2(r[1], r[1])), fma2(t3, x, v));
+}
+
+// Both halves in the resident band: t the offsets in their D cells (fk: the cells'
+// first rows), a0 and a1 the shared addresses of their first coefficients.
+template <bool POT>
+__device__ __forceinline__ void band_pair2(unsigned long long tex, uint32_t rs, float2 t, float2 fk, uint32_t a0,
+                                           uint32_t a1, float2 fl, const float2 wd[4], const float2 dwd[4],
                                            float2 &p, float2 &pt, float2 &pu) {
-    int k0, k1;
-    const float2 t = floor_split2(tD, k0, k1);
-    float2 wD[4], dwD[4];
-    bw2(t, wD);
-    if (POT) bdw2(t, dwD);
-    const uint32_t a0 = tb.s + 4u * static_cast<uint32_t>((k0 - tb.k0) * tb.SB + l0);
-    const uint32_t a1 = tb.s + 4u * static_cast<uint32_t>((k1 - tb.k0) * tb.SB + l1);
-    const uint32_t rs = 4u * static_cast<uint32_t>(tb.SB);
-    p = f2(0.0f);
-    pt = f2(0.0f);
-    pu = f2(0.0f);
+    const float4 g0 = tex_block(tex, fl.x, fk.x + 3.0f), g1 = tex_block(tex, fl.y, fk.y + 3.0f);
+    float2 r[4], dr[4];
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
         float2 c[4];
 #pragma unroll
-        for (int n = 0; n < 4; ++n)  // an unused half reads nothing
-            c[n] = make_float2(use0 ? lds32(a0 + m * rs + 4u * n) : 0.0f, use1 ? lds32(a1 + m * rs + 4u * n) : 0.0f);
-        const float2 row = fma2(wdb[3], c[3], fma2(wdb[2], c[2], fma2(wdb[1], c[1], mul2(wdb[0], c[0]))));
-        p = fma2(wD[m], row, p);
-        if (POT) {
-            // delta derivative from exact coefficient differences (see combine);
-            // fma(c0, -1, c_n) is c_n - c0 with one rounding
-            const float2 m1 = f2(-1.0f);
-            const float2 drow = fma2(dwdb[3], fma2(c[0], m1, c[3]),
-                                     fma2(dwdb[2], fma2(c[0], m1, c[2]), mul2(dwdb[1], fma2(c[0], m1, c[1]))));
-            pt = fma2(dwD[m], row, pt);
-            pu = fma2(wD[m], drow, pu);
+        for (int n = 0; n < 4; ++n) {
+            if (m < 2 || n < 2)
+                c[n] = make_float2(lds32(a0 + m * rs + 4u * n), lds32(a1 + m * rs + 4u * n));
+            else if (m == 2)
+                c[n] = n == 2 ? make_float2(g0.w, g1.w) : make_float2(g0.z, g1.z);
+            else
+                c[n] = n == 2 ? make_float2(g0.x, g1.x) : make_float2(g0.y, g1.y);
         }
+        row2<POT>(c, wd, dwd, r[m], dr[m]);
+    }
+    const float2 t3 = mul2(mul2(t, t), t);
+    p = spline2<POT>(r, t, t3, pt);
+    float2 unused;
+    if (POT) pu = spline2<false>(dr, t, t3, unused);
+}
+
+// Rows k, k + 1 (y0 = k + 1) of one half's stencil: from the band where the half is in
+// it (a0 its shared address), else from the texture.
+__device__ __forceinline__ void row_pair(bool inb, uint32_t a0, uint32_t rs, unsigned long long tex, float x, float y,
+                                         float lo[4], float hi[4]) {
+    if (inb) {
+#pragma unroll
+        for (int n = 0; n < 4; ++n) {
+            lo[n] = lds32(a0 + 4u * n);
+            hi[n] = lds32(a0 + rs + 4u * n);
+        }
+    } else {
+        const float4 l = tex_block(tex, x - 2.0f, y), r = tex_block(tex, x, y);
+        lo[0] = l.w, lo[1] = l.z, lo[2] = r.w, lo[3] = r.z;
+        hi[0] = l.x, hi[1] = l.y, hi[2] = r.x, hi[3] = r.y;
     }
 }
 
-// The same two evaluations from the table's copy in global memory (read-only
-// path, rows of stride S), for steps where a half lies off the resident band.
+// The same two evaluations where some lane is off the resident band: each half reads
+// the band or, off it, the texture (four gathers for a whole stencil: 89 SM clocks
+// against 310 for sixteen global loads, measured on random cells).
 template <bool POT>
-__device__ __forceinline__ void table_pair2(const Table<float> &tb, float2 tD, int l0, int l1, bool use0,
-                                           bool use1, const float2 wdb[4], const float2 dwdb[4],
-                                           float2 &p, float2 &pt, float2 &pu) {
-    int k0, k1;
-    const float2 t = floor_split2(tD, k0, k1);
-    float2 wD[4], dwD[4];
-    bw2(t, wD);
-    if (POT) bdw2(t, dwD);
-    const float *g0 = tb.g + static_cast<size_t>(k0) * tb.S + l0;
-    const float *g1 = tb.g + static_cast<size_t>(k1) * tb.S + l1;
-    const int rs = tb.S;
-    p = f2(0.0f);
-    pt = f2(0.0f);
-    pu = f2(0.0f);
+__device__ __forceinline__ void table_pair2(unsigned long long tex, uint32_t rs, bool inb0, bool inb1, uint32_t a0,
+                                            uint32_t a1, float2 tD, float2 fl, const float2 wd[4],
+                                            const float2 dwd[4], float2 &p, float2 &pt, float2 &pu) {
+    unsigned b0, b1;
+    const float2 fk = floor2(tD, b0, b1), t = sub2(tD, fk);
+    float2 r[4], dr[4];
 #pragma unroll
-    for (int m = 0; m < 4; ++m) {
-        float2 c[4];
-#pragma unroll
-        for (int n = 0; n < 4; ++n)  // an unused half reads nothing
-            c[n] = make_float2(use0 ? __ldg(g0 + m * rs + n) : 0.0f, use1 ? __ldg(g1 + m * rs + n) : 0.0f);
-        const float2 row = fma2(wdb[3], c[3], fma2(wdb[2], c[2], fma2(wdb[1], c[1], mul2(wdb[0], c[0]))));
-        p = fma2(wD[m], row, p);
-        if (POT) {
-            // delta derivative from exact coefficient differences (see combine);
-            // fma(c0, -1, c_n) is c_n - c0 with one rounding
-            const float2 m1 = f2(-1.0f);
-            const float2 drow = fma2(dwdb[3], fma2(c[0], m1, c[3]),
-                                     fma2(dwdb[2], fma2(c[0], m1, c[2]), mul2(dwdb[1], fma2(c[0], m1, c[1]))));
-            pt = fma2(dwD[m], row, pt);
-            pu = fma2(wD[m], drow, pu);
-        }
+    for (int h = 0; h < 2; ++h) {
+        float lo0[4], hi0[4], lo1[4], hi1[4];
+        row_pair(inb0, a0 + 2u * h * rs, rs, tex, fl.x, fk.x + (1.0f + 2.0f * h), lo0, hi0);
+        row_pair(inb1, a1 + 2u * h * rs, rs, tex, fl.y, fk.y + (1.0f + 2.0f * h), lo1, hi1);
+        const float2 ca[4] = {make_float2(lo0[0], lo1[0]), make_float2(lo0[1], lo1[1]), make_float2(lo0[2], lo1[2]),
+                              make_float2(lo0[3], lo1[3])};
+        const float2 cb[4] = {make_float2(hi0[0], hi1[0]), make_float2(hi0[1], hi1[1]), make_float2(hi0[2], hi1[2]),
+                              make_float2(hi0[3], hi1[3])};
+        row2<POT>(ca, wd, dwd, r[2 * h], dr[2 * h]);
+        row2<POT>(cb, wd, dwd, r[2 * h + 1], dr[2 * h + 1]);
     }
+    const float2 t3 = mul2(mul2(t, t), t);
+    p = spline2<POT>(r, t, t3, pt);
+    float2 unused;
+    if (POT) pu = spline2<false>(dr, t, t3, unused);
 }
 
-// The images of two j points j0, j1 for one i point (FP32): half 0 runs over the
-// images of mask m0 (those of j0), half 1 over m1 (those of j1), one image of each
-// per step; a half whose mask is spent idles.  ex, ey, ez: x_i - x_j per half in
-// index units (integers, so every shifted difference is exact).  ok0, ok1: the
-// pair counts for this lane.  Adds sum_images phi, r dphi/dd1, r dphi/dd2 per half
-// to A2, U2, V2 and counts per half the inside evaluations (ins; the self term,
-// the one at r = 0, is taken off once per point by the caller).
-template <bool POT, bool SKEW>
-__device__ __forceinline__ void images2_f32(unsigned m0, unsigned m1, const float4 *simg, float2 ex, float2 ey,
-                                            float2 ez, float qi, float inv_qi, float qi2, float2 qj,
-                                            const float h2[3], const float g2x[3], bool ok0, bool ok1,
-                                            bool use_cut, const Cut &cut, const Delta2 &dp,
-                                            const Consts<float> &K, const Table<float> &tb, float band_lo,
-                                            float band_hi, float2 &A2, float2 &U2, float2 &V2,
-                                            unsigned &ins0, unsigned &ins1) {
-    const float2 H0 = f2(h2[0]), H1 = f2(h2[1]), H2 = f2(h2[2]);
-    const float2 cD2 = f2(K.cD);
-    A2 = f2(0.0f);
-    U2 = f2(0.0f);
-    V2 = f2(0.0f);
-    // band evaluations: r dphi/dd1 = cD r pt + b1 pu with b1, b2 fixed for the j point,
-    // so the sums of r pt and of pu over the images are scaled once at the end
-    float2 Srpt = f2(0.0f), Spu = f2(0.0f);
-    do {
-        const bool u0 = m0 != 0u, u1 = m1 != 0u;
-        const int i0 = u0 ? __ffs(m0) - 1 : 0;  // a spent half reads a valid slot
-        const int i1 = u1 ? __ffs(m1) - 1 : 0;
-        m0 &= m0 - 1u;
-        m1 &= m1 - 1u;
-        const float4 s0 = simg[i0], s1 = simg[i1];
-        const float2 dx = add2(ex, make_float2(s0.x, s1.x));
-        const float2 dy = add2(ey, make_float2(s0.y, s1.y));
-        const float2 dz = add2(ez, make_float2(s0.z, s1.z));
-        float2 r2 = mul2(H2, mul2(dz, dz));
-        r2 = fma2(H1, mul2(dy, dy), r2);
-        r2 = fma2(H0, mul2(dx, dx), r2);
-        if (SKEW) {
-            r2 = fma2(f2(g2x[0]), mul2(dx, dy), r2);
-            r2 = fma2(f2(g2x[1]), mul2(dx, dz), r2);
-            r2 = fma2(f2(g2x[2]), mul2(dy, dz), r2);
-        }
-        const bool in0 = u0 && ok0 && !(use_cut && beyond<SKEW>(r2.x, dx.x, dy.x, dz.x, cut));
-        const bool in1 = u1 && ok1 && !(use_cut && beyond<SKEW>(r2.y, dx.y, dy.y, dz.y, cut));
-        if (!(in0 || in1)) continue;
-        ins0 += in0 ? 1u : 0u;
-        ins1 += in1 ? 1u : 0u;
-        const float2 rr = mul2(r2, make_float2(rsqrtf(fmaxf(r2.x, 1e-30f)), rsqrtf(fmaxf(r2.y, 1e-30f))));
-        const float2 tD = mul2(rr, dp.sqcD);
-        const bool f0 = !in0 || (tD.x >= band_lo && tD.x < band_hi);
-        const bool f1 = !in1 || (tD.y >= band_lo && tD.y < band_hi);
-        // nearly every step has both halves in the band: lay that path out as the
-        // fall-through one (measured 7 % faster for E + v than without the hint)
-        if (__builtin_expect(f0 && f1, 1)) {
-            // both halves in the resident band; an idle half reads nothing: p, pt,
-            // pu are 0 there and add nothing
-            const float2 tq = make_float2(in0 ? tD.x : band_lo, in1 ? tD.y : band_lo);
-            float2 p, pt, pu;
-            band_pair2<POT>(tb, tq, dp.l0, dp.l1, in0, in1, dp.wd, dp.dwd, p, pt, pu);
-            A2 = add2(A2, p);
-            if (POT) {
-                Srpt = fma2(rr, pt, Srpt);
-                Spu = add2(Spu, pu);
-            }
-        } else if (POT && (!in0 || tD.x <= K.tDmax) && (!in1 || tD.y <= K.tDmax)) {
-            // E + v: a half off the resident band but both on the table: both halves
-            // from the table's global copy, packed as in the band (measured 1-2 %
-            // faster on the monolayer and the molecule, 1 % slower on the slab;
-            // energy mode keeps the scalar path, where it cost registers)
-            const float2 tq = make_float2(in0 ? fminf(tD.x, K.tDclamp) : 0.0f, in1 ? fminf(tD.y, K.tDclamp) : 0.0f);
-            float2 p, pt, pu;
-            table_pair2<POT>(tb, tq, dp.l0, dp.l1, in0, in1, dp.wd, dp.dwd, p, pt, pu);
-            A2 = add2(A2, p);
-            if (POT) {
-                Srpt = fma2(rr, pt, Srpt);
-                Spu = add2(Spu, pu);
-            }
-        } else {
-            if (in0) {
-                float phi, rd = 0.0f, rd2 = 0.0f;
-                dist_part<POT, float>(r2.x, qi, qj.x, inv_qi, qi2, delta_half<0>(dp), K, tb, phi, rd, rd2);
-                A2.x += phi;
-                U2.x += rd;
-                V2.x += rd2;
-            }
-            if (in1) {
-                float phi, rd = 0.0f, rd2 = 0.0f;
-                dist_part<POT, float>(r2.y, qi, qj.y, inv_qi, qi2, delta_half<1>(dp), K, tb, phi, rd, rd2);
-                A2.y += phi;
-                U2.y += rd;
-                V2.y += rd2;
-            }
-        }
-    } while ((m0 | m1) != 0u);
-    if (POT) {
-        const float2 a = mul2(Srpt, cD2);
-        U2 = add2(U2, fma2(Spu, dp.b1, a));
-        V2 = add2(V2, fma2(Spu, dp.b2, a));
-    }
-}
-
-// Warp sums of four values: the total of v_k ends in lanes 8k .. 8k+7.  Two
-// halving exchanges (each lane keeps half of its values and sends the other
-// half) and three butterflies: 8 shuffles instead of 20 for four plain sums.
-__device__ __forceinline__ float warp_sum4(float v0, float v1, float v2, float v3) {
-    const unsigned lane = threadIdx.x & 31u;
-    const bool h16 = (lane & 16u) != 0u, h8 = (lane & 8u) != 0u;
-    const float w0 = (h16 ? v2 : v0) + __shfl_xor_sync(0xffffffffu, h16 ? v0 : v2, 16);
-    const float w1 = (h16 ? v3 : v1) + __shfl_xor_sync(0xffffffffu, h16 ? v1 : v3, 16);
-    float x = (h8 ? w1 : w0) + __shfl_xor_sync(0xffffffffu, h8 ? w0 : w1, 8);
+// Warp sums of two values: the total of v0 ends in lanes 0-15, that of v1 in lanes
+// 16-31 (hi: the lane is one of these).  One halving exchange and four butterflies.
+__device__ __forceinline__ float warp_sum2(float v0, float v1, bool hi) {
+    float x = (hi ? v1 : v0) + __shfl_xor_sync(0xffffffffu, hi ? v0 : v1, 16);
+    x += __shfl_xor_sync(0xffffffffu, x, 8);
     x += __shfl_xor_sync(0xffffffffu, x, 4);
     x += __shfl_xor_sync(0xffffffffu, x, 2);
     x += __shfl_xor_sync(0xffffffffu, x, 1);
     return x;
+}
+
+// Shared memory of a warp in the FP32 kernel: the staged j tile, the image shifts
+// and the j tile's sums.
+struct Warp32 {
+    float4 p[kTile];
+    float4 img[kTile];
+    float n[kTile];
+    float js[2][kTile];
+};
+
+// A pair on a table that is too large for a texture, scalar, from the band and the
+// global copy (out of line: no ordinary table comes here).
+template <bool POT>
+__device__ __noinline__ float3 table_generic(float r2, float qi, float qj, const PairShared *sh) {
+    Table<float> tb;
+    make_table<float>(*sh, tb);
+    unsigned ncl = 0u;
+    float3 v = make_float3(0.0f, 0.0f, 0.0f);
+    pair_phi<POT, float>(r2, qi, qj, 1.0f / qi, qi * qi, sh->k32, tb, v.x, v.y, v.z, ncl);
+    return v;
+}
+
+// r^2 of an index displacement in FP32: the packed loop's operations, one value.
+template <bool SKEW>
+__device__ __forceinline__ float dist2(float dx, float dy, float dz, const PairParams &pp) {
+    float r2 = pp.h2f[2] * (dz * dz);
+    r2 = fmaf(pp.h2f[1], dy * dy, r2);
+    r2 = fmaf(pp.h2f[0], dx * dx, r2);
+    if (SKEW) {
+        r2 = fmaf(pp.g2f[0], dx * dy, r2);
+        r2 = fmaf(pp.g2f[1], dx * dz, r2);
+        r2 = fmaf(pp.g2f[2], dy * dz, r2);
+    }
+    return r2;
+}
+
+// The FP32 work items of one warp.  An item is 64 i points (two tiles, a lane owns
+// one point of each) against a range of j points from the i points on.  All 64
+// share the image masks of a j point, its loop and its part of the j side; an image
+// that keeps the whole i box inside the cutoff (most of them) needs no test, weight
+// or count per lane.
+//
+// Bound by instruction issue: 350 instructions a step (a j point's image against 64
+// i points), 217 of them FP32 arithmetic, with the schedulers 84 % busy and the
+// shared-memory pipe 68 % (36 x 63 x 90 monolayer, E + v).  The kernel before this
+// one (a lane's halves held two j points, 14 warps of 128 registers, packed
+// arithmetic) against this one, ms per pass, E + v / E:
+//   monolayer 36 x 63 x 90  123.0 / 99.7 -> 102.7 / 78.5   slab 48 x 42 x 75  63.2 / - -> 51.4 / 39.9
+//   hexagonal 36 x 36 x 90   74.4 / 62.6 ->  60.9 / 49.2   molecule 48^3      58.0 / - -> 48.2 / -
+// What lies off the band costs code as well as loads: with one more copy of the step
+// (for tiles whose images all stay inside) the instruction cache no longer held
+// the loop, and the slab took 119 ms.
+template <int MODE, int NT, bool SKEW>
+__device__ __forceinline__ void pair_items_f32(const PairLaunch &pl, unsigned char *smem_raw,
+                                               const unsigned int *s_prefix, const int *s_C,
+                                               unsigned int n_items, unsigned int stride, const Table<float> &tb) {
+    constexpr bool POT = (MODE == 1);
+    const int warp = threadIdx.x >> 5;
+    int lane = threadIdx.x & 31;
+    asm volatile("" : "+r"(lane));  // kept, not read from the special register again
+    const bool hi = (lane & 16) != 0;
+    Warp32 &sw = reinterpret_cast<Warp32 *>(smem_raw)[warp];
+    const PairShared &sh = pl.sh;
+    const Consts<float> &K = sh.k32;
+    const unsigned long long tex = sh.tex32;
+    const uint32_t rs = 4u * static_cast<uint32_t>(tb.SB);
+    // cells [k0, k0 + span) have all four rows in the band (none without a texture)
+    const unsigned span =
+        tex ? static_cast<unsigned>(max(0, min(tb.k0 + tb.kn - 3, sh.nD - 1) - tb.k0)) : 0u;
+    const float band_lo = static_cast<float>(tb.k0);
+    const unsigned kbits = 0x4B400000u + static_cast<unsigned>(tb.k0);
+
+    for (unsigned int iter = 0;; ++iter) {
+        if (iter >= sh.max_iters) {
+            if (lane == 0) atomicAdd(&pl.inst[0].stats->guard_trips, 1u);
+            break;
+        }
+        unsigned int item = 0;
+        if (lane == 0) item = atomicAdd(sh.queue, 1u);
+        item = __shfl_sync(0xffffffffu, item, 0);
+        if (item >= n_items) break;
+        item *= stride;
+        int k = 0;
+        while (k + 1 < pl.ninst && item >= s_prefix[k + 1]) ++k;
+        const PairParams &pp = pl.inst[k];
+        const unsigned int local = item - s_prefix[k];
+        const int C = s_C[k];
+        const int I = static_cast<int>(local / C), c = static_cast<int>(local % C);
+        const int n_act = pp.stats->n_active;
+        const int j_first = I * 64 + c * sh.jpts, j_end = min(n_act, j_first + sh.jpts);
+        if (j_first >= j_end) {
+            if (!POT && lane == 0 && sh.item_E && item < sh.item_cap) sh.item_E[item] = 0.0;
+            continue;
+        }
+        const int i0 = I * 64 + lane, i1 = i0 + 32;
+        const bool act0 = i0 < n_act, act1 = i1 < n_act;
+        const int ni_act = min(64, n_act - I * 64);
+        float2 xi = f2(0.0f), yi = f2(0.0f), zi = f2(0.0f), qi = f2(1.0f), ni = f2(0.0f);
+        if (act0) {
+            const float4 p = __ldg(pp.p32 + i0);
+            xi.x = p.x, yi.x = p.y, zi.x = p.z, qi.x = p.w;
+            ni.x = __ldg(pp.n32 + i0);
+        }
+        if (act1) {
+            const float4 p = __ldg(pp.p32 + i1);
+            xi.y = p.x, yi.y = p.y, zi.y = p.z, qi.y = p.w;
+            ni.y = __ldg(pp.n32 + i1);
+        }
+        const bool use_cut = pp.use_cut != 0;
+        Cut cut;
+        cut.pp = &pp;
+        const float2 H0 = f2(pp.h2f[0]), H1 = f2(pp.h2f[1]), H2 = f2(pp.h2f[2]);
+        double E64 = 0.0;  // energy mode: this lane's part of the item's sum
+        unsigned int cnt = 0, nclamp = 0;  // per lane: images that are only partly inside
+        unsigned int cnt_full = 0;         // (j point, image) steps with all 64 i points inside
+        unsigned int evals = 0;            // (j point, image) steps
+        const int T0 = 2 * I, T1 = min(2 * I + 1, (n_act - 1) / kTile);  // the i tiles
+        for (int J = j_first / kTile; J * kTile < j_end; ++J) {
+            const int jb = J * kTile;
+            const int jl0 = max(0, j_first - jb), jl1 = min(kTile, j_end - jb);
+            const bool mine = lane >= jl0 && lane < jl1;
+            float ilo[3], ihi[3], jl[3], jh[3];
+            {
+                const float4 a0 = __ldg(pp.blo + T0), a1 = __ldg(pp.blo + T1), b0 = __ldg(pp.bhi + T0),
+                             b1 = __ldg(pp.bhi + T1), jlo = __ldg(pp.blo + J), jhi = __ldg(pp.bhi + J);
+                ilo[0] = fminf(a0.x, a1.x), ilo[1] = fminf(a0.y, a1.y), ilo[2] = fminf(a0.z, a1.z);
+                ihi[0] = fmaxf(b0.x, b1.x), ihi[1] = fmaxf(b0.y, b1.y), ihi[2] = fmaxf(b0.z, b1.z);
+                jl[0] = jlo.x, jl[1] = jlo.y, jl[2] = jlo.z;
+                jh[0] = jhi.x, jh[1] = jhi.y, jh[2] = jhi.z;
+            }
+            float4 cil = make_float4(0.f, 0.f, 0.f, 0.f), cih = cil, cjl = cil, cjh = cil;
+            if (SKEW) {  // Cartesian boxes
+                const float4 a0 = __ldg(pp.clo + T0), a1 = __ldg(pp.clo + T1), b0 = __ldg(pp.chi + T0),
+                             b1 = __ldg(pp.chi + T1);
+                cil = make_float4(fminf(a0.x, a1.x), fminf(a0.y, a1.y), fminf(a0.z, a1.z), 0.f);
+                cih = make_float4(fmaxf(b0.x, b1.x), fmaxf(b0.y, b1.y), fmaxf(b0.z, b1.z), 0.f);
+                cjl = __ldg(pp.clo + J);
+                cjh = __ldg(pp.chi + J);
+            }
+            const float rc2_box = pp.box_out, rc2_in = pp.box_in;
+            // culling metric: h2 on orthogonal cells, a lower bound of r^2/|d|^2 on skewed ones
+            const float cull[3] = {pp.cull_h2[0], pp.cull_h2[1], pp.cull_h2[2]};
+            int mlo[3], nm[3];
+#pragma unroll
+            for (int a = 0; a < 3; ++a) {
+                if (pp.M[a] == 0) {
+                    mlo[a] = 0;
+                    nm[a] = 1;
+                } else {
+                    const float N = static_cast<float>(pp.dims[a]), rcm = pp.rcm[a];
+                    mlo[a] = max(-pp.M[a], static_cast<int>(ceilf((-rcm - (ihi[a] - jl[a])) / N)));
+                    const int mhi = min(pp.M[a], static_cast<int>(floorf((rcm - (ilo[a] - jh[a])) / N)));
+                    nm[a] = max(0, mhi - mlo[a] + 1);
+                }
+            }
+            const int n_cand = nm[0] * nm[1] * nm[2];
+            const bool diag = (J >> 1) == I;
+            const bool special = diag || ni_act < 64;
+            bool staged = false;
+            // candidate images in chunks of 32, one per lane
+            for (int c0 = 0; c0 < n_cand; c0 += 32) {
+                const int t = c0 + lane;
+                bool ok = false;
+                int mm[3] = {0, 0, 0};
+                if (t < n_cand) {
+                    mm[2] = mlo[2] + t % nm[2];
+                    const int t1 = t / nm[2];
+                    mm[1] = mlo[1] + t1 % nm[1];
+                    mm[0] = mlo[0] + t1 / nm[1];
+                    if (SKEW)
+                        ok = !use_cut || box_gap2_cart(cil, cih, cjl, cjh, mm, pp.dims, pp.vrow) <= rc2_box;
+                    else
+                        ok = !use_cut || box_gap2(ilo, ihi, jl, jh, mm, pp.dims, cull) <= rc2_box;
+                }
+                const unsigned bal = __ballot_sync(0xffffffffu, ok);
+                if (bal == 0u) continue;
+                __syncwarp();  // earlier reads of img, p, n, js are done
+                if (ok)
+                    sw.img[__popc(bal & ((1u << lane) - 1u))] =
+                        make_float4(static_cast<float>(mm[0] * pp.dims[0]), static_cast<float>(mm[1] * pp.dims[1]),
+                                    static_cast<float>(mm[2] * pp.dims[2]), 0.0f);
+                if (!staged) {
+                    if (mine) {
+                        sw.p[lane] = __ldg(pp.p32 + jb + lane);
+                        sw.n[lane] = __ldg(pp.n32 + jb + lane);
+                    }
+                    staged = true;
+                }
+                __syncwarp();
+                const int nimg = __popc(bal);
+                // this lane's j point: images that bring the i box within the cutoff (jm), and
+                // those that keep all of it inside (jf; none in ragged or diagonal tiles)
+                unsigned jm = 0u, jf = 0u;
+                if (mine) {
+                    const float4 pj = sw.p[lane];
+                    for (int b = 0; b < nimg; ++b) {
+                        const float4 sft = sw.img[b];
+                        float d2, f2max;
+                        if (SKEW) {
+                            // the point less the shift, in Cartesian coordinates, against the i box
+                            const float ux = pj.x - sft.x, uy = pj.y - sft.y, uz = pj.z - sft.z;
+                            const CellRows &vr = pp.vrow;
+                            const float q0c = ux * vr.v[0] + uy * vr.v[3] + uz * vr.v[6];
+                            const float q1c = ux * vr.v[1] + uy * vr.v[4] + uz * vr.v[7];
+                            const float q2c = ux * vr.v[2] + uy * vr.v[5] + uz * vr.v[8];
+                            const float lx = cil.x - q0c, hx = q0c - cih.x, ly = cil.y - q1c, hy = q1c - cih.y,
+                                        lz = cil.z - q2c, hz = q2c - cih.z;
+                            const float gx = fmaxf(0.0f, fmaxf(lx, hx)), gy = fmaxf(0.0f, fmaxf(ly, hy)),
+                                        gz = fmaxf(0.0f, fmaxf(lz, hz));
+                            d2 = gx * gx + gy * gy + gz * gz;
+                            const float ex = fminf(lx, hx), ey = fminf(ly, hy), ez = fminf(lz, hz);
+                            f2max = ex * ex + ey * ey + ez * ez;
+                        } else {
+                            const float lx = ilo[0] + sft.x - pj.x, hx = pj.x - ihi[0] - sft.x,
+                                        ly = ilo[1] + sft.y - pj.y, hy = pj.y - ihi[1] - sft.y,
+                                        lz = ilo[2] + sft.z - pj.z, hz = pj.z - ihi[2] - sft.z;
+                            const float gx = fmaxf(0.0f, fmaxf(lx, hx)), gy = fmaxf(0.0f, fmaxf(ly, hy)),
+                                        gz = fmaxf(0.0f, fmaxf(lz, hz));
+                            d2 = cull[0] * gx * gx + cull[1] * gy * gy + cull[2] * gz * gz;
+                            // the farther face along each axis: the lower of the two (signed) gaps
+                            const float ex = fminf(lx, hx), ey = fminf(ly, hy), ez = fminf(lz, hz);
+                            f2max = cull[0] * ex * ex + cull[1] * ey * ey + cull[2] * ez * ez;
+                        }
+                        if (!use_cut || d2 <= rc2_box) jm |= 1u << b;
+                        if (!use_cut || f2max <= rc2_in) jf |= 1u << b;
+                    }
+                    if (special) jf = 0u;
+                }
+                float2 a_acc = f2(0.0f), u_acc = f2(0.0f);
+                float2 cwt = f2(0.0f);
+                unsigned jset = __ballot_sync(0xffffffffu, jm != 0u);
+                while (jset != 0u) {
+                    const int jj = __ffs(jset) - 1;
+                    jset &= jset - 1u;
+                    const unsigned m = __shfl_sync(0xffffffffu, jm, jj);
+                    const unsigned mf = __shfl_sync(0xffffffffu, jf, jj);
+                    evals += static_cast<unsigned>(__popc(m));
+                    cnt_full += static_cast<unsigned>(__popc(mf));
+                    const float4 pj = sw.p[jj];
+                    const float nj = sw.n[jj];
+                    Delta2 dp;
+                    bool cl0, cl1;
+                    delta_part2<POT>(qi, pj.w, K, dp, cl0, cl1);
+                    const uint32_t c0a = tb.s + 4u * dp.l0, c1a = tb.s + 4u * dp.l1;
+                    float2 A2 = f2(0.0f), V2 = f2(0.0f);
+                    // r dphi/dd1 = cD r pt + b1 pu with b1, b2 fixed for the j point: the
+                    // sums of r pt and of pu over the images are scaled once at the end
+                    float2 Srpt = f2(0.0f), Spu = f2(0.0f);
+                    unsigned mfar = 0u;  // images with some pair past the table
+                    float2 cw = f2(0.0f);  // partly inside images: those that count, per half
+                    for (unsigned mr = m; mr != 0u;) {
+                        const unsigned bit = mr & (0u - mr);
+                        const float4 sft = sw.img[__ffs(mr) - 1];
+                        mr ^= bit;
+                        // integers: every sum is exact
+                        const float2 dx = add2(xi, f2(sft.x - pj.x)), dy = add2(yi, f2(sft.y - pj.y)),
+                                     dz = add2(zi, f2(sft.z - pj.z));
+                        float2 r2 = mul2(H2, mul2(dz, dz));
+                        r2 = fma2(H1, mul2(dy, dy), r2);
+                        r2 = fma2(H0, mul2(dx, dx), r2);
+                        if (SKEW) {
+                            r2 = fma2(f2(pp.g2f[0]), mul2(dx, dy), r2);
+                            r2 = fma2(f2(pp.g2f[1]), mul2(dx, dz), r2);
+                            r2 = fma2(f2(pp.g2f[2]), mul2(dy, dz), r2);
+                        }
+                        float2 rr = mul2(r2, make_float2(rsqrt_ftz(r2.x), rsqrt_ftz(r2.y)));
+                        float2 tD = mul2(rr, dp.sqcD);
+                        float2 w = f2(1.0f);  // 0 in a half that does not count
+                        uint32_t l0a = c0a, l1a = c1a;
+                        if ((mf & bit) == 0u) {
+                            bool in0 = true, in1 = true;
+                            if (use_cut) {
+                                in0 = !beyond<SKEW>(r2.x, dx.x, dy.x, dz.x, cut);
+                                in1 = !beyond<SKEW>(r2.y, dx.y, dy.y, dz.y, cut);
+                            }
+                            if (special) {
+                                // ragged i tile, or a diagonal one, where only j >= i counts, self-images (j =
+                                // i, r > 0) for i only, and the self term is added in FP64 at the end
+                                if (!(r2.x > 0.0f)) in0 = false, rr.x = 0.0f;
+                                if (!(r2.y > 0.0f)) in1 = false, rr.y = 0.0f;
+                                in0 = in0 && act0 && (!diag || jb + jj >= i0);
+                                in1 = in1 && act1 && (!diag || jb + jj >= i1);
+                                cnt -= (in0 && diag && jb + jj == i0 ? 1u : 0u) + (in1 && diag && jb + jj == i1 ? 1u : 0u);
+                            }
+                            w = make_float2(in0 ? 1.0f : 0.0f, in1 ? 1.0f : 0.0f);
+                            cw = add2(cw, w);
+                            // an idle half reads the band's first cell (one address for all)
+                            if (!in0) tD.x = band_lo, l0a = tb.s;
+                            if (!in1) tD.y = band_lo, l1a = tb.s;
+                        }
+                        unsigned kb0, kb1;
+                        const float2 fk = floor2(tD, kb0, kb1);
+                        kb0 -= kbits;
+                        kb1 -= kbits;
+                        if (__all_sync(0xffffffffu, kb0 < span && kb1 < span)) {
+                            float2 p, pt, pu;
+                            band_pair2<POT>(tex, rs, sub2(tD, fk), fk, l0a + kb0 * rs, l1a + kb1 * rs, dp.fl, dp.wd,
+                                            dp.dwd, p, pt, pu);
+                            A2 = fma2(w, p, A2);
+                            if (POT) {
+                                Srpt = fma2(mul2(w, rr), pt, Srpt);
+                                Spu = fma2(w, pu, Spu);
+                            }
+                        } else {
+                            // some lane off the band: what lies on the table from its texture copy, what
+                            // lies past it (false for NaN as well) in the loop below
+                            const bool on0 = tD.x >= 0.0f && tD.x <= K.tDmax, on1 = tD.y >= 0.0f && tD.y <= K.tDmax;
+                            if (tex) {
+                                const float2 tq = make_float2(on0 ? fminf(tD.x, K.tDclamp) : 0.0f,
+                                                              on1 ? fminf(tD.y, K.tDclamp) : 0.0f);
+                                const float2 wt = make_float2(on0 ? w.x : 0.0f, on1 ? w.y : 0.0f);
+                                float2 p, pt, pu;
+                                table_pair2<POT>(tex, rs, kb0 < span, kb1 < span, l0a + kb0 * rs, l1a + kb1 * rs, tq,
+                                                 dp.fl, dp.wd, dp.dwd, p, pt, pu);
+                                A2 = fma2(wt, p, A2);
+                                if (POT) {
+                                    Srpt = fma2(make_float2(wt.x == 0.0f ? 0.0f : rr.x, wt.y == 0.0f ? 0.0f : rr.y), pt,
+                                                Srpt);
+                                    Spu = fma2(wt, pu, Spu);
+                                }
+                            }
+                            if (__any_sync(0xffffffffu, (w.x != 0.0f && !(tex && on0)) || (w.y != 0.0f && !(tex && on1))))
+                                mfar |= bit;
+                        }
+                    }
+                    // ordered pairs: two for every inside evaluation (once for i, once for j), less
+                    // the one of a self-image taken off above
+                    cwt = add2(cwt, cw);
+                    if (cl0 || cl1) {
+                        const float nf = static_cast<float>(__popc(mf));
+                        nclamp += 2u * static_cast<unsigned>((cl0 ? nf + cw.x : 0.0f) + (cl1 ? nf + cw.y : 0.0f));
+                    }
+                    if (POT) {
+                        const float2 a = mul2(Srpt, f2(3.0f * K.cD));  // spline2 gives a third of the derivative
+                        const float2 u = fma2(Spu, dp.b1, a), v = mul2(Spu, dp.sb);
+                        u_acc = fma2(f2(nj), u, u_acc);
+                        V2 = sub2(sub2(u, v), v);
+                    }
+                    // the halves past the table (once more from the geometry, so that the loop above
+                    // keeps nothing for them in registers)
+                    while (mfar != 0u) {
+                        const float4 sft = sw.img[__ffs(mfar) - 1];
+                        const bool part = (mf & mfar & (0u - mfar)) == 0u;
+                        mfar &= mfar - 1u;
+#pragma unroll
+                        for (int h = 0; h < 2; ++h) {
+                            const float q = h ? qi.y : qi.x;
+                            const float dx = (h ? xi.y : xi.x) + (sft.x - pj.x), dy = (h ? yi.y : yi.x) + (sft.y - pj.y),
+                                        dz = (h ? zi.y : zi.x) + (sft.z - pj.z);
+                            const float r2 = dist2<SKEW>(dx, dy, dz, pp);
+                            const float r = r2 * rsqrt_ftz(fmaxf(r2, 1e-30f)), tD = r * ((q + pj.w) * K.cD);
+                            const bool on = tD >= 0.0f && tD <= K.tDmax;
+                            if ((tex && on) || !(r2 > 0.0f)) continue;
+                            if (part && (!(h ? act1 : act0) || (diag && jb + jj < (h ? i1 : i0)) ||
+                                         (use_cut && beyond<SKEW>(r2, dx, dy, dz, cut))))
+                                continue;
+                            float phi, rd = 0.0f, rd2 = 0.0f;
+                            if (on) {  // (only with a table too large for a texture)
+                                const float3 g = table_generic<POT>(r2, q, pj.w, &sh);
+                                phi = g.x, rd = g.y, rd2 = g.z;
+                            } else
+                                past_part<POT, float>(r, r2, tD, q, pj.w, 1.0f / q, q * q, K, tb.rho, phi, rd, rd2);
+                            const float p0 = h ? 0.0f : phi, p1 = h ? phi : 0.0f, u0 = h ? 0.0f : rd, u1 = h ? rd : 0.0f;
+                            A2 = add2(A2, make_float2(p0, p1));
+                            if (POT) {
+                                u_acc = fma2(f2(nj), make_float2(u0, u1), u_acc);
+                                V2 = add2(V2, make_float2(h ? 0.0f : rd2, h ? rd2 : 0.0f));
+                            }
+                        }
+                    }
+                    if (POT) {
+                        a_acc = fma2(f2(nj), A2, a_acc);
+                        // (j = i counts for i only)
+                        const float2 nb = make_float2(diag && jb + jj == i0 ? 0.0f : ni.x,
+                                                      diag && jb + jj == i1 ? 0.0f : ni.y);
+                        const float tot = warp_sum2(nb.x * A2.x + nb.y * A2.y, nb.x * V2.x + nb.y * V2.y, hi);
+                        if ((lane & 15) == 0) sw.js[lane >> 4][jj] = tot;
+                    } else {
+                        // every pair counts for i and for j, j = i for i only
+                        const float n2 = nj + nj;
+                        a_acc = fma2(make_float2(diag && jb + jj == i0 ? nj : n2, diag && jb + jj == i1 ? nj : n2), A2,
+                                     a_acc);
+                    }
+                }
+                cnt += 2u * static_cast<unsigned>(cwt.x + cwt.y);
+                // the j tile's FP32 sums, folded into FP64
+                if (POT) {
+                    if (act0) {
+                        atomicAdd(pp.A + i0, static_cast<double>(a_acc.x));
+                        atomicAdd(pp.U + i0, static_cast<double>(ni.x) * static_cast<double>(u_acc.x));
+                    }
+                    if (act1) {
+                        atomicAdd(pp.A + i1, static_cast<double>(a_acc.y));
+                        atomicAdd(pp.U + i1, static_cast<double>(ni.y) * static_cast<double>(u_acc.y));
+                    }
+                    __syncwarp();
+                    if (jm != 0u) {
+                        const float ja = sw.js[0][lane], ju = sw.js[1][lane];
+                        if (ja != 0.0f) atomicAdd(pp.A + jb + lane, static_cast<double>(ja));
+                        if (ju != 0.0f)
+                            atomicAdd(pp.U + jb + lane, static_cast<double>(sw.n[lane]) * static_cast<double>(ju));
+                    }
+                } else {
+                    E64 += static_cast<double>(ni.x) * static_cast<double>(a_acc.x) +
+                           static_cast<double>(ni.y) * static_cast<double>(a_acc.y);
+                }
+            }
+        }
+        // the self terms n_i phi(0, 0) of the i points whose own j lies in this item, from
+        // the table's node: near a nucleus they outweigh the rest of A_i, and FP32 sums that
+        // hold them round at their size (r dphi/dd1 is 0 there)
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+            const int i = h ? i1 : i0;
+            if (i < n_act && i >= j_first && i < j_end) {
+                const double n = __ldg(pp.n64 + i);
+                if (POT)
+                    atomicAdd(pp.A + i, n * sh.phi00);
+                else
+                    E64 += n * n * sh.phi00;
+            }
+        }
+        count_item(pp.stats, cnt, nclamp, static_cast<unsigned long long>(evals) * static_cast<unsigned long long>(ni_act),
+                   128ull * cnt_full);
+        if (!POT) {
+            // the item's energy partial, summed over lanes in a fixed order (items
+            // beyond the partials' capacity are added atomically)
+            const double e = warp_sum(E64);
+            if (lane == 0) {
+                if (sh.item_E && item < sh.item_cap)
+                    sh.item_E[item] = e;
+                else if (e != 0.0)
+                    atomicAdd(&pp.stats->E_pair, e);
+            }
+        }
+    }
 }
 
 // MODE 0: energy (unordered pairs), MODE 1: potential (A, U per point).
@@ -688,17 +1070,11 @@ __global__ void __launch_bounds__(NT, 1) k_pair(const __grid_constant__ PairLaun
     __shared__ int s_C[kMaxInst];
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    P *sp = reinterpret_cast<P *>(smem_raw) + warp * kTile;             // j tile
-    P *simg = reinterpret_cast<P *>(smem_raw) + (NW + warp) * kTile;    // image shifts
-    R *sn = reinterpret_cast<R *>(smem_raw + 2 * sizeof(P) * kTile * NW) + warp * kTile;
-
     const PairShared &sh = pl.sh;
     Table<R> tb;
     make_table<R>(sh, tb);
-    Consts<R> K;
-    make_consts<R>(sh, K);
     if constexpr (sizeof(R) == 4) {
-        float *band = reinterpret_cast<float *>(smem_raw + (2 * sizeof(P) + sizeof(R)) * kTile * NW);
+        float *band = reinterpret_cast<float *>(smem_raw + sizeof(Warp32) * NW);
         tb.s = static_cast<uint32_t>(__cvta_generic_to_shared(band));
         tb.k0 = sh.ks0 >= 0 ? sh.ks0 : pl.inst[0].stats->band_row0;
         tb.kn = sh.ksn;
@@ -712,22 +1088,25 @@ __global__ void __launch_bounds__(NT, 1) k_pair(const __grid_constant__ PairLaun
         unsigned int acc = 0;
         for (int k = 0; k < pl.ninst; ++k) {
             const int na = pl.inst[k].stats->n_active;
-            const int nT = (na + kTile - 1) / kTile;
-            const int C = max(1, (nT + sh.jtiles_per_item - 1) / sh.jtiles_per_item);
             s_prefix[k] = acc;
-            s_C[k] = C;
-            acc += static_cast<unsigned int>(pair_items(na, sh.jtiles_per_item));
+            s_C[k] = max(1, (na + sh.jpts - 1) / sh.jpts);
+            acc += static_cast<unsigned int>(pair_items(na, sh.itile, sh.jpts));
         }
         s_prefix[pl.ninst] = acc;
     }
-    // cell coordinates tD with all four rows of the cell in the resident band
-    const float band_lo = static_cast<float>(tb.k0);
-    const float band_hi = static_cast<float>(min(tb.k0 + tb.kn - 3, sh.nD - 1));
     __syncthreads();  // the only block barrier: table band and item counts ready
     // autotuning samples every item_stride-th item (item * stride < the total)
     const unsigned int stride = max(1u, sh.item_stride);
     const unsigned int n_items = min((s_prefix[pl.ninst] + stride - 1u) / stride, sh.item_limit);
-
+    if constexpr (sizeof(R) == 4) {
+        pair_items_f32<MODE, NT, SKEW>(pl, smem_raw, s_prefix, s_C, n_items, stride, tb);
+        return;
+    } else {
+    Consts<R> K;
+    make_consts<R>(sh, K);
+    P *sp = reinterpret_cast<P *>(smem_raw) + warp * kTile;             // j tile
+    P *simg = reinterpret_cast<P *>(smem_raw) + (NW + warp) * kTile;    // image shifts
+    R *sn = reinterpret_cast<R *>(smem_raw + 2 * sizeof(P) * kTile * NW) + warp * kTile;
 
     for (unsigned int iter = 0;; ++iter) {
         if (iter >= sh.max_iters) {
@@ -748,8 +1127,8 @@ __global__ void __launch_bounds__(NT, 1) k_pair(const __grid_constant__ PairLaun
         const int n_act = pp.stats->n_active;
         const int nT = (n_act + kTile - 1) / kTile;
         const int Js = I;  // i <-> j folded: j tiles from the i tile on
-        const int J0 = Js + c * sh.jtiles_per_item;
-        const int J1 = min(nT, J0 + sh.jtiles_per_item);
+        const int J0 = Js + c * (sh.jpts / kTile);
+        const int J1 = min(nT, J0 + sh.jpts / kTile);
         if (J0 >= J1) {
             if (!POT && lane == 0 && sh.item_E && item < sh.item_cap) sh.item_E[item] = 0.0;
             continue;
@@ -774,9 +1153,7 @@ __global__ void __launch_bounds__(NT, 1) k_pair(const __grid_constant__ PairLaun
         (void)h2f;
         Cut cut;
         cut.pp = &pp;
-        cut.lo = static_cast<float>(pp.rc2) * (1.0f - 1e-5f);
-        cut.hi = static_cast<float>(pp.rc2) * (1.0f + 1e-5f);
-        const float rc2_box = static_cast<float>(pp.rc2) * 1.0002f + 1e-6f;
+        const float rc2_box = pp.box_out;
         const bool use_cut = pp.use_cut != 0;
         const P *pts = PT<R>::pts(pp);
         const R *nsrc = PT<R>::ns(pp);
@@ -898,60 +1275,6 @@ __global__ void __launch_bounds__(NT, 1) k_pair(const __grid_constant__ PairLaun
                 }
                 R a_acc = 0, u_acc = 0;  // i side (this lane's i)
                 R ja = 0, ju = 0;        // j side: lane L collects j = jb + L
-                if constexpr (sizeof(R) == 4) {
-                    // two j points per pass (packed halves), in order of their lanes
-                    unsigned jset = __ballot_sync(0xffffffffu, jm != 0u);
-                    while (jset != 0u) {
-                        const int j0 = __ffs(jset) - 1;
-                        jset &= jset - 1u;
-                        const bool has1 = jset != 0u;
-                        const int j1 = has1 ? __ffs(jset) - 1 : j0;
-                        jset &= jset - 1u;
-                        const unsigned m0 = __shfl_sync(0xffffffffu, jm, j0);
-                        const unsigned m1s = __shfl_sync(0xffffffffu, jm, j1);
-                        const unsigned m1 = has1 ? m1s : 0u;
-                        item_evals += static_cast<unsigned>(__popc(m0) + __popc(m1));
-                        const float4 p0 = sp[j0], p1 = sp[j1];
-                        // weights: off-diagonal tiles count every pair for i and for j; in
-                        // the diagonal tile j > i counts for both, j == i (self and
-                        // self-images) for i only
-                        const bool both0 = !diag || j0 > lane, both1 = !diag || j1 > lane;
-                        const bool ok0 = act && (both0 || j0 == lane);
-                        const bool ok1 = has1 && act && (both1 || j1 == lane);
-                        Delta2 dp;
-                        bool cl0, cl1;
-                        const float2 qj = make_float2(p0.w, p1.w);
-                        delta_part2<POT>(qi, qj, K, dp, cl0, cl1);
-                        float2 A2, U2, V2;
-                        unsigned ins0 = 0, ins1 = 0;
-                        images2_f32<POT, SKEW>(m0, m1, simg, make_float2(xi - p0.x, xi - p1.x),
-                                               make_float2(yi - p0.y, yi - p1.y), make_float2(zi - p0.z, zi - p1.z),
-                                               qi, inv_qi, qi2, qj, h2, g2f, ok0, ok1, use_cut, cut, dp, K, tb,
-                                               band_lo, band_hi, A2, U2, V2, ins0, ins1);
-                        const unsigned wt0 = both0 ? 2u : 1u, wt1 = both1 ? 2u : 1u;  // ordered pairs
-                        cnt += ins0 * wt0 + ins1 * wt1;
-                        nclamp += (cl0 ? ins0 * wt0 : 0u) + (cl1 ? ins1 * wt1 : 0u);
-                        const float n0 = sn[j0], n1 = sn[j1];
-                        if (POT) {
-                            a_acc += n0 * A2.x + n1 * A2.y;
-                            u_acc += n0 * U2.x + n1 * U2.y;
-                            const float cA0 = both0 ? ni * A2.x : 0.0f, cU0 = both0 ? ni * V2.x : 0.0f;
-                            const float cA1 = both1 ? ni * A2.y : 0.0f, cU1 = both1 ? ni * V2.y : 0.0f;
-                            if (__any_sync(0xffffffffu, cA0 != 0.0f || cU0 != 0.0f || cA1 != 0.0f || cU1 != 0.0f)) {
-                                const float tot = warp_sum4(cA0, cU0, cA1, cU1);
-                                const bool second = has1 && lane == j1;
-                                const float gA = __shfl_sync(0xffffffffu, tot, second ? 16 : 0);
-                                const float gU = __shfl_sync(0xffffffffu, tot, second ? 24 : 8);
-                                if (lane == j0 || second) {
-                                    ja += gA;
-                                    ju += gU;
-                                }
-                            }
-                        } else {
-                            a_acc += static_cast<float>(wt0) * n0 * A2.x + static_cast<float>(wt1) * n1 * A2.y;
-                        }
-                    }
-                } else {
                     for (int jj = 0; jj < jn; ++jj) {
                         unsigned m = __shfl_sync(0xffffffffu, jm, jj);
                         if (m == 0u) continue;
@@ -1006,7 +1329,6 @@ __global__ void __launch_bounds__(NT, 1) k_pair(const __grid_constant__ PairLaun
                             }
                         }
                     }
-                }
                 A64 += static_cast<double>(a_acc);
                 U64 += static_cast<double>(u_acc);
                 if (POT && lane < jn) {
@@ -1015,14 +1337,12 @@ __global__ void __launch_bounds__(NT, 1) k_pair(const __grid_constant__ PairLaun
                 }
             }
         }
-        // FP32 counts every inside evaluation; the self term (j = i, L = 0, the one
-        // evaluation at r = 0) sits in the diagonal tile, which chunk 0 holds
-        if (sizeof(R) == 4 && c == 0 && act) cnt -= 1u;
         if (act && POT) {
             if (A64 != 0.0) atomicAdd(pp.A + ig, A64);
             if (U64 != 0.0) atomicAdd(pp.U + ig, static_cast<double>(ni) * U64);
         }
-        count_item(pp.stats, act ? cnt : 0u, act ? nclamp : 0u, item_evals * static_cast<unsigned>(ni_act));
+        count_item(pp.stats, act ? cnt : 0u, act ? nclamp : 0u,
+                   static_cast<unsigned long long>(item_evals) * static_cast<unsigned long long>(ni_act));
         if (!POT) {
             // the item's energy partial, summed over lanes in a fixed order (items
             // beyond the partials' capacity are added atomically)
@@ -1034,6 +1354,7 @@ __global__ void __launch_bounds__(NT, 1) k_pair(const __grid_constant__ PairLaun
                     atomicAdd(&pp.stats->E_pair, e);
             }
         }
+    }
     }
 }
 
@@ -1137,8 +1458,8 @@ __global__ void k_reduce_items(const __grid_constant__ PairLaunch pl) {
     if (k >= pl.ninst) return;
     unsigned int lo = 0;
     for (int t = 0; t < k; ++t)
-        lo += static_cast<unsigned int>(pair_items(pl.inst[t].stats->n_active, pl.sh.jtiles_per_item));
-    const unsigned int n = static_cast<unsigned int>(pair_items(pl.inst[k].stats->n_active, pl.sh.jtiles_per_item));
+        lo += static_cast<unsigned int>(pair_items(pl.inst[t].stats->n_active, pl.sh.itile, pl.sh.jpts));
+    const unsigned int n = static_cast<unsigned int>(pair_items(pl.inst[k].stats->n_active, pl.sh.itile, pl.sh.jpts));
     const unsigned int hi = min(lo + n, pl.sh.item_cap);
     double s = 0.0;
     for (unsigned int i = lo + threadIdx.x; i < hi; i += blockDim.x) s += pl.sh.item_E[i];
@@ -1245,10 +1566,12 @@ int launch_one(const PairLaunch &pl, int nctas, size_t smem, cudaStream_t st) {
     return VDWDF_OK;
 }
 
-// Skewed cells run the 512-thread kernel only (the launch configuration is
-// chosen for 512 threads when any instance is skewed).
 template <typename R, int MODE>
 int launch_nt(int threads, bool skew, const PairLaunch &pl, int nctas, size_t smem, cudaStream_t st) {
+    if constexpr (sizeof(R) == 4)
+        if (threads == 640)
+            return skew ? launch_one<R, MODE, 640, true>(pl, nctas, smem, st)
+                        : launch_one<R, MODE, 640, false>(pl, nctas, smem, st);
     if (skew) {
         if (threads == 448) return launch_one<R, MODE, 448, true>(pl, nctas, smem, st);
         return threads == 384 ? launch_one<R, MODE, 384, true>(pl, nctas, smem, st)
@@ -1267,16 +1590,15 @@ int launch_nt(int threads, bool skew, const PairLaunch &pl, int nctas, size_t sm
 
 int pair_smem_bytes(int precision, int threads, int ksn, int S) {
     // per warp: j tile (points, densities) and image shifts; FP32: the table band
-    const size_t pt = precision == VDWDF_FP64 ? 2 * sizeof(dvec4) + sizeof(double)
-                                              : 2 * sizeof(float4) + sizeof(float);
-    size_t b = pt * kTile * static_cast<size_t>(threads / 32);
+    const size_t warp = precision == VDWDF_FP64 ? (2 * sizeof(dvec4) + sizeof(double)) * kTile : sizeof(Warp32);
+    size_t b = warp * static_cast<size_t>(threads / 32);
     if (precision != VDWDF_FP64) b += static_cast<size_t>(ksn) * band_stride(S) * sizeof(float);
     return static_cast<int>(b);
 }
 
 int launch_pair(int precision, bool potential, bool skew, int threads, const PairLaunch &pl, int nctas,
                 cudaStream_t st) {
-    if (skew && threads != 512 && threads != 448 && threads != 384) return VDWDF_EINVAL;  // skewed: 384, 448, 512
+    if (skew && threads != 640 && threads != 512 && threads != 448 && threads != 384) return VDWDF_EINVAL;  // skewed: 384, 448, 512
     const size_t smem = static_cast<size_t>(pair_smem_bytes(precision, threads, pl.sh.ksn, pl.sh.S));
     if (precision == VDWDF_FP64)
         return potential ? launch_nt<double, 1>(threads, skew, pl, nctas, smem, st)
