@@ -1688,6 +1688,11 @@ int vdwdf_energy_batched(int ninst, const vdwdf_grid *grids, const double *const
         rc = check_tuning(tuning, geo[k].skew, true);
         if (rc) return rc;
     }
+    // one launch runs its instances with or without the cross terms: beside a skewed
+    // cell the orthogonal ones run as skewed cells too (their cross terms are 0)
+    bool any_skew = false;
+    for (const Geom &g : geo) any_skew = any_skew || g.skew;
+    for (Geom &g : geo) g.skew = any_skew;
     const bool tune_auto = tuning && tuning->threads == VDWDF_TUNE_AUTO;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     TableDev td;

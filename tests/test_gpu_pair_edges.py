@@ -96,3 +96,16 @@ def test_table_shapes(V, oracle_mod, shape):
     cell, periodic, r_cut = CELLS["slab"]
     n = _density((9, 8, 7), cell, 6)
     _check(V, oracle_mod, table, spline, n, cell, periodic, 1e-6, r_cut)
+
+
+@pytest.mark.parametrize("precision,tol", [("fp32", 1e-6), ("fp64", 1e-12)])
+def test_orthogonal_beside_skewed_in_a_batch(V, gtable, precision, tol):
+    """Orthogonal and skewed cells in one batched launch give the single calls' energies."""
+    kinds = ["slab", "skew", "slab"]
+    ns = [_t(_density((9 + k, 8, 7), CELLS[c][0], k)) for k, c in enumerate(kinds)]
+    geo = [CELLS[c][0] if c == "skew" else np.diag(CELLS[c][0]) for c in kinds]
+    per = [CELLS[c][1] for c in kinds]
+    E, _ = V.energy_batched(ns, geo, per, 1e-6, 6.0, gtable, precision)
+    for n, g, p, e in zip(ns, geo, per, E):
+        one, _ = V.energy(n, g, p, 1e-6, 6.0, gtable, precision)
+        assert abs(e - one) <= tol * abs(one)
