@@ -149,7 +149,8 @@ typedef struct {
                                  other fields are ignored) */
 typedef struct {
     int32_t threads;      /* threads per CTA: 256, 384, 448, 512 or 1024 (0 = default:
-                             FP32 640, which only the default takes; FP64 512);
+                             FP32 640, which only the default takes; FP64 512,
+                             for E + v 256, or 384 on skewed cells);
                              skewed cells take 384, 448 or 512; VDWDF_TUNE_AUTO in
                              vdwdf_energy_batched                                    */
     int32_t items_per_sm; /* target work items per warp slot for load balance (0 = 256) */

@@ -33,6 +33,7 @@ struct vdwdf_table {
     struct Dev {
         double *d64 = nullptr;
         float *d32 = nullptr;
+        double *poly = nullptr;         // per cell cubics of d64 (NULL: the table is too large)
         cudaArray_t arr = nullptr;      // the bicubic block of coef32 for texture gathers
         cudaTextureObject_t tex = 0;    // 0: the table exceeds the texture limits
     };
@@ -72,6 +73,8 @@ cudaError_t scratch_malloc(void **p, size_t bytes) {
 }
 constexpr double kPi = 3.14159265358979323846;
 constexpr int kMaxImages = 64;
+constexpr long long kMaxRTable = 1LL << 23;  // entries of the FP64 path's displacement table (64 MB)
+constexpr long long kMaxPoly = 1LL << 22;    // cells of a table kept as polynomials (128 MB)
 
 // Device layout of the coefficients: (nD + 2) x (nd + 2) bicubic coefficients / 36,
 // then nd + 2 coefficients / 6 of the beyond-table normalisation rho(delta).
@@ -98,6 +101,7 @@ int finish_table(vdwdf_table *t) {
 struct TableDev {
     double *d64 = nullptr;
     float *d32 = nullptr;
+    double *poly = nullptr;
     cudaTextureObject_t tex = 0;
 };
 
@@ -129,6 +133,7 @@ int make_texture(const vdwdf_table *t, int dev, vdwdf_table::Dev &d) {
 void free_copies(vdwdf_table::Dev &d) {
     if (d.tex) cudaDestroyTextureObject(d.tex);
     if (d.arr) cudaFreeArray(d.arr);
+    if (d.poly) cudaFree(d.poly);
     if (d.d64) cudaFree(d.d64);
     if (d.d32) cudaFree(d.d32);
     d = vdwdf_table::Dev();
@@ -138,6 +143,7 @@ TableDev view_of(const vdwdf_table::Dev &d) {
     TableDev v;
     v.d64 = d.d64;
     v.d32 = d.d32;
+    v.poly = d.poly;
     v.tex = d.tex;
     return v;
 }
@@ -156,6 +162,14 @@ int table_on_device(const vdwdf_table *tc, TableDev *out) {
             if (cudaMalloc(&d.d32, n * sizeof(float)) != cudaSuccess) return VDWDF_EALLOC;
             VDWDF_CUDA_TRY(cudaMemcpy(d.d64, t->coef64.data(), n * sizeof(double), cudaMemcpyHostToDevice));
             VDWDF_CUDA_TRY(cudaMemcpy(d.d32, t->coef32.data(), n * sizeof(float), cudaMemcpyHostToDevice));
+            const int S = t->nd + 2;
+            if (static_cast<long long>(t->nD - 1) * S <= kMaxPoly) {
+                if (cudaMalloc(&d.poly, static_cast<size_t>(t->nD - 1) * S * 4 * sizeof(double)) != cudaSuccess)
+                    return VDWDF_EALLOC;
+                const int rc = launch_table_poly(d.d64, t->nD, S, d.poly);
+                if (rc) return rc;
+                VDWDF_CUDA_TRY(cudaStreamSynchronize(nullptr));
+            }
             return make_texture(t, dev, d);
         };
         const int rc = fill();
@@ -230,6 +244,7 @@ struct Geom {
     double dV;
     long long N;
     int M[3];
+    int rtm[3];         // FP64: largest |index displacement| that can lie inside the cutoff
     double rc;
     bool use_cut;
     double B[9];        // reciprocal rows: B_a . M_b = delta_ab
@@ -327,6 +342,10 @@ int check_cut(double n_cut, double r_cut, Geom &G) {
         const double ext = G.skew ? r_cut * bl : r_cut / G.L[a];
         G.M[a] = G.per[a] ? static_cast<int>(std::ceil(ext)) + 1 : 0;
         if (G.M[a] > kMaxImages) return VDWDF_EINVAL;
+        // r_cut spans r_cut |B_a| N_a cells along a; without images the grid bounds it too
+        const double cells = std::floor(G.rc * bl * G.dims[a] * (1.0 + 1e-9)) + 1.0;
+        const double most = G.per[a] ? cells : (G.use_cut ? std::min<double>(cells, G.dims[a] - 1) : G.dims[a] - 1);
+        G.rtm[a] = static_cast<int>(std::min(most, 1e6));
     }
     return VDWDF_OK;
 }
@@ -350,7 +369,8 @@ struct Work {
     int *cnt = nullptr, *off = nullptr, *slot = nullptr;
     float4 *p32 = nullptr;
     float *n32 = nullptr;
-    dvec4 *p64 = nullptr;
+    double *q64 = nullptr;
+    double *rt = nullptr;  // FP64: the displacement table (NULL: none)
     double *n64 = nullptr;
     float4 *blo = nullptr, *bhi = nullptr;
     float4 *clo = nullptr, *chi = nullptr;  // skewed cells only
@@ -361,8 +381,11 @@ struct Work {
     double *gsp = nullptr, *coef = nullptr, *div = nullptr;  // spectral gradient only
 };
 
-size_t layout(const Geom &G, int nb, bool pot, bool fp64, Work *w, unsigned char *base) {
+// alloc_free: the layout inside the static array of vdwdf_energy_noalloc (no displacement
+// table, so that the grids it takes do not depend on the cutoff)
+size_t layout(const Geom &G, int nb, bool pot, bool fp64, Work *w, unsigned char *base, bool alloc_free = false) {
     Carve c;
+    const bool rtab = fp64 && !alloc_free && r_table_entries(G.rtm, G.skew) <= kMaxRTable;
     const size_t N = static_cast<size_t>(G.N);
     const size_t tiles = (N + kTile - 1) / kTile;
     const size_t o_q0 = c.take<double>(N);
@@ -373,7 +396,8 @@ size_t layout(const Geom &G, int nb, bool pot, bool fp64, Work *w, unsigned char
     const size_t o_slot = c.take<int>(N);
     const size_t o_p32 = c.take<float4>(N);
     const size_t o_n32 = c.take<float>(N);
-    const size_t o_p64 = fp64 ? c.take<dvec4>(N) : 0;
+    const size_t o_q64 = fp64 ? c.take<double>(N) : 0;
+    const size_t o_rt = rtab ? c.take<double>(static_cast<size_t>(r_table_entries(G.rtm, G.skew))) : 0;
     const size_t o_n64 = c.take<double>(N);
     const size_t o_blo = c.take<float4>(tiles);
     const size_t o_bhi = c.take<float4>(tiles);
@@ -397,7 +421,8 @@ size_t layout(const Geom &G, int nb, bool pot, bool fp64, Work *w, unsigned char
         w->slot = reinterpret_cast<int *>(base + o_slot);
         w->p32 = reinterpret_cast<float4 *>(base + o_p32);
         w->n32 = reinterpret_cast<float *>(base + o_n32);
-        w->p64 = fp64 ? reinterpret_cast<dvec4 *>(base + o_p64) : nullptr;
+        w->q64 = fp64 ? reinterpret_cast<double *>(base + o_q64) : nullptr;
+        w->rt = rtab ? reinterpret_cast<double *>(base + o_rt) : nullptr;
         w->n64 = reinterpret_cast<double *>(base + o_n64);
         w->blo = reinterpret_cast<float4 *>(base + o_blo);
         w->bhi = reinterpret_cast<float4 *>(base + o_bhi);
@@ -468,7 +493,7 @@ int prepare(const Geom &G, const double *n_dev, const double *grad_dev, double n
     rc = launch_grad_q0(G.dims, G.am, n_dev, g_use, w.q0, w.qn, w.qg, st);
     if (rc) return rc;
     rc = launch_compact(G.dims, n_dev, n_cut, w.q0, order, nb, w.cnt, w.off, pot ? w.slot : nullptr,
-                        w.p32, w.n32, w.p64, w.n64, w.blo, w.bhi, w.stats, st);
+                        w.p32, w.n32, w.q64, w.n64, w.blo, w.bhi, w.stats, st);
     if (rc || !G.skew) return rc;
     return launch_tiles_cart(w.p32, w.stats, G.vrow, w.clo, w.chi, G.N, st);
 }
@@ -487,6 +512,7 @@ void fill_params(const Geom &G, const Work &w, PairParams &pp) {
         pp.g2f[a] = static_cast<float>(pp.g2x[a]);
         pp.dims[a] = G.dims[a];
         pp.M[a] = G.M[a];
+        pp.rtm[a] = G.rtm[a];
         // culling: exact per-axis metric on orthogonal cells, its smallest eigenvalue
         // (a lower bound of r^2 / |d|^2) on skewed ones; the cutoff's extent in index
         // units along a is r_cut sqrt(1/h2) or r_cut |B_a| N_a
@@ -499,7 +525,8 @@ void fill_params(const Geom &G, const Work &w, PairParams &pp) {
     pp.use_cut = G.use_cut ? 1 : 0;
     pp.p32 = w.p32;
     pp.n32 = w.n32;
-    pp.p64 = w.p64;
+    pp.q64 = w.q64;
+    pp.rt = w.rt;
     pp.n64 = w.n64;
     pp.blo = w.blo;
     pp.bhi = w.bhi;
@@ -562,6 +589,7 @@ void fill_shared(const vdwdf_table *t, const TableDev &td, const Launch &ln,
                  unsigned int *queue, unsigned int max_iters, PairShared &sh) {
     sh.tab64 = td.d64;
     sh.tab32 = td.d32;
+    sh.poly64 = td.poly;
     sh.tex32 = td.tex;
     sh.S = t->nd + 2;
     sh.nD = t->nD;
@@ -615,10 +643,12 @@ Launch choose_launch(int precision, bool pot, const vdwdf_tuning *tu, const vdwd
                      long long n_active, bool skew, int ninst = 1) {
     Launch ln;
     const int S = t->nd + 2;
-    // Default shape: FP64 512 threads, FP32 640: the FP32 kernel is bound by instruction
-    // issue, and 20 warps of 96 registers keep the schedulers 84 % busy (E + v on the
-    // 36 x 63 x 90 monolayer 102.7 ms against 111.9 with 16 warps of 128).
-    if (precision == VDWDF_FP32) ln.threads = 640;
+    // Default shape.  FP32 640: that kernel is bound by instruction issue, and 20 warps
+    // of 96 registers keep the schedulers 84 % busy (E + v on the 36 x 63 x 90 monolayer
+    // 102.7 ms against 111.9 with 16 warps of 128).  FP64 is bound by the FP64 pipe, and
+    // few warps are enough: E + v with 256 threads (384 on skewed cells) 274.5 ms on the
+    // 24 x 42 x 60 monolayer against 281.7 with 512; energy 143.3 with 512 against 144.7.
+    ln.threads = precision == VDWDF_FP32 ? 640 : (!pot ? 512 : (skew ? 384 : 256));
     if (tu && (tu->threads == 384 || tu->threads == 448 || tu->threads == 512 ||
                (!skew && (tu->threads == 256 || tu->threads == 1024))))
         ln.threads = tu->threads;  // skewed cells: the 384-, 448- and 512-thread kernels only
@@ -2007,7 +2037,7 @@ int vdwdf_energy_noalloc(const vdwdf_grid *grid, const double *n_dev, const doub
     if (nbl > kNoAllocMaxBricks) return VDWDF_EUNSUPPORTED;
     const int nb = static_cast<int>(nbl);
     const bool fp64 = precision == VDWDF_FP64;
-    const size_t o_order = round256(layout(G, nb, false, fp64, nullptr, nullptr));
+    const size_t o_order = round256(layout(G, nb, false, fp64, nullptr, nullptr, true));
     const size_t o_items = o_order + round256(sizeof(int) * nb);
     if (o_items + 256 * sizeof(double) > kNoAllocBytes) return VDWDF_EUNSUPPORTED;
     const unsigned int item_space = static_cast<unsigned int>((kNoAllocBytes - o_items) / sizeof(double));
@@ -2026,7 +2056,7 @@ int vdwdf_energy_noalloc(const vdwdf_grid *grid, const double *n_dev, const doub
         rc = noalloc_base(&base);
         if (rc) return rc;
         Work w;
-        layout(G, nb, false, fp64, &w, base);
+        layout(G, nb, false, fp64, &w, base, true);
         int *order_dev = reinterpret_cast<int *>(base + o_order);
         double *item_E = reinterpret_cast<double *>(base + o_items);
 
@@ -2042,7 +2072,7 @@ int vdwdf_energy_noalloc(const vdwdf_grid *grid, const double *n_dev, const doub
         rc = launch_grad_q0(G.dims, G.am, n_dev, g_use, w.q0, w.qn, w.qg, st);
         if (rc) return rc;
         rc = launch_compact(G.dims, n_dev, n_cut, w.q0, order_dev, nb, w.cnt, w.off, nullptr, w.p32, w.n32,
-                            w.p64, w.n64, w.blo, w.bhi, w.stats, st);
+                            w.q64, w.n64, w.blo, w.bhi, w.stats, st);
         if (rc) return rc;
         if (G.skew) {
             rc = launch_tiles_cart(w.p32, w.stats, G.vrow, w.clo, w.chi, G.N, st);

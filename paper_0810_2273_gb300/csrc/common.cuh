@@ -25,11 +25,6 @@ constexpr int kBrick = 4;               // 4 x 4 x 4 grid bricks order the activ
 constexpr int kMaxSmemBytes = 232448;   // 227 KiB opt-in shared memory per block (cc 10.x)
 constexpr int kMaxInst = 24;            // instances per pair-kernel launch
 
-// FP64 point record (x, y, z in grid index units, q0).
-struct __align__(32) dvec4 {
-    double x, y, z, w;
-};
-
 // Device-side counters of one instance (zeroed before use).
 struct Stats {
     double E_pair;             // sum over ordered pairs of n_i n_j phi (self term included)
@@ -76,8 +71,10 @@ struct PairParams {
     int use_cut;
     const float4 *p32;   // active points: x, y, z (index units), q0
     const float *n32;
-    const dvec4 *p64;
+    const double *q64;   // q0 of the active points (FP64 path only)
     const double *n64;
+    const double *rt;    // FP64 path: r over index displacements up to rtm (NULL: computed)
+    int rtm[3];
     const float4 *blo, *bhi;  // bounding boxes of kTile-point tiles (index units)
     const float4 *clo, *chi;  // skewed cells: Cartesian bounding boxes of the tiles
     CellRows vrow;            // skewed cells: v_a = M_a / N_a
@@ -102,6 +99,7 @@ struct LoopConsts {
 struct PairShared {
     const double *tab64;  // (nD + 2) x (nd + 2) B-spline coefficients / 36, D outer,
     const float *tab32;   // then nd + 2 coefficients / 6 of rho(delta) (beyond-table factor)
+    const double *poly64; // per D cell and delta column of tab64 its cubic in the cell (NULL: none)
     int S;                // row stride (nd + 2)
     int nD, nd;
     double cD, cd;        // tD = r (q_i + q_j) cD,  td = |q_i - q_j|/(q_i + q_j) cd
@@ -145,11 +143,19 @@ int launch_grad_q0(const int dims[3], const AxisMap &am, const double *n, const 
                    double *q0, double *dq0dn, double *dq0dg, cudaStream_t st);
 int launch_compact(const int dims[3], const double *n, double n_cut, const double *q0,
                    const int *brick_order, int nbricks, int *brick_cnt, int *brick_off, int *slot,
-                   float4 *p32, float *n32, dvec4 *p64, double *n64, float4 *blo, float4 *bhi,
+                   float4 *p32, float *n32, double *q64, double *n64, float4 *blo, float4 *bhi,
                    Stats *stats, cudaStream_t st);
 // skew: some instance has a non-diagonal metric (the kernel adds the cross terms)
 int launch_pair(int precision, bool potential, bool skew, int threads, const PairLaunch &pl, int nctas,
                 cudaStream_t st);
+// Size of the FP64 path's displacement table.
+inline long long r_table_entries(const int rtm[3], bool skew) {
+    const long long x = rtm[0], y = rtm[1], z = rtm[2] + 1LL;
+    return skew ? (2 * x + 1) * (2 * y + 1) * z : (x + 1) * (y + 1) * z;
+}
+// The polynomials of a device table (rows nD + 2, stride S) into poly ((nD - 1) S 4
+// doubles), on the default stream.
+int launch_table_poly(const double *coef, int nD, int S, double *poly);
 // Row stride of the shared-memory table band: odd, so that one column of
 // consecutive rows falls in distinct banks.
 __host__ __device__ inline int band_stride(int S) { return S | 1; }

@@ -42,32 +42,6 @@ namespace vdwdf {
 
 namespace {
 
-template <typename R>
-struct PT;
-template <>
-struct PT<float> {
-    using P = float4;
-    static __device__ __forceinline__ const P *pts(const PairParams &pp) { return pp.p32; }
-    static __device__ __forceinline__ const float *ns(const PairParams &pp) { return pp.n32; }
-    static __device__ __forceinline__ P load(const P *p, int i) { return __ldg(p + i); }
-};
-template <>
-struct PT<double> {
-    using P = dvec4;
-    static __device__ __forceinline__ const P *pts(const PairParams &pp) { return pp.p64; }
-    static __device__ __forceinline__ const double *ns(const PairParams &pp) { return pp.n64; }
-    static __device__ __forceinline__ P load(const P *p, int i) {
-        const double2 *q = reinterpret_cast<const double2 *>(p + i);
-        const double2 a = __ldg(q), b = __ldg(q + 1);
-        P r;
-        r.x = a.x;
-        r.y = a.y;
-        r.z = b.x;
-        r.w = b.y;
-        return r;
-    }
-};
-
 // floor of a non-negative float below 2^22 without a conversion instruction:
 // adding 1.5 * 2^23 rounded toward minus infinity leaves floor(x) in the low
 // mantissa bits.
@@ -361,10 +335,9 @@ __device__ __forceinline__ void past_part(R r, R r2, R tD, R qi, R qj, R inv_qi,
 
 // The distance-dependent part: phi and (POT) r dphi/dd1, r dphi/dd2 at r^2.
 template <bool POT, typename R>
-__device__ __forceinline__ void dist_part(R r2, R qi, R qj, R inv_qi, R qi2, const Delta<R> &d,
+__device__ __forceinline__ void dist_part(R r, R r2, R qi, R qj, R inv_qi, R qi2, const Delta<R> &d,
                                           const Consts<R> &K, const Table<R> &tb, R &phi, R &rd,
                                           R &rd2) {
-    const R r = rlen(r2);
     R tD = r * d.sqcD;
     // the table is read only for 0 <= tD <= nD - 1 (false for NaN as well)
     if (tD >= R(0) && tD <= K.tDmax) {
@@ -397,7 +370,7 @@ __device__ __forceinline__ void pair_phi(R r2, R qi, R qj, R inv_qi, R qi2, cons
     Delta<R> d;
     delta_part<POT, R>(qi, qj, K, d);
     ncl += d.cl ? 1u : 0u;
-    dist_part<POT, R>(r2, qi, qj, inv_qi, qi2, d, K, tb, phi, rd, rd2);
+    dist_part<POT, R>(rlen(r2), r2, qi, qj, inv_qi, qi2, d, K, tb, phi, rd, rd2);
 }
 
 template <typename R>
@@ -426,6 +399,15 @@ __device__ __forceinline__ T warp_sum(T v) {
     return v;
 }
 
+// r of an index displacement in FP64, -1 outside the cutoff.
+template <bool SKEW>
+__device__ __forceinline__ double index_r(const PairParams &p, int dx, int dy, int dz) {
+    const double X = dx, Y = dy, Z = dz;
+    double e = p.h2[0] * (X * X) + p.h2[1] * (Y * Y) + p.h2[2] * (Z * Z);
+    if (SKEW) e += p.g2x[0] * (X * Y) + p.g2x[1] * (X * Z) + p.g2x[2] * (Y * Z);
+    return p.use_cut && e > p.rc2 ? -1.0 : sqrt(e);
+}
+
 // Spherical cutoff, inclusive: a pair is inside iff r^2 <= rc2 (the host folds a
 // 1e-12 relative allowance into rc2 so that distances equal to the cutoff up to
 // rounding count as inside in every path).  FP32 decides pairs clearly away from
@@ -444,11 +426,6 @@ __device__ __forceinline__ bool beyond(float r2, float dx, float dy, float dz, c
     if (SKEW) e += p.g2x[0] * (X * Y) + p.g2x[1] * (X * Z) + p.g2x[2] * (Y * Z);
     return e > p.rc2;
 }
-template <bool SKEW>
-__device__ __forceinline__ bool beyond(double r2, double, double, double, const Cut &c) {
-    return r2 > c.pp->rc2;
-}
-
 // Squared distance between the i box shifted by image m and the j box.
 __device__ __forceinline__ float box_gap2(const float ilo[3], const float ihi[3], const float jl[3],
                                           const float jh[3], const int m[3], const int dims[3],
@@ -1049,22 +1026,219 @@ __device__ __forceinline__ void pair_items_f32(const PairLaunch &pl, unsigned ch
     }
 }
 
+// ---------------------------------------------------------------------------
+// FP64
+// ---------------------------------------------------------------------------
+
+// 1/x to the last bit or so (x positive and normal): a 20-bit seed and two Newton
+// steps, four FP64 operations instead of a division's nine and its special cases.
+__device__ __forceinline__ double rcp_newton(double x) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    y = fma(y, fma(-x, y, 1.0), y);
+    return fma(y, fma(-x, y, 1.0), y);
+}
+
+// The cell of a coordinate x in [0, n): floor(x) in k and x - k, from the low word of x
+// shifted by 1.5 2^52 (rounded down).  False for x outside and for NaN.
+__device__ __forceinline__ bool cell_of(double x, int n, int &k, double &t) {
+    const double b = __dadd_rd(x, 6755399441055744.0);
+    k = __double2loint(b);
+    t = x - (b - 6755399441055744.0);
+    return __double2hiint(b) == 0x43380000 && static_cast<unsigned>(k) < static_cast<unsigned>(n);
+}
+
+// The delta part of a pair in FP64, for all lanes of a warp (the quantities of delta_part): (q_i + q_j) cD, the
+// derivative factors b1 and sb (see Delta2), the delta cell and weights.
+struct Delta64 {
+    double sqcD, b1, sb;
+    double wd[4], dwd[4];
+    int l;
+    bool cl;
+};
+template <bool POT>
+__device__ __forceinline__ void delta_part64(double qi, double qj, const Consts<double> &K, Delta64 &d) {
+    const double sq = qi + qj, dq = qi - qj, isq = rcp_newton(sq), ds = dq * isq;
+    const double td0 = fabs(ds) * K.cd;
+    double u;
+    d.cl = false;
+    double e = 0.0;
+    const bool ok = cell_of(td0, K.lmax + 1, d.l, u);
+    // (a vote, so that the operations of the rare case are not run for all)
+    if (__any_sync(0xffffffffu, !ok)) {
+        // the last node itself (its cell at u = 1), or past it: the weights continue
+        // linearly (see delta_part)
+        const double td = fmin(fmax(td0, 0.0), K.tdmax);
+        const int l = min(static_cast<int>(td), K.lmax);
+        d.cl = td0 > K.tdmax;
+        e = td0 - td;
+        u = ok ? u : td - l;
+        d.l = ok ? d.l : l;
+    }
+    const double s = 1.0 - u, u2 = u * u, s2 = s * s;
+    d.wd[0] = s2 * s;
+    d.wd[1] = fma(u2, fma(u, 3.0, -6.0), 4.0);
+    d.wd[2] = fma(s2, fma(s, 3.0, -6.0), 4.0);
+    d.wd[3] = u2 * u;
+    if (POT || __any_sync(0xffffffffu, d.cl)) {
+        d.dwd[0] = -3.0 * s2;
+        d.dwd[1] = u * fma(u, 9.0, -12.0);
+        d.dwd[2] = s * fma(s, -9.0, 12.0);
+        d.dwd[3] = 3.0 * u2;
+    }
+    if (__any_sync(0xffffffffu, d.cl)) {
+#pragma unroll
+        for (int n = 0; n < 4; ++n) d.wd[n] = fma(d.cl ? e : 0.0, d.dwd[n], d.wd[n]);
+    }
+    d.sqcD = sq * K.cD;
+    d.sb = copysign(isq * K.cd, dq);
+    d.b1 = fma(-ds, d.sb, d.sb);
+}
+
+// The spline at cell (k, l), offset t along D: phi and, with POT, the cell-coordinate
+// derivatives.  poly holds, per D cell and delta column, the column's cubic in t.
+template <bool POT>
+__device__ __forceinline__ void spline64(const double *poly, int S, int k, double t, const Delta64 &d, double &p,
+                                         double &pt, double &pu) {
+    const double2 *c = reinterpret_cast<const double2 *>(poly) + 2 * (static_cast<size_t>(k) * S + d.l);
+    double s[4], P1 = 0.0, P2 = 0.0, P3 = 0.0;
+#pragma unroll
+    for (int n = 0; n < 4; ++n) {
+        const double2 a = __ldg(c + 2 * n), b = __ldg(c + 2 * n + 1);
+        s[n] = fma(t, fma(t, fma(t, b.y, b.x), a.y), a.x);
+        if (POT) {
+            P1 = n ? fma(d.wd[n], a.y, P1) : d.wd[0] * a.y;
+            P2 = n ? fma(d.wd[n], b.x, P2) : d.wd[0] * b.x;
+            P3 = n ? fma(d.wd[n], b.y, P3) : d.wd[0] * b.y;
+        }
+    }
+    p = fma(d.wd[3], s[3], fma(d.wd[2], s[2], fma(d.wd[1], s[1], d.wd[0] * s[0])));
+    if (POT) {
+        pt = fma(t, fma(t, 3.0 * P3, P2 + P2), P1);
+        // the derivative weights sum to zero: differences to the first column
+        pu = fma(d.dwd[3], s[3] - s[0], fma(d.dwd[2], s[2] - s[0], d.dwd[1] * (s[1] - s[0])));
+    }
+}
+
+// past_part in FP64 with one reciprocal (of eq. (17)'s denominator times tD) in place
+// of five divisions.  y = q_i q_j and s2 = q_i^2 + q_j^2.
+template <bool POT>
+__device__ __forceinline__ void past_part64(double r, double tD, double qi, double qj, const Consts<double> &K,
+                                            const double *rho_c, double &phi, double &rd, double &rd2) {
+    const double r2 = r * r, r6 = r2 * r2 * r2, y = qi * qj, s2 = fma(qi, qi, qj * qj);
+    const double z = r6 * (y * y), X = z * s2;
+    const double w = rcp_newton(X * tD);
+    const double inv = w * tD, itD = w * X;  // 1/X, 1/tD
+    const double p17 = -K.C * inv;
+    const bool i_small = qi < qj;
+    // rho at delta* (see past_part)
+    const double a = r * K.iDmax * K.cd, ts0 = fma(-(i_small ? qi : qj), a, K.cd);
+    double u, e = 0.0;
+    int l;
+    bool up = true;
+    if (!cell_of(ts0, K.lmax + 1, l, u)) {
+        const double ts = fmin(fmax(ts0, 0.0), K.tdmax);
+        up = ts0 > 0.0;
+        l = min(static_cast<int>(ts), K.lmax);
+        u = ts - l;
+        e = ts0 > K.tdmax ? ts0 - ts : 0.0;
+    }
+    const double s = 1.0 - u, u2 = u * u, s2u = s * s;
+    const double c0 = __ldg(rho_c + l), c1 = __ldg(rho_c + l + 1), c2 = __ldg(rho_c + l + 2), c3 = __ldg(rho_c + l + 3);
+    double rho = fma(u2 * u, c3, fma(fma(s2u, fma(s, 3.0, -6.0), 4.0), c2,
+                                     fma(fma(u2, fma(u, 3.0, -6.0), 4.0), c1, s2u * s * c0)));
+    double drho = 0.0;
+    if (POT || e != 0.0) {
+        drho = up ? fma(3.0 * u2, c3 - c0, fma(s * fma(s, -9.0, 12.0), c2 - c0, u * fma(u, 9.0, -12.0) * (c1 - c0)))
+                  : 0.0;
+        rho = fma(e, drho, rho);
+    }
+    const double Dr = K.tDmax * itD, m = K.om_rho0 * (Dr * Dr);
+    const double g = rho + (K.om_rho0 - m);
+    phi = g * p17;
+    if (POT) {
+        const double is2 = inv * z, iy = inv * (r6 * s2 * y);  // 1/s2, 1/(q_i q_j)
+        const double ramp = m * (2.0 * K.cD) * r * itD, sl = drho * a, t = -2.0 * phi;
+        rd = fma(t, fma(qi, is2, qj * iy), p17 * (i_small ? ramp - sl : ramp));
+        rd2 = fma(t, fma(qj, is2, qi * iy), p17 * (i_small ? ramp : ramp - sl));
+    }
+}
+
+// FP64 warp sums of two values (as warp_sum2).
+__device__ __forceinline__ double warp_sum2(double v0, double v1, bool hi) {
+    double x = (hi ? v1 : v0) + __shfl_xor_sync(0xffffffffu, hi ? v0 : v1, 16);
+    x += __shfl_xor_sync(0xffffffffu, x, 8);
+    x += __shfl_xor_sync(0xffffffffu, x, 4);
+    x += __shfl_xor_sync(0xffffffffu, x, 2);
+    x += __shfl_xor_sync(0xffffffffu, x, 1);
+    return x;
+}
+
+// r of an index displacement, negative outside the cutoff: from the table of
+// k_r_table, or computed where there is none.
+template <bool SKEW>
+__device__ __forceinline__ double pair_r(const PairParams &pp, int dx, int dy, int dz) {
+    if (pp.rt) {
+        if (SKEW) {
+            if (dz < 0) dx = -dx, dy = -dy, dz = -dz;
+            const unsigned ux = static_cast<unsigned>(dx + pp.rtm[0]), uy = static_cast<unsigned>(dy + pp.rtm[1]);
+            const unsigned wx = 2u * pp.rtm[0] + 1u, wy = 2u * pp.rtm[1] + 1u;
+            if (ux >= wx || uy >= wy || dz > pp.rtm[2]) return -1.0;
+            return __ldg(pp.rt + (static_cast<size_t>(ux) * wy + uy) * (pp.rtm[2] + 1) + dz);
+        }
+        dx = abs(dx), dy = abs(dy), dz = abs(dz);
+        if (dx > pp.rtm[0] || dy > pp.rtm[1] || dz > pp.rtm[2]) return -1.0;
+        return __ldg(pp.rt + (static_cast<size_t>(dx) * (pp.rtm[1] + 1) + dy) * (pp.rtm[2] + 1) + dz);
+    }
+    return index_r<SKEW>(pp, dx, dy, dz);
+}
+
+// The table of pair_r: entry (x, y, z) of extents rtm + 1, or 2 rtm + 1 along the
+// first two axes of a skewed cell (signed differences; z >= 0 by inversion).
+template <bool SKEW>
+__global__ void k_r_table(const __grid_constant__ PairParams pp, double *__restrict__ rt) {
+    const int wx = SKEW ? 2 * pp.rtm[0] + 1 : pp.rtm[0] + 1, wy = SKEW ? 2 * pp.rtm[1] + 1 : pp.rtm[1] + 1,
+              wz = pp.rtm[2] + 1;
+    const long long total = static_cast<long long>(wx) * wy * wz;
+    for (long long e = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; e < total;
+         e += static_cast<long long>(gridDim.x) * blockDim.x) {
+        const int z = static_cast<int>(e % wz), y = static_cast<int>(e / wz % wy),
+                  x = static_cast<int>(e / (static_cast<long long>(wz) * wy));
+        rt[e] = index_r<SKEW>(pp, SKEW ? x - pp.rtm[0] : x, SKEW ? y - pp.rtm[1] : y, z);
+    }
+}
+
+// Shared memory of a warp in the FP64 kernel: the j tile, image shifts, j sums.
+struct Warp64 {
+    int4 p[kTile];    // index coordinates
+    int4 img[kTile];
+    double2 qn[kTile];
+    double js[2][kTile];
+};
+
 // MODE 0: energy (unordered pairs), MODE 1: potential (A, U per point).
 //
-// Per work item the warp holds an i tile (lane = i point).  For each j tile it
-// lists the images whose shifted i box comes within the cutoff of the j box, then
-// each lane marks, for its own j point, which of those images bring the i box
-// within the cutoff of that point.  The pair loop runs over j points (broadcast)
-// and, inside, over the marked images: the delta part of a pair is computed once
-// for all its images.  FP32 takes the j points with images two at a time, half x
-// of every packed step on the images of the first and half y on those of the
-// second, and reduces the four j-side sums of the potential over the warp once
-// per such pair (warp_sum4); FP64 takes them one at a time.
+// Per work item the warp holds an i tile (lane = i point; two of them in FP32,
+// pair_items_f32).  For each j tile it lists the images whose shifted i box comes
+// within the cutoff of the j box, then each lane marks, for its own j point, which
+// of those images bring the i box within the cutoff of that point.  The pair loop
+// runs over j points (broadcast) and, inside, over the marked images: the delta part
+// of a pair is computed once for all its images.
+//
+// The FP64 instances are bound by the FP64 pipe (1.7 lanes an SM and clock, 1/73 of
+// FP32), so what need not run on it does not: r comes from a table over index
+// displacements (k_r_table; it also holds the cutoff test), the D cell's cubic from
+// a table of polynomials instead of weights and rows (spline64), cells and signs from
+// integer operations on the bits.  Rare cases (past the table, the last delta node)
+// stand behind votes: behind a lane's branch the compiler ran them for all, predicated.
+// FP64 operations per evaluation 136 -> 89 (16 x 28 x 40 monolayer, E + v, a third of
+// whose warps hold a lane past the table), the pipe 88 % busy as before.  ms per pass,
+// 24 x 42 x 60 monolayer E + v 453 -> 274 and E 242 -> 143, hexagonal 20 x 20 x 50
+// 93 -> 47, slab 32 x 28 x 50 185 -> 138, open dimer 31 x 23 x 19 E 16.7 -> 14.0.
 template <typename R, int MODE, int NT, bool SKEW>
 __global__ void __launch_bounds__(NT, 1) k_pair(const __grid_constant__ PairLaunch pl) {
     constexpr bool POT = (MODE == 1);
     constexpr int NW = NT / 32;
-    using P = typename PT<R>::P;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ unsigned int s_prefix[kMaxInst + 1];
     __shared__ int s_C[kMaxInst];
@@ -1102,11 +1276,10 @@ __global__ void __launch_bounds__(NT, 1) k_pair(const __grid_constant__ PairLaun
         pair_items_f32<MODE, NT, SKEW>(pl, smem_raw, s_prefix, s_C, n_items, stride, tb);
         return;
     } else {
-    Consts<R> K;
-    make_consts<R>(sh, K);
-    P *sp = reinterpret_cast<P *>(smem_raw) + warp * kTile;             // j tile
-    P *simg = reinterpret_cast<P *>(smem_raw) + (NW + warp) * kTile;    // image shifts
-    R *sn = reinterpret_cast<R *>(smem_raw + 2 * sizeof(P) * kTile * NW) + warp * kTile;
+    const Consts<double> &K = sh.k64;
+    const double *poly = sh.poly64;
+    const bool hi = (lane & 16) != 0;
+    Warp64 &sw = reinterpret_cast<Warp64 *>(smem_raw)[warp];
 
     for (unsigned int iter = 0;; ++iter) {
         if (iter >= sh.max_iters) {
@@ -1134,15 +1307,10 @@ __global__ void __launch_bounds__(NT, 1) k_pair(const __grid_constant__ PairLaun
             continue;
         }
 
-        R h2[3], g2x[3];
-        float h2f[3], g2f[3], rcm[3];
+        float rcm[3];
         int dims[3], M[3];
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            h2[a] = static_cast<R>(pp.h2[a]);
-            g2x[a] = static_cast<R>(pp.g2x[a]);
-            h2f[a] = static_cast<float>(pp.h2[a]);
-            g2f[a] = static_cast<float>(pp.g2x[a]);
             dims[a] = pp.dims[a];
             M[a] = pp.M[a];
             // cutoff in index units along a, widened so that rounding never drops an image
@@ -1150,27 +1318,22 @@ __global__ void __launch_bounds__(NT, 1) k_pair(const __grid_constant__ PairLaun
         }
         // culling metric: h2 on orthogonal cells, a lower bound of r^2/|d|^2 on skewed ones
         const float cull[3] = {pp.cull_h2[0], pp.cull_h2[1], pp.cull_h2[2]};
-        (void)h2f;
-        Cut cut;
-        cut.pp = &pp;
         const float rc2_box = pp.box_out;
         const bool use_cut = pp.use_cut != 0;
-        const P *pts = PT<R>::pts(pp);
-        const R *nsrc = PT<R>::ns(pp);
 
         const int ig = I * kTile + lane;
         const bool act = ig < n_act;
         const int ni_act = min(kTile, n_act - I * kTile);
-        R xi = 0, yi = 0, zi = 0, qi = 1, ni = 0;
+        int xi = 0, yi = 0, zi = 0;
+        double qi = 1.0, ni = 0.0;
         if (act) {
-            const P pi = PT<R>::load(pts, ig);
-            xi = pi.x;
-            yi = pi.y;
-            zi = pi.z;
-            qi = pi.w;
-            ni = __ldg(nsrc + ig);
+            const float4 pi = __ldg(pp.p32 + ig);
+            xi = static_cast<int>(pi.x);
+            yi = static_cast<int>(pi.y);
+            zi = static_cast<int>(pi.z);
+            qi = __ldg(pp.q64 + ig);
+            ni = __ldg(pp.n64 + ig);
         }
-        const R inv_qi = R(1) / qi, qi2 = qi * qi;
         const float4 ib0 = __ldg(pp.blo + I), ib1 = __ldg(pp.bhi + I);
         const float ilo[3] = {ib0.x, ib0.y, ib0.z}, ihi[3] = {ib1.x, ib1.y, ib1.z};
         float4 cil = make_float4(0.f, 0.f, 0.f, 0.f), cih = cil;  // skewed: Cartesian i box
@@ -1225,18 +1388,14 @@ __global__ void __launch_bounds__(NT, 1) k_pair(const __grid_constant__ PairLaun
                 const unsigned bal = __ballot_sync(0xffffffffu, ok);
                 if (bal == 0u) continue;
                 __syncwarp();  // earlier reads of simg, sp, sn are done
-                if (ok) {
-                    P sft;
-                    sft.x = static_cast<R>(mm[0] * dims[0]);
-                    sft.y = static_cast<R>(mm[1] * dims[1]);
-                    sft.z = static_cast<R>(mm[2] * dims[2]);
-                    sft.w = R(0);
-                    simg[__popc(bal & ((1u << lane) - 1u))] = sft;
-                }
+                if (ok)
+                    sw.img[__popc(bal & ((1u << lane) - 1u))] =
+                        make_int4(mm[0] * dims[0], mm[1] * dims[1], mm[2] * dims[2], 0);
                 if (!staged) {
                     if (lane < jn) {
-                        sp[lane] = PT<R>::load(pts, jb + lane);
-                        sn[lane] = __ldg(nsrc + jb + lane);
+                        const float4 pj = __ldg(pp.p32 + jb + lane);
+                        sw.p[lane] = make_int4(static_cast<int>(pj.x), static_cast<int>(pj.y), static_cast<int>(pj.z), 0);
+                        sw.qn[lane] = make_double2(__ldg(pp.q64 + jb + lane), __ldg(pp.n64 + jb + lane));
                     }
                     staged = true;
                 }
@@ -1245,11 +1404,11 @@ __global__ void __launch_bounds__(NT, 1) k_pair(const __grid_constant__ PairLaun
                 // this lane's j point: images that bring the i box within the cutoff
                 unsigned jm = 0u;
                 if (lane < jn) {
-                    const P pjl = sp[lane];
+                    const int4 pjl = sw.p[lane];
                     const float px = static_cast<float>(pjl.x), py = static_cast<float>(pjl.y),
                                 pz = static_cast<float>(pjl.z);
                     for (int b = 0; b < nimg; ++b) {
-                        const P sft = simg[b];
+                        const int4 sft = sw.img[b];
                         const float sx = static_cast<float>(sft.x), sy = static_cast<float>(sft.y),
                                     sz = static_cast<float>(sft.z);
                         float d2;
@@ -1273,80 +1432,99 @@ __global__ void __launch_bounds__(NT, 1) k_pair(const __grid_constant__ PairLaun
                         if (!use_cut || d2 <= rc2_box) jm |= 1u << b;
                     }
                 }
-                R a_acc = 0, u_acc = 0;  // i side (this lane's i)
-                R ja = 0, ju = 0;        // j side: lane L collects j = jb + L
-                    for (int jj = 0; jj < jn; ++jj) {
-                        unsigned m = __shfl_sync(0xffffffffu, jm, jj);
-                        if (m == 0u) continue;
-                        item_evals += static_cast<unsigned>(__popc(m));
-                        const P pj = sp[jj];
-                        const R nj = sn[jj];
-                        const bool both = !diag || jj > lane;
-                        const bool lane_ok = act && (both || jj == lane);
-                        Delta<R> dp;
-                        delta_part<POT, R>(qi, pj.w, K, dp);
-                        R sA = 0, sU = 0, cA = 0, cU = 0;
-                        unsigned ins = 0, hits = 0;
-                        do {
-                            const int b = __ffs(m) - 1;
-                            m &= m - 1u;
-                            const P sft = simg[b];
-                            const R dx = (xi + sft.x) - pj.x, dy = (yi + sft.y) - pj.y, dz = (zi + sft.z) - pj.z;
-                            R r2 = h2[0] * (dx * dx) + h2[1] * (dy * dy) + h2[2] * (dz * dz);
-                            if (SKEW) r2 += g2x[0] * (dx * dy) + g2x[1] * (dx * dz) + g2x[2] * (dy * dz);
-                            if (lane_ok && !(use_cut && beyond<SKEW>(r2, dx, dy, dz, cut))) {
-                                R phi, rd = 0, rd2 = 0;
-                                dist_part<POT, R>(r2, qi, pj.w, inv_qi, qi2, dp, K, tb, phi, rd, rd2);
-                                sA += phi;
+                for (unsigned jset = __ballot_sync(0xffffffffu, jm != 0u); jset != 0u; jset &= jset - 1u) {
+                    const int jj = __ffs(jset) - 1;
+                    unsigned m = __shfl_sync(0xffffffffu, jm, jj);
+                    item_evals += static_cast<unsigned>(__popc(m));
+                    const int4 pj = sw.p[jj];
+                    const double2 qnj = sw.qn[jj];
+                    const double qj = qnj.x, nj = qnj.y;
+                    // off the diagonal every pair counts for i and for j; in the diagonal tile j > i
+                    // for both, j = i (self-images; the self term is added at the end) for i only
+                    const bool both = !diag || jj > lane;
+                    const bool lane_ok = act && (both || jj == lane);
+                    Delta64 dp;
+                    delta_part64<POT>(qi, qj, K, dp);
+                    double A = 0.0, Srpt = 0.0, Spu = 0.0, Uf = 0.0, Vf = 0.0;
+                    unsigned ins = 0;
+                    do {
+                        const int4 sft = sw.img[__ffs(m) - 1];
+                        m &= m - 1u;
+                        double r = pair_r<SKEW>(pp, xi + (sft.x - pj.x), yi + (sft.y - pj.y), zi + (sft.z - pj.z));
+                        const bool in = lane_ok && __double2hiint(r) > 0;  // r <= 0: outside, or the self term
+                        ins += in ? 1u : 0u;
+                        r = in ? r : 0.0;
+                        const double tD = r * dp.sqcD;
+                        int kc;
+                        double t;
+                        bool on = cell_of(tD, K.kmax + 1, kc, t);
+                        if (__any_sync(0xffffffffu, !on || !poly)) {
+                            const bool end = !on && tD == K.tDmax;  // the last node: its cell at t = 1
+                            on = on || end;
+                            kc = end ? K.kmax : (on ? kc : 0);
+                            t = end ? 1.0 : (on ? t : 0.0);
+                            if (in && !(on && poly)) {
+                                double phi, rd = 0.0, rd2 = 0.0;
+                                if (on) {
+                                    // a table too large for polynomials: from its coefficients
+                                    Delta<double> dd;
+                                    delta_part<POT, double>(qi, qj, K, dd);
+                                    dist_part<POT, double>(r, r * r, qi, qj, 1.0 / qi, qi * qi, dd, K, tb, phi, rd, rd2);
+                                } else {
+                                    past_part64<POT>(r, tD, qi, qj, K, tb.rho, phi, rd, rd2);
+                                }
+                                A += phi;
                                 if (POT) {
-                                    sU += rd;
-                                    cA += phi;
-                                    cU += rd2;
-                                }
-                                ins += 1u;
-                                hits += (r2 > R(0)) ? 1u : 0u;
-                            }
-                        } while (m != 0u);
-                        const unsigned wt = both ? 2u : 1u;  // ordered pairs represented
-                        cnt += hits * wt;
-                        nclamp += dp.cl ? ins * wt : 0u;
-                        if (POT) {
-                            a_acc += nj * sA;
-                            u_acc += nj * sU;
-                        } else {
-                            a_acc += static_cast<R>(wt) * nj * sA;
-                        }
-                        if (POT) {
-                            cA = both ? ni * cA : R(0);
-                            cU = both ? ni * cU : R(0);
-                            if (__any_sync(0xffffffffu, cA != R(0) || cU != R(0))) {
-                                cA = warp_sum(cA);
-                                cU = warp_sum(cU);
-                                if (lane == jj) {
-                                    ja += cA;
-                                    ju += cU;
+                                    Uf += rd;
+                                    Vf += rd2;
                                 }
                             }
+                            if (!poly) continue;
                         }
+                        double p, pt, pu;
+                        spline64<POT>(poly, sh.S, kc, t, dp, p, pt, pu);
+                        A += in && on ? p : 0.0;
+                        if (POT) {
+                            Srpt = fma(on ? r : 0.0, pt, Srpt);
+                            Spu += in && on ? pu : 0.0;
+                        }
+                    } while (m != 0u);
+                    const unsigned wt = both ? 2u : 1u;  // ordered pairs represented
+                    cnt += ins * wt;
+                    nclamp += dp.cl ? ins * wt : 0u;
+                    if (POT) {
+                        const double u = fma(Spu, dp.b1, Srpt * K.cD), v = Spu * dp.sb;
+                        A64 = fma(nj, A, A64);
+                        U64 = fma(nj, u + Uf, U64);
+                        const double nb = both ? ni : 0.0;
+                        const double tot = warp_sum2(nb * A, nb * ((u - v) - v + Vf), hi);
+                        if ((lane & 15) == 0) sw.js[lane >> 4][jj] = tot;
+                    } else {
+                        A64 = fma(both ? nj + nj : nj, A, A64);
                     }
-                A64 += static_cast<double>(a_acc);
-                U64 += static_cast<double>(u_acc);
-                if (POT && lane < jn) {
-                    if (ja != R(0)) atomicAdd(pp.A + jb + lane, static_cast<double>(ja));
-                    if (ju != R(0)) atomicAdd(pp.U + jb + lane, static_cast<double>(sn[lane]) * static_cast<double>(ju));
+                }
+                if (POT) {
+                    __syncwarp();
+                    if (jm != 0u) {
+                        const double ja = sw.js[0][lane], ju = sw.js[1][lane];
+                        if (ja != 0.0) atomicAdd(pp.A + jb + lane, ja);
+                        if (ju != 0.0) atomicAdd(pp.U + jb + lane, sw.qn[lane].y * ju);
+                    }
                 }
             }
         }
+        // the self term n_i phi(0, 0) of the i points whose diagonal tile this item holds
+        if (act && c == 0) A64 = fma(ni, sh.phi00, A64);
         if (act && POT) {
             if (A64 != 0.0) atomicAdd(pp.A + ig, A64);
-            if (U64 != 0.0) atomicAdd(pp.U + ig, static_cast<double>(ni) * U64);
+            if (U64 != 0.0) atomicAdd(pp.U + ig, ni * U64);
         }
         count_item(pp.stats, act ? cnt : 0u, act ? nclamp : 0u,
                    static_cast<unsigned long long>(item_evals) * static_cast<unsigned long long>(ni_act));
         if (!POT) {
             // the item's energy partial, summed over lanes in a fixed order (items
             // beyond the partials' capacity are added atomically)
-            const double e = warp_sum(act ? static_cast<double>(ni) * A64 : 0.0);
+            const double e = warp_sum(act ? ni * A64 : 0.0);
             if (lane == 0) {
                 if (sh.item_E && item < sh.item_cap)
                     sh.item_E[item] = e;
@@ -1356,6 +1534,18 @@ __global__ void __launch_bounds__(NT, 1) k_pair(const __grid_constant__ PairLaun
         }
     }
     }
+}
+
+// Per D cell k and delta column l the cubic in t (times 1, as the coefficients / 36 give
+// it) through rows k .. k + 3 of the bicubic coefficients: poly[(k S + l) 4 ...].
+__global__ void k_table_poly(const double *__restrict__ c, long long n, int S, double *__restrict__ poly) {
+    const long long e = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x;
+    if (e >= n) return;
+    const double c0 = c[e], c1 = c[e + S], c2 = c[e + 2LL * S], c3 = c[e + 3LL * S];
+    poly[4 * e] = c0 + 4.0 * c1 + c2;
+    poly[4 * e + 1] = 3.0 * (c2 - c0);
+    poly[4 * e + 2] = 3.0 * ((c0 - c1) + (c2 - c1));
+    poly[4 * e + 3] = (c3 - c0) + 3.0 * (c1 - c2);
 }
 
 // The splitmix64 output function (Steele, Lea and Flood, "Fast splittable
@@ -1590,10 +1780,23 @@ int launch_nt(int threads, bool skew, const PairLaunch &pl, int nctas, size_t sm
 
 int pair_smem_bytes(int precision, int threads, int ksn, int S) {
     // per warp: j tile (points, densities) and image shifts; FP32: the table band
-    const size_t warp = precision == VDWDF_FP64 ? (2 * sizeof(dvec4) + sizeof(double)) * kTile : sizeof(Warp32);
+    const size_t warp = precision == VDWDF_FP64 ? sizeof(Warp64) : sizeof(Warp32);
     size_t b = warp * static_cast<size_t>(threads / 32);
     if (precision != VDWDF_FP64) b += static_cast<size_t>(ksn) * band_stride(S) * sizeof(float);
     return static_cast<int>(b);
+}
+
+// The displacement table of an instance into rt.
+static int launch_r_table(const PairParams &pp, bool skew, double *rt, cudaStream_t st) {
+    const long long n = r_table_entries(pp.rtm, skew);
+    const int nb = static_cast<int>(n < (1LL << 18) ? (n + 255) / 256 : 1024);
+    if (skew)
+        k_r_table<true><<<nb, 256, 0, st>>>(pp, rt);
+    else
+        k_r_table<false><<<nb, 256, 0, st>>>(pp, rt);
+    count_launches(1);
+    VDWDF_CUDA_TRY(cudaGetLastError());
+    return VDWDF_OK;
 }
 
 int launch_pair(int precision, bool potential, bool skew, int threads, const PairLaunch &pl, int nctas,
@@ -1601,10 +1804,23 @@ int launch_pair(int precision, bool potential, bool skew, int threads, const Pai
     if (skew && threads != 640 && threads != 512 && threads != 448 && threads != 384) return VDWDF_EINVAL;  // skewed: 384, 448, 512
     const size_t smem = static_cast<size_t>(pair_smem_bytes(precision, threads, pl.sh.ksn, pl.sh.S));
     if (precision == VDWDF_FP64)
+        for (int k = 0; k < pl.ninst; ++k)
+            if (pl.inst[k].rt) {
+                const int rc = launch_r_table(pl.inst[k], skew, const_cast<double *>(pl.inst[k].rt), st);
+                if (rc) return rc;
+            }
+    if (precision == VDWDF_FP64)
         return potential ? launch_nt<double, 1>(threads, skew, pl, nctas, smem, st)
                          : launch_nt<double, 0>(threads, skew, pl, nctas, smem, st);
     return potential ? launch_nt<float, 1>(threads, skew, pl, nctas, smem, st)
                      : launch_nt<float, 0>(threads, skew, pl, nctas, smem, st);
+}
+
+int launch_table_poly(const double *coef, int nD, int S, double *poly) {
+    const long long n = static_cast<long long>(nD - 1) * S;
+    k_table_poly<<<static_cast<int>((n + 255) / 256), 256>>>(coef, n, S, poly);
+    VDWDF_CUDA_TRY(cudaGetLastError());
+    return VDWDF_OK;
 }
 
 int launch_band_choose(const PairLaunch &pl, unsigned int *hist, cudaStream_t st) {

@@ -198,7 +198,7 @@ __global__ void k_scan(const int *__restrict__ cnt, int nb, int *__restrict__ of
 __global__ void k_scatter(BrickGeom g, const int *__restrict__ order, int nb,
                           const double *__restrict__ n, double n_cut, const double *__restrict__ q0,
                           const int *__restrict__ off, int *__restrict__ slot, float4 *__restrict__ p32,
-                          float *__restrict__ n32, dvec4 *__restrict__ p64, double *__restrict__ n64) {
+                          float *__restrict__ n32, double *__restrict__ q64, double *__restrict__ n64) {
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int lane = threadIdx.x & 31;
     if (warp >= nb) return;
@@ -220,14 +220,7 @@ __global__ void k_scatter(BrickGeom g, const int *__restrict__ order, int nb,
             p32[s] = make_float4(static_cast<float>(a), static_cast<float>(b), static_cast<float>(c),
                                  static_cast<float>(q));
             n32[s] = static_cast<float>(nn);
-            if (p64) {
-                dvec4 v;
-                v.x = a;
-                v.y = b;
-                v.z = c;
-                v.w = q;
-                p64[s] = v;
-            }
+            if (q64) q64[s] = q;
             n64[s] = nn;
             if (slot) slot[m] = s;
         } else if (valid && slot) {
@@ -440,7 +433,7 @@ int launch_grad_q0(const int dims[3], const AxisMap &am, const double *n, const 
 
 int launch_compact(const int dims[3], const double *n, double n_cut, const double *q0,
                    const int *brick_order, int nbricks, int *brick_cnt, int *brick_off, int *slot,
-                   float4 *p32, float *n32, dvec4 *p64, double *n64, float4 *blo, float4 *bhi,
+                   float4 *p32, float *n32, double *q64, double *n64, float4 *blo, float4 *bhi,
                    Stats *stats, cudaStream_t st) {
     BrickGeom g;
     g.n0 = dims[0];
@@ -455,7 +448,7 @@ int launch_compact(const int dims[3], const double *n, double n_cut, const doubl
     k_scan<<<1, 1024, 0, st>>>(brick_cnt, nbricks, brick_off, stats);
     VDWDF_CUDA_TRY(cudaGetLastError());
     k_scatter<<<blocks, 32 * wpb, 0, st>>>(g, brick_order, nbricks, n, n_cut, q0, brick_off, slot, p32,
-                                           n32, p64, n64);
+                                           n32, q64, n64);
     VDWDF_CUDA_TRY(cudaGetLastError());
     const long long N = static_cast<long long>(dims[0]) * dims[1] * dims[2];
     const int tiles = static_cast<int>((N + kTile - 1) / kTile);

@@ -98,6 +98,52 @@ def test_table_shapes(V, oracle_mod, shape):
     _check(V, oracle_mod, table, spline, n, cell, periodic, 1e-6, r_cut)
 
 
+def _check_fp64(V, oracle_mod, table, spline, n, cell, periodic, n_cut, r_cut):
+    """The FP64 path against the oracle with its stated tolerances: E and v 1e-10."""
+    diagonal = np.array_equal(cell, np.diag(np.diag(cell)))
+    P = oracle_mod.Problem(n, np.diag(cell), periodic, n_cut, r_cut, spline, cell=None if diagonal else cell)
+    e = P.energy()
+    v = P.potential(e["A"], e["U"])
+    geo = np.diag(cell) if diagonal else cell
+    E, r = V.energy(_t(n), geo, periodic, n_cut, r_cut, table, "fp64")
+    Ev, vg, rv = V.potential(_t(n), geo, periodic, n_cut, r_cut, table, "fp64")
+    assert abs(E - e["E"]) <= 1e-10 * abs(e["E"])
+    assert abs(Ev - e["E"]) <= 1e-10 * abs(e["E"])
+    assert np.max(np.abs(vg.cpu().numpy() - v)) <= 1e-10 * np.max(np.abs(v))
+    for res in (r, rv):
+        assert res["n_active"] == P.n_active and res["pairs"] == e["pairs"]
+
+
+@pytest.mark.parametrize("kind", sorted(CELLS))
+@pytest.mark.parametrize("active", [1, 31, 32, 33, 64, 65, 97])
+def test_active_counts_fp64(V, oracle_mod, gtable, oracle_spline, kind, active):
+    cell, periodic, r_cut = CELLS[kind]
+    n = _density((9, 8, 7), cell, active)
+    s = np.sort(n, axis=None)[::-1]
+    _check_fp64(V, oracle_mod, gtable, oracle_spline, n, cell, periodic, 0.5 * (s[active - 1] + s[active]), r_cut)
+
+
+@pytest.mark.parametrize("shape", [(4, 4), (9, 5), (70000, 60)])
+def test_table_shapes_fp64(V, oracle_mod, shape):
+    """The smallest table, a small one, and one too large to be kept as polynomials."""
+    nD, nd = shape
+    D = np.linspace(0.0, 12.0, nD)[:, None]
+    dl = (np.arange(nd) / nd)[None, :]
+    nodes = (1.0 - 0.3 * dl ** 2) * np.exp(-0.2 * D) * np.cos(0.3 * D) - 1e-3
+    cell, periodic, r_cut = CELLS["slab"]
+    n = _density((9, 8, 7), cell, 6)
+    _check_fp64(V, oracle_mod, V.Table.from_nodes(nodes, 12.0), oracle_mod.Spline(nodes, 12.0), n, cell, periodic,
+                1e-6, r_cut)
+
+
+def test_displacements_beyond_a_table_fp64(V, oracle_mod, gtable, oracle_spline):
+    """Three points and a cutoff so long that the index displacements fill no table."""
+    cell = np.diag((5.0, 4.4, 8.0))
+    n = _density((9, 8, 7), cell, 8)
+    s = np.sort(n, axis=None)[::-1]
+    _check_fp64(V, oracle_mod, gtable, oracle_spline, n, cell, (True, True, True), 0.5 * (s[2] + s[3]), 150.0)
+
+
 @pytest.mark.parametrize("precision,tol", [("fp32", 1e-6), ("fp64", 1e-12)])
 def test_orthogonal_beside_skewed_in_a_batch(V, gtable, precision, tol):
     """Orthogonal and skewed cells in one batched launch give the single calls' energies."""
