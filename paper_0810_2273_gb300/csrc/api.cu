@@ -1,7 +1,7 @@
 // extern "C" entry points of libvdwdf (declared in include/vdwdf.h).
 //
-// A call validates its arguments on the host, takes scratch with
-// cudaMallocAsync on the caller's stream, runs
+// A call validates its arguments on the host, takes scratch from the library's
+// memory pool on the caller's stream, runs
 //   gradient + q0  ->  trimming into brick order  ->  tile boxes  ->  pair kernel
 //   (-> potential assembly)  ->  reductions,
 // reads the counters back and frees the scratch on the same stream.
@@ -62,7 +62,58 @@ unsigned int max_iters_override(unsigned int v) {
     const long long k = std::atoll(e);
     return (k > 0 && static_cast<unsigned long long>(k) < v) ? static_cast<unsigned int>(k) : v;
 }
-// cudaMallocAsync / cudaMalloc of a call's scratch, with the fault-injection hook
+// The library's own stream-ordered memory pool of a device, which the calls that wait
+// for their stream take scratch from.  It keeps at most kPoolKeep bytes between calls:
+// the device's default pool gives its memory back at every synchronisation, and
+// mapping it again took half of a small call (Kr dimer 24 x 18 x 18, E FP32: 533 us of
+// which the pair pass is 220, against 343 with the pool).  Trimmed to nothing
+// when the last table is freed.
+constexpr unsigned long long kPoolKeep = 64ull << 20;
+std::mutex g_pool_mu;
+std::map<int, cudaMemPool_t> g_pools;
+std::atomic<long long> g_tables{0};  // live tables
+
+cudaError_t scratch_pool(cudaMemPool_t *pool) {
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    auto it = g_pools.find(dev);
+    if (it == g_pools.end()) {
+        cudaMemPoolProps props;
+        std::memset(&props, 0, sizeof(props));
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = dev;
+        cudaMemPool_t p = nullptr;
+        e = cudaMemPoolCreate(&p, &props);
+        if (e != cudaSuccess) return e;
+        unsigned long long keep = kPoolKeep;
+        e = cudaMemPoolSetAttribute(p, cudaMemPoolAttrReleaseThreshold, &keep);
+        if (e != cudaSuccess) {
+            cudaMemPoolDestroy(p);
+            return e;
+        }
+        it = g_pools.emplace(dev, p).first;
+    }
+    *pool = it->second;
+    return cudaSuccess;
+}
+
+void trim_pools() {
+    std::lock_guard<std::mutex> lk(g_pool_mu);
+    for (auto &kv : g_pools) cudaMemPoolTrimTo(kv.second, 0);
+}
+
+// A call's scratch, with the fault-injection hook: from the library's pool (freed with
+// cudaFreeAsync), from the device's default pool for the calls that do not wait for
+// their stream (a caller may capture those), or for a batch plan.
+cudaError_t scratch_malloc_pool(void **p, size_t bytes, cudaStream_t st) {
+    if (fail_alloc_requested()) return cudaErrorMemoryAllocation;
+    cudaMemPool_t pool = nullptr;
+    const cudaError_t e = scratch_pool(&pool);
+    return e != cudaSuccess ? e : cudaMallocFromPoolAsync(p, bytes, pool, st);
+}
 cudaError_t scratch_malloc_async(void **p, size_t bytes, cudaStream_t st) {
     if (fail_alloc_requested()) return cudaErrorMemoryAllocation;
     return cudaMallocAsync(p, bytes, st);
@@ -94,6 +145,7 @@ int finish_table(vdwdf_table *t) {
         t->coef64[i] /= (i < main) ? 36.0 : 6.0;
         t->coef32[i] = static_cast<float>(t->coef64[i]);
     }
+    ++g_tables;  // (both callers keep the table from here on)
     return VDWDF_OK;
 }
 
@@ -753,7 +805,7 @@ int run_single(const vdwdf_grid *grid, const double *n_dev, const double *grad_d
     const bool fp64 = precision == VDWDF_FP64;
     const size_t bytes = layout(G, nb, pot, fp64, nullptr, nullptr);
     unsigned char *base = nullptr;
-    if (scratch_malloc_async(reinterpret_cast<void **>(&base), bytes, st) != cudaSuccess) return VDWDF_EALLOC;
+    if (scratch_malloc_pool(reinterpret_cast<void **>(&base), bytes, st) != cudaSuccess) return VDWDF_EALLOC;
     Work w;
     layout(G, nb, pot, fp64, &w, base);
     Timer tm;
@@ -783,7 +835,7 @@ int run_single(const vdwdf_grid *grid, const double *n_dev, const double *grad_d
             fill_shared(table, td, ln, w.queue, static_cast<unsigned int>(items + 2), pl.sh);
             if (!pot) {
                 // one energy partial per work item, summed afterwards in a fixed order
-                if (scratch_malloc_async(reinterpret_cast<void **>(&item_buf), sizeof(double) * items, st) != cudaSuccess)
+                if (scratch_malloc_pool(reinterpret_cast<void **>(&item_buf), sizeof(double) * items, st) != cudaSuccess)
                     return VDWDF_EALLOC;
                 pl.sh.item_E = item_buf;
                 pl.sh.item_cap = static_cast<unsigned int>(items);
@@ -1133,6 +1185,7 @@ void vdwdf_table_free(vdwdf_table *t) {
     }
     if (have) cudaSetDevice(cur);
     delete t;
+    if (--g_tables == 0) trim_pools();
 }
 
 int vdwdf_kernel_eval(const vdwdf_table *t, int precision, int64_t npts, const double *r_dev,
@@ -1202,7 +1255,7 @@ int vdwdf_semilocal(const vdwdf_grid *grid, const double *n_dev, const double *g
     // the spectral gradient (when the grid asks for it and none is given) after the sums
     const size_t nsp = (G.spectral && !grad_dev) ? 3 * static_cast<size_t>(G.N) + G.dims[0] + G.dims[1] + G.dims[2] : 0;
     double *scratch = nullptr;
-    if (scratch_malloc_async(reinterpret_cast<void **>(&scratch), (nd + nsp) * sizeof(double), st) != cudaSuccess)
+    if (scratch_malloc_pool(reinterpret_cast<void **>(&scratch), (nd + nsp) * sizeof(double), st) != cudaSuccess)
         return VDWDF_EALLOC;
     Timer tm;
     double sums[6] = {0, 0, 0, 0, 0, 0};
@@ -1246,7 +1299,7 @@ int vdwdf_phi0_eval(const vdwdf_table *table, const double *voxel, int64_t nq, c
     std::vector<double> xw;
     phi0_rule(xw);
     double *xw_dev = nullptr;
-    if (scratch_malloc_async(reinterpret_cast<void **>(&xw_dev), sizeof(double) * (xw.size() + 8 * nq), st) !=
+    if (scratch_malloc_pool(reinterpret_cast<void **>(&xw_dev), sizeof(double) * (xw.size() + 8 * nq), st) !=
         cudaSuccess)
         return VDWDF_EALLOC;
     Launch ln;
@@ -1306,7 +1359,7 @@ int diag_voxel(const vdwdf_grid *grid, const double *n_dev, const double *grad_d
                  o_coef = G.spectral ? c.take<double>(G.dims[0] + G.dims[1] + G.dims[2]) : 0,
                  o_div = (G.spectral && pot) ? c.take<double>(G.N) : 0;
     unsigned char *base = nullptr;
-    if (scratch_malloc_async(reinterpret_cast<void **>(&base), c.off, st) != cudaSuccess) return VDWDF_EALLOC;
+    if (scratch_malloc_pool(reinterpret_cast<void **>(&base), c.off, st) != cudaSuccess) return VDWDF_EALLOC;
     double *q0 = reinterpret_cast<double *>(base + o_q0);
     unsigned long long *mm = reinterpret_cast<unsigned long long *>(base + o_mm);
     double *part = reinterpret_cast<double *>(base + o_part), *sums = reinterpret_cast<double *>(base + o_sums);
@@ -1404,7 +1457,7 @@ int autotune_one(const Geom &G, const double *n_dev, double n_cut, const vdwdf_t
     const bool fp64 = precision == VDWDF_FP64;
     const size_t bytes = layout(G, nb, false, fp64, nullptr, nullptr);
     unsigned char *base = nullptr;
-    if (scratch_malloc_async(reinterpret_cast<void **>(&base), bytes, st) != cudaSuccess) return VDWDF_EALLOC;
+    if (scratch_malloc_pool(reinterpret_cast<void **>(&base), bytes, st) != cudaSuccess) return VDWDF_EALLOC;
     Work w;
     layout(G, nb, false, fp64, &w, base);
     rc = prepare(G, n_dev, nullptr, n_cut, false, w, st);
@@ -1553,7 +1606,7 @@ int vdwdf_far_tail(const vdwdf_grid *grid, const double *n_dev, const double *gr
                  o_slot = pot ? cv.take<int>(G.N) : 0, o_A = pot ? cv.take<double>(G.N) : 0,
                  o_U = pot ? cv.take<double>(G.N) : 0, o_div = (pot && G.spectral) ? cv.take<double>(G.N) : 0;
     unsigned char *base = nullptr;
-    if (scratch_malloc_async(reinterpret_cast<void **>(&base), cv.off, st) != cudaSuccess) return VDWDF_EALLOC;
+    if (scratch_malloc_pool(reinterpret_cast<void **>(&base), cv.off, st) != cudaSuccess) return VDWDF_EALLOC;
     double *Gk = pot ? reinterpret_cast<double *>(base + o_G) : nullptr;
     double *qn = pot ? reinterpret_cast<double *>(base + o_qn) : nullptr;
     double *qgr = pot ? reinterpret_cast<double *>(base + o_qg) : nullptr;
@@ -1628,7 +1681,7 @@ int vdwdf_far_tail(const vdwdf_grid *grid, const double *n_dev, const double *gr
                          o_lF = lc.take<double>(static_cast<size_t>(nodes) * La),
                          o_lG = lc.take<double>(static_cast<size_t>(nodes) * La),
                          o_Kt = lc.take<double>(static_cast<size_t>(Nb) * (2 * Nc - 1));
-            if (scratch_malloc_async(reinterpret_cast<void **>(&lbase), lc.off, st) != cudaSuccess) return VDWDF_EALLOC;
+            if (scratch_malloc_pool(reinterpret_cast<void **>(&lbase), lc.off, st) != cudaSuccess) return VDWDF_EALLOC;
             int *dlist = reinterpret_cast<int *>(lbase + o_list);
             int *dlslot = reinterpret_cast<int *>(lbase + o_lslot);
             double *lF = reinterpret_cast<double *>(lbase + o_lF), *lG = reinterpret_cast<double *>(lbase + o_lG);
