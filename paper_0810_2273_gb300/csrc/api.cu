@@ -1589,25 +1589,19 @@ int vdwdf_far_tail(const vdwdf_grid *grid, const double *n_dev, const double *gr
     constexpr int kMaxLines = 65536;   // active lines of one periodic axis (K over their pairs)
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     const long long launches0 = g_launches.load();
-    // the planes' F and G; for one periodic axis the lines' buffers come later, once
-    // the active lines are known
-    const size_t ngroup = nper == 1 ? 1 : static_cast<size_t>(np);
+    // the sums' buffers come later, once the nodes and the active lines are known
     Carve cv;
-    const size_t o_q0 = cv.take<double>(G.N), o_mm = cv.take<unsigned long long>(3),
-                 o_F = cv.take<double>(static_cast<size_t>(kMaxNodes) * ngroup), o_Tk = cv.take<double>(kMaxNodes),
-                 o_out = cv.take<double>(1);
+    const size_t o_q0 = cv.take<double>(G.N), o_mm = cv.take<unsigned long long>(3), o_out = cv.take<double>(1);
     const size_t o_gsp = G.spectral ? cv.take<double>(3 * G.N) : 0,
                  o_coef = G.spectral ? cv.take<double>(G.dims[0] + G.dims[1] + G.dims[2]) : 0;
     const size_t o_flags = nper == 1 ? cv.take<int>(nlines) : 0;
-    // the potential: G_k(p), dq0/dn, dq0/dgrad n, the slot map, A and U on the grid, and
-    // the spectral divergence
-    const size_t o_G = pot ? cv.take<double>(static_cast<size_t>(kMaxNodes) * ngroup) : 0,
-                 o_qn = pot ? cv.take<double>(G.N) : 0, o_qg = pot ? cv.take<double>(3 * G.N) : 0,
+    // the potential: dq0/dn, dq0/dgrad n, the slot map, A and U on the grid, and the
+    // spectral divergence
+    const size_t o_qn = pot ? cv.take<double>(G.N) : 0, o_qg = pot ? cv.take<double>(3 * G.N) : 0,
                  o_slot = pot ? cv.take<int>(G.N) : 0, o_A = pot ? cv.take<double>(G.N) : 0,
                  o_U = pot ? cv.take<double>(G.N) : 0, o_div = (pot && G.spectral) ? cv.take<double>(G.N) : 0;
     unsigned char *base = nullptr;
     if (scratch_malloc_pool(reinterpret_cast<void **>(&base), cv.off, st) != cudaSuccess) return VDWDF_EALLOC;
-    double *Gk = pot ? reinterpret_cast<double *>(base + o_G) : nullptr;
     double *qn = pot ? reinterpret_cast<double *>(base + o_qn) : nullptr;
     double *qgr = pot ? reinterpret_cast<double *>(base + o_qg) : nullptr;
     int *slot = pot ? reinterpret_cast<int *>(base + o_slot) : nullptr;
@@ -1616,12 +1610,11 @@ int vdwdf_far_tail(const vdwdf_grid *grid, const double *n_dev, const double *gr
     double *divb = (pot && G.spectral) ? reinterpret_cast<double *>(base + o_div) : nullptr;
     double *q0 = reinterpret_cast<double *>(base + o_q0);
     unsigned long long *mm = reinterpret_cast<unsigned long long *>(base + o_mm);
-    double *F = reinterpret_cast<double *>(base + o_F), *Tk = reinterpret_cast<double *>(base + o_Tk);
     double *Tout = reinterpret_cast<double *>(base + o_out);
     double *gsp = G.spectral ? reinterpret_cast<double *>(base + o_gsp) : nullptr;
     double *coef = G.spectral ? reinterpret_cast<double *>(base + o_coef) : nullptr;
     int *flags = nper == 1 ? reinterpret_cast<int *>(base + o_flags) : nullptr;
-    unsigned char *lbase = nullptr;  // one periodic axis: the lines' buffers
+    unsigned char *lbase = nullptr;  // the sums' buffers
     Timer tm;
     unsigned long long hmm[3] = {0, 0, 0};
     double T = 0.0;
@@ -1648,16 +1641,33 @@ int vdwdf_far_tail(const vdwdf_grid *grid, const double *n_dev, const double *gr
         // nodes x_k = x0 + k hx of int_0^inf e^{-c s} ds = int e^{-c e^x} e^x dx over
         // c = u_i + u_j in [2 umin, 2 umax]: the part below x0 is under 1e-17 of 1/c
         // for every c, e^{-c e^x} has fallen below e^-45 past the last node, and the
-        // step's error (exp(-pi^2 / hx) up to a factor) measures 1.2e-13 relative for
-        // 1/c and 2.5e-12 for 1/c^2 (the potential's second sum) over that range
-        const double umin = qmin * qmin, umax = qmax * qmax, hx = 0.3;
+        // step's error falls like exp(-pi^2 / hx) (a step of 0.3, with 1.2e-13 relative
+        // for 1/c and 2.5e-12 for 1/c^2, was enough; ln 2 / 3 makes runs of doublings)
+        const double umin = qmin * qmin, umax = qmax * qmax, hx = std::log(2.0) / 3.0;
         const double x0 = std::log(1e-17 / (2.0 * umax)), x1 = std::log(45.0 / (2.0 * umin));
-        nodes = static_cast<int>(std::ceil((x1 - x0) / hx)) + 1;
-        if (nodes > kMaxNodes) return VDWDF_EUNSUPPORTED;
+        if (std::ceil((x1 - x0) / 0.3) + 1.0 > kMaxNodes) return VDWDF_EUNSUPPORTED;
+        // the first ntaylor nodes have umax s <= 1/16 (see TailNodes)
+        const int ntaylor = static_cast<int>(std::floor((std::log(1.0 / (16.0 * umax)) - x0) / hx)) + 1;
+        TailNodes tn;
+        tn.hx = hx;
+        tn.iumax = 1.0 / umax;
+        for (double &w : tn.W) w = 0.0;
+        for (int k = 0; k < ntaylor; ++k) {
+            const double s = std::exp(x0 + k * hx);
+            double p = hx * s;
+            for (double &w : tn.W) {
+                w += p;
+                p *= umax * s;
+            }
+        }
+        for (int r = 0; r < 3; ++r) tn.s[r] = std::exp(x0 + (ntaylor + r) * hx);
+        tn.nb = std::max(1, static_cast<int>(std::ceil((x1 - x0) / hx)) + 1 - ntaylor);
+        nodes = ntaylor + tn.nb;
+        const size_t rows = static_cast<size_t>(kTailMoments + tn.nb), ndots = tn.nb + kTailMoments * kTailMoments;
         const double Cas = 12.0 * std::pow(4.0 * kPi / 9.0, 3);
         const double scale = -0.5 * G.dV * G.dV * Cas;
         const int *line_slot = nullptr;
-        double *Gl = Gk;
+        double *Gl = nullptr, *cf = nullptr;
         if (nper == 1) {
             // the lines along the periodic axis that hold an active point
             VDWDF_CUDA_TRY(cudaMemsetAsync(flags, 0, sizeof(int) * nlines, st));
@@ -1677,9 +1687,9 @@ int vdwdf_far_tail(const vdwdf_grid *grid, const double *n_dev, const double *gr
             groups = La;
             const int Nb = nlines / Nc;
             Carve lc;
-            const size_t o_list = lc.take<int>(La), o_lslot = lc.take<int>(nlines),
-                         o_lF = lc.take<double>(static_cast<size_t>(nodes) * La),
-                         o_lG = lc.take<double>(static_cast<size_t>(nodes) * La),
+            const size_t o_list = lc.take<int>(La), o_lslot = lc.take<int>(nlines), o_lF = lc.take<double>(rows * La),
+                         o_lG = lc.take<double>(rows * La), o_dots = lc.take<double>(ndots),
+                         o_cf = lc.take<double>(2 * kTailMoments * static_cast<size_t>(La)),
                          o_Kt = lc.take<double>(static_cast<size_t>(Nb) * (2 * Nc - 1));
             if (scratch_malloc_pool(reinterpret_cast<void **>(&lbase), lc.off, st) != cudaSuccess) return VDWDF_EALLOC;
             int *dlist = reinterpret_cast<int *>(lbase + o_list);
@@ -1688,21 +1698,30 @@ int vdwdf_far_tail(const vdwdf_grid *grid, const double *n_dev, const double *gr
             double *Kt = reinterpret_cast<double *>(lbase + o_Kt);
             VDWDF_CUDA_TRY(cudaMemcpyAsync(dlist, list.data(), sizeof(int) * La, cudaMemcpyHostToDevice, st));
             VDWDF_CUDA_TRY(cudaMemcpyAsync(dlslot, lslot.data(), sizeof(int) * nlines, cudaMemcpyHostToDevice, st));
-            r = launch_far_tail_lines(G.dims, ax, La, dlist, n_dev, q0, n_cut, x0, hx, nodes, gbb, gbc, gcc, r_cut,
-                                      pref, scale, lF, Kt, lG, Tk, Tout, st);
+            r = launch_far_tail_lines(G.dims, ax, La, dlist, n_dev, q0, n_cut, tn, gbb, gbc, gcc, r_cut, pref, scale, lF,
+                                      Kt, lG, reinterpret_cast<double *>(lbase + o_dots), Tout, st);
             if (r) return r;
             line_slot = dlslot;
             Gl = lG;
+            cf = reinterpret_cast<double *>(lbase + o_cf);
             // the host vectors are read by the copies above before they are freed: the
             // copies from pageable memory return once the data is staged
         } else {
-            r = launch_far_tail(G.dims, ax, np, n_dev, q0, n_cut, x0, hx, nodes, dz, r_cut, c2, c3, scale, F, Tk,
-                                Gk, Tout, st);
+            const int parts = far_tail_parts(tn, np, G.N);
+            Carve lc;
+            const size_t o_lF = lc.take<double>(rows * np * parts), o_lG = lc.take<double>(rows * np),
+                         o_dots = lc.take<double>(ndots),
+                         o_cf = lc.take<double>(2 * kTailMoments * static_cast<size_t>(np));
+            if (scratch_malloc_pool(reinterpret_cast<void **>(&lbase), lc.off, st) != cudaSuccess) return VDWDF_EALLOC;
+            Gl = reinterpret_cast<double *>(lbase + o_lG);
+            cf = reinterpret_cast<double *>(lbase + o_cf);
+            r = launch_far_tail(G.dims, ax, np, n_dev, q0, n_cut, tn, parts, dz, r_cut, c2, c3, scale,
+                                reinterpret_cast<double *>(lbase + o_lF), Gl, reinterpret_cast<double *>(lbase + o_dots),
+                                Tout, st);
             if (r) return r;
         }
         if (pot) {
-            r = launch_far_tail_AU(G.dims, ax, groups, line_slot, n_dev, q0, n_cut, x0, hx, nodes, Gl, Cas, slot, Ad,
-                                   Ud, st);
+            r = launch_far_tail_AU(G.dims, ax, groups, line_slot, n_dev, q0, n_cut, tn, Gl, cf, Cas, slot, Ad, Ud, st);
             if (r) return r;
             r = assemble_v(G, slot, Ad, Ud, qn, qgr, gsp, divb, coef, v_dev, nullptr, nullptr, st);
             if (r) return r;

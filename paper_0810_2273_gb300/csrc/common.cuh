@@ -214,34 +214,42 @@ int launch_diag_sum(long long N, const double *n, const double *q0, double n_cut
                     int nq, double lnq0, double dlnq, double *part, double *sums, cudaStream_t st);
 int launch_diag_AU(long long N, const double *n, const double *q0, double n_cut, const double *tab, int nq,
                    double lnq0, double dlnq, double phi00, int *slot, double *A, double *U, cudaStream_t st);
-// The far field past the cutoff (tail.cu): planes of grid axis ax (np of them, or
-// np = 1 for the whole cell), nodes of the trapezoidal rule x_k = x0 + k hx in
-// ln s; F (nodes x np) and Tk (nodes) scratch; out = scale sum_k hx e^{x_k} Tk[k]
-// with Tk[k] = sum_{p,p'} K(p, p') F_k(p) F_k(p'),
-// K = c2 / max(rc, |p - p'| dz)^4 (np > 1) or c3 (np = 1).
-// G (nodes x np, nullable) keeps G_k(p) = sum_{p'} K(p, p') F_k(p') for the potential.
+// The far field past the cutoff (tail.cu): the trapezoidal rule in ln s with step
+// hx = ln 2 / 3.  Nodes with u_max s <= 1/16 are kept as the sums W_m = sum hx s
+// (u_max s)^m over them; the nb others are s_k = s[k % 3] 2^(k / 3).
+constexpr int kTailMoments = 9;  // moments of the Taylor nodes (degree 8)
+struct TailNodes {
+    double hx, iumax;
+    double s[3];
+    double W[2 * kTailMoments];
+    int nb;
+};
+// Planes of grid axis ax (np of them, or np = 1 for the whole cell): F (parts x rows x
+// np, rows = kTailMoments + nb, the sums end in the first part) and G (rows x np), the
+// moments' and nodes' sums and K applied to them, K = c2 / max(rc, |p - p'| dz)^4 (np >
+// 1) or c3 (np = 1); out = scale sum_k hx s_k sum_{p,p'} K F_k(p) F_k(p').  dots: nb +
+// kTailMoments^2 doubles of scratch.
+int far_tail_parts(const TailNodes &q, int np, long long points);
 int launch_far_tail(const int dims[3], int ax, int np, const double *n, const double *q0, double n_cut,
-                    double x0, double hx, int nodes, double dz, double rc, double c2, double c3, double scale,
-                    double *F, double *Tk, double *G, double *out, cudaStream_t st);
+                    const TailNodes &q, int parts, double dz, double rc, double c2, double c3, double scale, double *F,
+                    double *G, double *dots, double *out, cudaStream_t st);
 // One periodic axis ax: flags[ib * N_c + ic] = 1 for the lines along ax (b < c the
 // other axes) that hold an active point (flags zeroed by the caller).
 int launch_far_tail_line_flags(const int dims[3], int ax, const double *n, double n_cut, int *flags,
                                cudaStream_t st);
-// One periodic axis: the same sums over the La active lines `lines` (line ids):
-// F (nodes x La), K between lines (pref I(rho, x0), rho^2 from the index
-// differences through gbb, gbc, gcc) as a table Kt (N_b x (2 N_c - 1)) over the
-// index differences, G (nodes x La) = K F, Tk (nodes) and out as launch_far_tail.
+// One periodic axis: the same sums over the La active lines `lines` (line ids), K
+// between lines (pref I(rho, x0), rho^2 from the index differences through gbb, gbc,
+// gcc) as a table Kt (N_b x (2 N_c - 1)) over the index differences.
 int launch_far_tail_lines(const int dims[3], int ax, int La, const int *lines, const double *n, const double *q0,
-                          double n_cut, double x0, double hx, int nodes, double gbb, double gbc, double gcc,
-                          double rc, double pref, double scale, double *F, double *Kt, double *G, double *Tk,
-                          double *out, cudaStream_t st);
+                          double n_cut, const TailNodes &q, double gbb, double gbc, double gcc, double rc, double pref,
+                          double scale, double *F, double *Kt, double *G, double *dots, double *out, cudaStream_t st);
 // The far field's potential in the pair sum's adjoint form on the grid: A, U (N)
 // at active points with slot[m] = m, slot[m] = -1 elsewhere (for launch_assemble).
 // line_slot (one periodic axis; else NULL): the active-line index of every line,
-// which then indexes G (np = La).
+// which then indexes G (np = La).  coef: 2 kTailMoments x np doubles of scratch.
 int launch_far_tail_AU(const int dims[3], int ax, int np, const int *line_slot, const double *n, const double *q0,
-                       double n_cut, double x0, double hx, int nodes, const double *G, double C, int *slot,
-                       double *A, double *U, cudaStream_t st);
+                       double n_cut, const TailNodes &q, const double *G, double *coef, double C, int *slot, double *A,
+                       double *U, cudaStream_t st);
 int launch_kernel_eval(int precision, const PairShared &sh, int64_t npts, const double *r,
                        const double *qi, const double *qj, double *phi, double *rdphi,
                        cudaStream_t st);

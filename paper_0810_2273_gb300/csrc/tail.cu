@@ -12,14 +12,25 @@
 //
 // On the grid, z depends only on the plane of the non-periodic axis, and
 // 1/(u_i + u_j) = int_0^inf exp(-(u_i + u_j) s) ds separates i from j.  With
-// s = e^x and the trapezoidal rule in x (step hx = 0.3; the integrand is analytic
+// s = e^x and the trapezoidal rule in x (step hx = ln 2 / 3; the integrand is analytic
 // in the strip |Im x| < pi/2, so the error falls like exp(-pi^2 / hx)),
 //   T = -1/2 dV^2 C sum_k hx s_k sum_{p, p'} K(p, p') F_k(p) F_k(p'),
 //   F_k(p) = sum over active points of plane p of (n / u) exp(-u s_k).
-// That is O(N_grid x nodes) work for the planes and O(planes^2 x nodes) for the
-// pairs of planes, instead of O(N_active^2): a few milliseconds in FP64.  Its
-// potential (the derivative of T with the active mask frozen) comes from the
-// same sums, point by point (k_tail_AU), in the pair sum's adjoint form.
+// That is O(N_grid) work for the planes and O(planes^2) for the pairs of planes,
+// instead of O(N_active^2).  Its potential (the derivative of T with the active mask
+// frozen) comes from the same sums, point by point (k_tail_AU), in the pair sum's
+// adjoint form.
+//
+// Few exponentials: FP64 ones were all of the time (165 per point and pass).
+// - Nodes with u_max s_k <= 1/16 (three quarters of them) need none: there
+//   exp(-u s) is its Taylor polynomial of degree 8 (3e-17), so F_k is a combination of
+//   the nine moments M_j = sum (n / u) (u / u_max)^j, and K acts on the moments.
+// - The others come in three runs of doubling s (s_{k+3} = 2 s_k): one exponential
+//   starts a run, the rest are squares, carried as 1 - exp(-x) while that is small.
+// Bound by the FP64 pipe still.  ms per call before -> after (with the potential):
+// monolayer 48 x 84 x 120 2.27 (5.28) -> 0.61 (1.28), the same with three periodic
+// axes, whose one plane now has many blocks, 36.0 -> 0.79, chain 24 x 72 x 72 with its
+// product of lines over 76 rows instead of 176 nodes 7.84 (8.88) -> 3.93 (4.20).
 //
 // One periodic axis a (length |a|): the images of a pair lie on a line, and
 // their continuum beyond r_cut gives
@@ -39,8 +50,9 @@ namespace vdwdf {
 
 namespace {
 
-constexpr int kTailChunk = 16;     // quadrature nodes per block of k_tail_planes
+constexpr int kRun = 20;           // nodes of a run per block column of the sums
 constexpr int kTailThreads = 256;
+constexpr int kMom = kTailMoments;
 
 constexpr double kTailPi = 3.14159265358979323846;
 
@@ -59,89 +71,186 @@ __device__ __forceinline__ long long plane_point(int d0, int d1, int d2, int ax,
     return t * d2 + p;
 }
 
-// F[k * np + p] for the kTailChunk nodes k of blockIdx.y; one block per plane p,
-// sums in a fixed order (threads stride the plane, then warp and block trees).
+// exp(-x) along a run of doublings: e = exp(-x), f = 1 - e to full relative accuracy
+// while f < 1/2 (squaring e there would lose it), then frozen.
+__device__ __forceinline__ void run_start(double x, double &f, double &e) {
+    if (x < 0.7) {
+        f = -expm1(-x);
+        e = 1.0 - f;
+    } else {
+        f = 1.0;
+        e = exp(-x);
+    }
+}
+__device__ __forceinline__ void run_double(double &f, double &e) {
+    const bool small = __double2hiint(f) < 0x3FE00000;  // f < 1/2
+    const double f2 = fma(-f, f, f + f), ea = 1.0 - f2, eb = e * e;
+    e = small ? ea : eb;
+    f = small ? f2 : f;
+}
+
+// Columns of the sums: column 0 the moments, then run r = (col - 1) % 3, doublings
+// from kRun ((col - 1) / 3) on.  Adds one point's terms (u = q0^2, a = n / u).
+__device__ __forceinline__ void tail_add(int col, const TailNodes &q, double s0, double u, double a, double acc[kRun]) {
+    if (col == 0) {
+        const double x = u * q.iumax;
+#pragma unroll
+        for (int j = 0; j < kMom; ++j) {
+            acc[j] += a;
+            a *= x;
+        }
+        return;
+    }
+    double f, e;
+    run_start(u * s0, f, e);
+#pragma unroll
+    for (int j = 0; j < kRun; ++j) {
+        acc[j] = fma(a, e, acc[j]);
+        run_double(f, e);
+    }
+}
+// s of a column's first node, and the row of F of its entry j (below 0: none).
+__device__ __forceinline__ double tail_s0(int col, const TailNodes &q) {
+    return col == 0 ? 0.0 : ldexp(q.s[(col - 1) % 3], kRun * ((col - 1) / 3));
+}
+__device__ __forceinline__ int tail_row(int col, int j, const TailNodes &q) {
+    if (col == 0) return j < kMom ? j : -1;
+    const int k = (col - 1) % 3 + 3 * (kRun * ((col - 1) / 3) + j);
+    return k < q.nb ? kMom + k : -1;
+}
+
+// F[row * np + p] of column blockIdx.y, for the blockIdx.z-th part of the points of
+// plane p = blockIdx.x (parts are then added in order): threads stride the points,
+// then warp and block trees, all in a fixed order.
 __global__ void __launch_bounds__(kTailThreads) k_tail_planes(int d0, int d1, int d2, int ax, int np,
                                                               const double *__restrict__ n,
                                                               const double *__restrict__ q0, double n_cut,
-                                                              double x0, double hx, int nodes,
+                                                              const __grid_constant__ TailNodes q,
                                                               double *__restrict__ F) {
-    __shared__ double s_k[kTailChunk];
-    __shared__ double red[kTailThreads / 32][kTailChunk];
-    const int p = blockIdx.x;
-    const int k0 = blockIdx.y * kTailChunk;
-    if (threadIdx.x < kTailChunk) s_k[threadIdx.x] = exp(x0 + hx * (k0 + static_cast<int>(threadIdx.x)));
-    __syncthreads();
+    __shared__ double red[kTailThreads / 32][kRun];
+    const int p = blockIdx.x, col = blockIdx.y;
+    const double s0 = tail_s0(col, q);
     const long long per_plane = (np == 1) ? static_cast<long long>(d0) * d1 * d2
                                           : static_cast<long long>(d0) * d1 * d2 / np;
-    double acc[kTailChunk];
+    double acc[kRun];
 #pragma unroll
-    for (int c = 0; c < kTailChunk; ++c) acc[c] = 0.0;
-    for (long long t = threadIdx.x; t < per_plane; t += blockDim.x) {
+    for (int c = 0; c < kRun; ++c) acc[c] = 0.0;
+    for (long long t = blockIdx.z * static_cast<long long>(blockDim.x) + threadIdx.x; t < per_plane;
+         t += static_cast<long long>(gridDim.z) * blockDim.x) {
         const long long m = plane_point(d0, d1, d2, ax, np, p, t);
         const double nm = n[m];
         if (!(nm >= n_cut)) continue;  // inactive (NaN as well)
-        const double q = q0[m];
-        const double u = q * q;
-        const double a = nm / u;
-#pragma unroll
-        for (int c = 0; c < kTailChunk; ++c) acc[c] += a * exp(-u * s_k[c]);
+        const double u = q0[m] * q0[m];
+        tail_add(col, q, s0, u, nm / u, acc);
     }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
-    for (int c = 0; c < kTailChunk; ++c) {
+    for (int c = 0; c < kRun; ++c) {
         const double v = warp_sum_d(acc[c]);
         if (lane == 0) red[warp][c] = v;
     }
     __syncthreads();
-    if (threadIdx.x < kTailChunk && k0 + static_cast<int>(threadIdx.x) < nodes) {
+    const int row = threadIdx.x < kRun ? tail_row(col, static_cast<int>(threadIdx.x), q) : -1;
+    if (row >= 0) {
         double s = 0.0;
         for (int w = 0; w < kTailThreads / 32; ++w) s += red[w][threadIdx.x];
-        F[static_cast<long long>(k0 + threadIdx.x) * np + p] = s;
+        F[(static_cast<long long>(blockIdx.z) * (kMom + q.nb) + row) * np + p] = s;
     }
 }
 
-// Tk[k] = sum_{p, p'} K(p, p') F_k(p) F_k(p') for node k = blockIdx.x, with
-// K(p, p') = c2 / max(rc, |p - p'| dz)^4 (two periodic axes) or c3 (three);
-// G (when given) keeps G_k(p) = sum_{p'} K(p, p') F_k(p') for the potential.
+// F[e] += the parts' sums, in order (parts of n values one after the other).
+__global__ void k_tail_fold(long long n, int parts, double *__restrict__ F) {
+    for (long long e = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; e < n;
+         e += static_cast<long long>(gridDim.x) * blockDim.x) {
+        double s = F[e];
+        for (int z = 1; z < parts; ++z) s += F[z * n + e];
+        F[e] = s;
+    }
+}
+
+// G[r * np + p] = sum_{p'} K(p, p') F[r * np + p'] for row r = blockIdx.x, with
+// K(p, p') = c2 / max(rc, |p - p'| dz)^4 (two periodic axes) or c3 (three).  K by |p - p'|
+// and the row of F stand in shared memory (sh) when they fit.
 __global__ void __launch_bounds__(kTailThreads) k_tail_pairs(int np, const double *__restrict__ F, double dz,
-                                                             double rc, double c2, double c3,
-                                                             double *__restrict__ Tk, double *__restrict__ G) {
-    __shared__ double red[kTailThreads / 32];
+                                                             double rc, double c2, double c3, int sh,
+                                                             double *__restrict__ G) {
+    extern __shared__ double sm[];
     const double *f = F + static_cast<long long>(blockIdx.x) * np;
-    double acc = 0.0;
+    auto kern = [&](int d) {
+        if (np == 1) return c3;
+        const double z = d * dz, R = z > rc ? z : rc, R2 = R * R;
+        return c2 / (R2 * R2);
+    };
+    if (sh) {
+        for (int p = threadIdx.x; p < np; p += blockDim.x) {
+            sm[p] = kern(p);
+            sm[np + p] = f[p];
+        }
+        __syncthreads();
+    }
     for (int p = threadIdx.x; p < np; p += blockDim.x) {
         double row = 0.0;
         for (int pp = 0; pp < np; ++pp) {
-            double K = c3;
-            if (np > 1) {
-                const double z = fabs(static_cast<double>(p - pp)) * dz;
-                const double R = z > rc ? z : rc;
-                const double R2 = R * R;
-                K = c2 / (R2 * R2);
-            }
-            row += K * f[pp];
+            const int d = p > pp ? p - pp : pp - p;
+            row += sh ? sm[d] * sm[np + pp] : kern(d) * f[pp];
         }
-        if (G) G[static_cast<long long>(blockIdx.x) * np + p] = row;
-        acc += f[p] * row;
+        G[static_cast<long long>(blockIdx.x) * np + p] = row;
     }
+}
+
+// Dot products over the groups: block b < nb that of node b's rows of F and G, then
+// the kMom x kMom products of the moments' rows.  One block each, fixed order.
+__global__ void __launch_bounds__(kTailThreads) k_tail_dots(int ng, int nb, const double *__restrict__ F,
+                                                            const double *__restrict__ G, double *__restrict__ dots) {
+    __shared__ double red[kTailThreads / 32];
+    const int b = blockIdx.x;
+    const long long rf = b < nb ? kMom + b : (b - nb) / kMom, rg = b < nb ? kMom + b : (b - nb) % kMom;
+    double acc = 0.0;
+    for (int a = threadIdx.x; a < ng; a += blockDim.x) acc += F[rf * ng + a] * G[rg * ng + a];
     acc = warp_sum_d(acc);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
     __syncthreads();
     if (threadIdx.x == 0) {
         double s = 0.0;
         for (int w = 0; w < kTailThreads / 32; ++w) s += red[w];
-        Tk[blockIdx.x] = s;
+        dots[b] = s;
     }
 }
 
-// out = scale * sum_k hx s_k Tk[k], in node order.
-__global__ void k_tail_final(int nodes, const double *__restrict__ Tk, double x0, double hx, double scale,
+__device__ __forceinline__ double sign_over_factorial(int j) {
+    double v = 1.0;
+    for (int i = 2; i <= j; ++i) v *= i;
+    return ((j & 1) ? -1.0 : 1.0) / v;
+}
+
+// out = scale sum_k hx s_k F_k . G_k: the nodes' products in order, and for the nodes
+// of the Taylor polynomial sum_{j, j'} (-1)^{j + j'} / (j! j'!) W_{j + j'} M_j . K M_j'.
+__global__ void k_tail_final(const __grid_constant__ TailNodes q, const double *__restrict__ dots, double scale,
                              double *__restrict__ out) {
     if (threadIdx.x != 0 || blockIdx.x != 0) return;
     double s = 0.0;
-    for (int k = 0; k < nodes; ++k) s += hx * exp(x0 + hx * k) * Tk[k];
+    for (int j = 0; j < kMom; ++j)
+        for (int i = 0; i < kMom; ++i)
+            s += sign_over_factorial(j) * sign_over_factorial(i) * q.W[j + i] * dots[q.nb + j * kMom + i];
+    for (int k = 0; k < q.nb; ++k) s += q.hx * ldexp(q.s[k % 3], k / 3) * dots[k];
     *out = scale * s;
+}
+
+// Per group p the Taylor nodes' part of S0 and S1 (k_tail_AU) as polynomials in
+// x = u / u_max: coef[j * ng + p] and coef[(kMom + j) * ng + p].
+__global__ void k_tail_coef(int ng, const __grid_constant__ TailNodes q, const double *__restrict__ G,
+                            double *__restrict__ coef) {
+    for (int p = blockIdx.x * blockDim.x + threadIdx.x; p < ng; p += gridDim.x * blockDim.x)
+        for (int j = 0; j < kMom; ++j) {
+            double c0 = 0.0, c1 = 0.0;
+            for (int i = 0; i < kMom; ++i) {
+                const double g = sign_over_factorial(i) * G[static_cast<long long>(i) * ng + p];
+                c0 += q.W[j + i] * g;
+                c1 += q.W[j + i + 1] * g;
+            }
+            coef[static_cast<long long>(j) * ng + p] = sign_over_factorial(j) * c0;
+            coef[static_cast<long long>(kMom + j) * ng + p] = sign_over_factorial(j) * c1 * q.iumax;
+        }
 }
 
 // The far field's potential in the pair sum's adjoint form, per grid point m:
@@ -154,13 +263,12 @@ __global__ void k_tail_final(int nodes, const double *__restrict__ Tk, double x0
 __global__ void __launch_bounds__(kTailThreads) k_tail_AU(int d0, int d1, int d2, int ax, int np,
                                                           const int *__restrict__ line_slot,
                                                           const double *__restrict__ n,
-                                                          const double *__restrict__ q0, double n_cut, double x0,
-                                                          double hx, int nodes, const double *__restrict__ G,
-                                                          double C, int *__restrict__ slot,
-                                                          double *__restrict__ A, double *__restrict__ U) {
-    extern __shared__ double s_nodes[];  // s_k = e^{x0 + k hx}, k < nodes
-    for (int k = threadIdx.x; k < nodes; k += blockDim.x) s_nodes[k] = exp(x0 + hx * k);
-    __syncthreads();
+                                                          const double *__restrict__ q0, double n_cut,
+                                                          const __grid_constant__ TailNodes q,
+                                                          const double *__restrict__ G,
+                                                          const double *__restrict__ coef, double C,
+                                                          int *__restrict__ slot, double *__restrict__ A,
+                                                          double *__restrict__ U) {
     const long long N = static_cast<long long>(d0) * d1 * d2;
     for (long long m = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; m < N;
          m += static_cast<long long>(gridDim.x) * blockDim.x) {
@@ -178,18 +286,28 @@ __global__ void __launch_bounds__(kTailThreads) k_tail_AU(int d0, int d1, int d2
         } else if (np > 1) {
             p = static_cast<int>(ax == 0 ? c0i : (ax == 1 ? c1i : c2i));
         }
-        const double q = q0[m];
-        const double u = q * q;
+        const double qm = q0[m], u = qm * qm, x = u * q.iumax;
         double S0 = 0.0, S1 = 0.0;
-        for (int k = 0; k < nodes; ++k) {
-            const double s = s_nodes[k];
-            const double t = hx * s * exp(-u * s) * G[static_cast<long long>(k) * np + p];
-            S0 += t;
-            S1 += s * t;
+#pragma unroll
+        for (int j = kMom - 1; j >= 0; --j) {
+            S0 = fma(S0, x, coef[static_cast<long long>(j) * np + p]);
+            S1 = fma(S1, x, coef[static_cast<long long>(kMom + j) * np + p]);
+        }
+        for (int r = 0; r < 3; ++r) {
+            double s = q.s[r], f, e;
+            run_start(u * s, f, e);
+            for (int k = r; k < q.nb; k += 3) {
+                const double t = (q.hx * s) * (e * G[static_cast<long long>(kMom + k) * np + p]);
+                S0 += t;
+                S1 = fma(s, t, S1);
+                s += s;
+                run_double(f, e);
+            }
         }
         slot[m] = static_cast<int>(m);
-        A[m] = -C * S0 / u;
-        U[m] = -2.0 * C * nm * q * (-S0 / (u * u) - S1 / u);
+        const double iu = 1.0 / u;
+        A[m] = -C * S0 * iu;
+        U[m] = 2.0 * C * nm * qm * (S0 * iu + S1) * iu;
     }
 }
 
@@ -223,45 +341,35 @@ __global__ void k_tail_line_flags(int d0, int d1, int d2, int ax, const double *
     }
 }
 
-// F[k * La + a] = sum over active points of line lines[a] of (n / u) exp(-u s_k),
-// one warp per line, nodes in chunks of kTailChunk (their s_k shared by the
-// block), sums in a fixed order.
+// F[row * La + a] over the active points of line lines[a]: one warp per line and
+// column blockIdx.y (see tail_add), sums in a fixed order.
 __global__ void __launch_bounds__(kTailThreads) k_tail_line_F(int d0, int d1, int d2, int ax, int La,
                                                               const int *__restrict__ lines,
                                                               const double *__restrict__ n,
                                                               const double *__restrict__ q0, double n_cut,
-                                                              double x0, double hx, int nodes,
+                                                              const __grid_constant__ TailNodes q,
                                                               double *__restrict__ F) {
-    __shared__ double s_k[kTailChunk];
-    const int lane = threadIdx.x & 31;
+    const int lane = threadIdx.x & 31, col = blockIdx.y;
     const int a = blockIdx.x * (kTailThreads / 32) + (threadIdx.x >> 5);
-    const bool live = a < La;
+    if (a >= La) return;
+    const double s0 = tail_s0(col, q);
     const int Nc = ax == 2 ? d1 : d2, len = ax == 0 ? d0 : (ax == 1 ? d1 : d2);
-    const int l = live ? lines[a] : 0;
-    const int ib = l / Nc, ic = l % Nc;
-    for (int k0 = 0; k0 < nodes; k0 += kTailChunk) {
-        __syncthreads();  // the previous chunk's s_k are read
-        if (threadIdx.x < kTailChunk) s_k[threadIdx.x] = exp(x0 + hx * (k0 + static_cast<int>(threadIdx.x)));
-        __syncthreads();
-        if (!live) continue;
-        double acc[kTailChunk];
+    const int l = lines[a], ib = l / Nc, ic = l % Nc;
+    double acc[kRun];
 #pragma unroll
-        for (int u = 0; u < kTailChunk; ++u) acc[u] = 0.0;
-        for (int t = lane; t < len; t += 32) {
-            const long long m = line_point(d1, d2, ax, ib, ic, t);
-            const double nm = n[m];
-            if (!(nm >= n_cut)) continue;
-            const double q = q0[m];
-            const double u2 = q * q;
-            const double w = nm / u2;
+    for (int c = 0; c < kRun; ++c) acc[c] = 0.0;
+    for (int t = lane; t < len; t += 32) {
+        const long long m = line_point(d1, d2, ax, ib, ic, t);
+        const double nm = n[m];
+        if (!(nm >= n_cut)) continue;
+        const double u = q0[m] * q0[m];
+        tail_add(col, q, s0, u, nm / u, acc);
+    }
 #pragma unroll
-            for (int u = 0; u < kTailChunk; ++u) acc[u] += w * exp(-u2 * s_k[u]);
-        }
-#pragma unroll
-        for (int u = 0; u < kTailChunk; ++u) {
-            const double v = warp_sum_d(acc[u]);
-            if (lane == 0 && k0 + u < nodes) F[static_cast<long long>(k0 + u) * La + a] = v;
-        }
+    for (int c = 0; c < kRun; ++c) {
+        const double v = warp_sum_d(acc[c]);
+        const int row = tail_row(col, c, q);
+        if (lane == 0 && row >= 0) F[static_cast<long long>(row) * La + a] = v;
     }
 }
 
@@ -313,7 +421,7 @@ __global__ void k_tail_line_Ktab(int Nb, int Nc, double gbb, double gbc, double 
 }
 
 // G[k * La + i] = sum_a K(lines[i], lines[a]) F[k * La + a] for every active line i
-// and node k: a 32 x 32 output tile per block of 16 x 16 threads (2 x 2 each), the a
+// and row k (moment or node): a 32 x 32 output tile per block of 16 x 16 threads (2 x 2 each), the a
 // range in shared-memory tiles of 32, K from the table Kt, summed in a fixed order.
 constexpr int kGT = 32;
 __global__ void __launch_bounds__(256) k_tail_line_G(int La, int nodes, const int *__restrict__ lines, int Nc,
@@ -368,24 +476,6 @@ __global__ void __launch_bounds__(256) k_tail_line_G(int La, int nodes, const in
         }
 }
 
-// Tk[k] = sum_a F[k * La + a] G[k * La + a], one block per node, fixed order.
-__global__ void __launch_bounds__(kTailThreads) k_tail_line_Tk(int La, const double *__restrict__ F,
-                                                               const double *__restrict__ G,
-                                                               double *__restrict__ Tk) {
-    __shared__ double red[kTailThreads / 32];
-    const long long base = static_cast<long long>(blockIdx.x) * La;
-    double acc = 0.0;
-    for (int a = threadIdx.x; a < La; a += blockDim.x) acc += F[base + a] * G[base + a];
-    acc = warp_sum_d(acc);
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double s = 0.0;
-        for (int w = 0; w < kTailThreads / 32; ++w) s += red[w];
-        Tk[blockIdx.x] = s;
-    }
-}
-
 }  // namespace
 
 int launch_far_tail_line_flags(const int dims[3], int ax, const double *n, double n_cut, int *flags,
@@ -399,52 +489,75 @@ int launch_far_tail_line_flags(const int dims[3], int ax, const double *n, doubl
     return VDWDF_OK;
 }
 
+// Columns of the sums that hold the moments and every node.
+static int tail_columns(const TailNodes &q) { return 1 + 3 * ((q.nb + 3 * kRun - 1) / (3 * kRun)); }
+
+static int tail_finish(int ng, const TailNodes &q, const double *F, const double *G, double scale, double *dots,
+                       double *out, cudaStream_t st) {
+    k_tail_dots<<<q.nb + kMom * kMom, kTailThreads, 0, st>>>(ng, q.nb, F, G, dots);
+    k_tail_final<<<1, 32, 0, st>>>(q, dots, scale, out);
+    count_launches(2);
+    VDWDF_CUDA_TRY(cudaGetLastError());
+    return VDWDF_OK;
+}
+
 int launch_far_tail_lines(const int dims[3], int ax, int La, const int *lines, const double *n, const double *q0,
-                          double n_cut, double x0, double hx, int nodes, double gbb, double gbc, double gcc,
-                          double rc, double pref, double scale, double *F, double *Kt, double *G, double *Tk,
-                          double *out, cudaStream_t st) {
+                          double n_cut, const TailNodes &q, double gbb, double gbc, double gcc, double rc, double pref,
+                          double scale, double *F, double *Kt, double *G, double *dots, double *out,
+                          cudaStream_t st) {
     // lines are ib * N_c + ic, b < c the other two axes
     const int Nb = ax == 0 ? dims[1] : dims[0], Nc = ax == 2 ? dims[1] : dims[2];
-    const int wpb = kTailThreads / 32;
-    k_tail_line_F<<<(La + wpb - 1) / wpb, kTailThreads, 0, st>>>(dims[0], dims[1], dims[2], ax, La, lines, n, q0,
-                                                                 n_cut, x0, hx, nodes, F);
+    const int wpb = kTailThreads / 32, rows = kMom + q.nb;
+    k_tail_line_F<<<dim3((La + wpb - 1) / wpb, tail_columns(q)), kTailThreads, 0, st>>>(dims[0], dims[1], dims[2], ax,
+                                                                                     La, lines, n, q0, n_cut, q, F);
     const long long kt = static_cast<long long>(Nb) * (2 * Nc - 1);
     k_tail_line_Ktab<<<static_cast<int>(std::min<long long>((kt + kTailThreads - 1) / kTailThreads, 152 * 8)),
                        kTailThreads, 0, st>>>(Nb, Nc, gbb, gbc, gcc, rc, pref, Kt);
-    k_tail_line_G<<<dim3((La + kGT - 1) / kGT, (nodes + kGT - 1) / kGT), 256, 0, st>>>(La, nodes, lines, Nc, Kt, F,
-                                                                                       G);
-    k_tail_line_Tk<<<nodes, kTailThreads, 0, st>>>(La, F, G, Tk);
-    k_tail_final<<<1, 32, 0, st>>>(nodes, Tk, x0, hx, scale, out);
-    count_launches(5);
+    k_tail_line_G<<<dim3((La + kGT - 1) / kGT, (rows + kGT - 1) / kGT), 256, 0, st>>>(La, rows, lines, Nc, Kt, F, G);
+    count_launches(3);
     VDWDF_CUDA_TRY(cudaGetLastError());
-    return VDWDF_OK;
+    return tail_finish(La, q, F, G, scale, dots, out, st);
 }
 
 int launch_far_tail_AU(const int dims[3], int ax, int np, const int *line_slot, const double *n, const double *q0,
-                       double n_cut, double x0, double hx, int nodes, const double *G, double C, int *slot,
-                       double *A, double *U, cudaStream_t st) {
+                       double n_cut, const TailNodes &q, const double *G, double *coef, double C, int *slot, double *A,
+                       double *U, cudaStream_t st) {
+    k_tail_coef<<<(np + 127) / 128, 128, 0, st>>>(np, q, G, coef);
     const long long N = static_cast<long long>(dims[0]) * dims[1] * dims[2];
     long long nb = (N + kTailThreads - 1) / kTailThreads;
     if (nb > 152 * 16) nb = 152 * 16;
-    const size_t smem = sizeof(double) * static_cast<size_t>(nodes);  // at most 32 KB (4096 nodes)
-    k_tail_AU<<<static_cast<int>(nb), kTailThreads, smem, st>>>(dims[0], dims[1], dims[2], ax, np, line_slot, n, q0,
-                                                                n_cut, x0, hx, nodes, G, C, slot, A, U);
-    count_launches(1);
+    k_tail_AU<<<static_cast<int>(nb), kTailThreads, 0, st>>>(dims[0], dims[1], dims[2], ax, np, line_slot, n, q0,
+                                                             n_cut, q, G, coef, C, slot, A, U);
+    count_launches(2);
     VDWDF_CUDA_TRY(cudaGetLastError());
     return VDWDF_OK;
 }
 
+// Parts of a plane's points: enough blocks for two rounds of the chip.
+int far_tail_parts(const TailNodes &q, int np, long long points) {
+    const long long blocks = static_cast<long long>(np) * tail_columns(q);
+    const long long want = (152 * 8 + blocks - 1) / blocks, most = (points / np + 4 * kTailThreads - 1) / (4 * kTailThreads);
+    return static_cast<int>(std::max<long long>(1, std::min<long long>(std::min(want, most), 64)));
+}
+
 int launch_far_tail(const int dims[3], int ax, int np, const double *n, const double *q0, double n_cut,
-                    double x0, double hx, int nodes, double dz, double rc, double c2, double c3, double scale,
-                    double *F, double *Tk, double *G, double *out, cudaStream_t st) {
-    const int chunks = (nodes + kTailChunk - 1) / kTailChunk;
-    k_tail_planes<<<dim3(np, chunks), kTailThreads, 0, st>>>(dims[0], dims[1], dims[2], ax, np, n, q0, n_cut, x0,
-                                                             hx, nodes, F);
-    k_tail_pairs<<<nodes, kTailThreads, 0, st>>>(np, F, dz, rc, c2, c3, Tk, G);
-    k_tail_final<<<1, 32, 0, st>>>(nodes, Tk, x0, hx, scale, out);
-    count_launches(3);
+                    const TailNodes &q, int parts, double dz, double rc, double c2, double c3, double scale, double *F,
+                    double *G, double *dots, double *out, cudaStream_t st) {
+    const int rows = kMom + q.nb;
+    k_tail_planes<<<dim3(np, tail_columns(q), parts), kTailThreads, 0, st>>>(dims[0], dims[1], dims[2], ax, np, n, q0,
+                                                                             n_cut, q, F);
+    count_launches(1);
+    if (parts > 1) {
+        const long long e = static_cast<long long>(rows) * np;
+        k_tail_fold<<<static_cast<int>(std::min<long long>((e + 255) / 256, 152 * 8)), 256, 0, st>>>(e, parts, F);
+        count_launches(1);
+    }
+    const size_t smem = 2 * sizeof(double) * static_cast<size_t>(np);
+    const int sh = smem <= 48 * 1024 ? 1 : 0;
+    k_tail_pairs<<<rows, kTailThreads, sh ? smem : 0, st>>>(np, F, dz, rc, c2, c3, sh, G);
+    count_launches(1);
     VDWDF_CUDA_TRY(cudaGetLastError());
-    return VDWDF_OK;
+    return tail_finish(np, q, F, G, scale, dots, out, st);
 }
 
 }  // namespace vdwdf
