@@ -25,6 +25,78 @@ constexpr int kBrick = 4;               // 4 x 4 x 4 grid bricks order the activ
 constexpr int kMaxSmemBytes = 232448;   // 227 KiB opt-in shared memory per block (cc 10.x)
 constexpr int kMaxInst = 24;            // instances per pair-kernel launch
 
+#ifdef __CUDACC__
+// 1/x to the last bit or so (x positive and normal, 1/x normal): a 20-bit seed and two
+// Newton steps, four FP64 operations instead of a division's nine and its special cases.
+__device__ __forceinline__ double rcp_newton(double x) {
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    y = fma(y, fma(-x, y, 1.0), y);
+    return fma(y, fma(-x, y, 1.0), y);
+}
+// x^(-1/2), likewise.
+__device__ __forceinline__ double rsqrt_newton(double x) {
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    y = fma(0.5 * y, fma(-x * y, y, 1.0), y);
+    return fma(0.5 * y, fma(-x * y, y, 1.0), y);
+}
+// x^(-1/3), likewise: an FP32 seed of the part in [1, 8), one step of third order
+// (y (1 + e/3 + 2 e^2/9), e = 1 - x y^3), the power of eight back by the exponent.
+__device__ __forceinline__ double rcbrt_newton(double x) {
+    const int hi = __double2hiint(x), q = ((hi >> 20) - 1023 + 1200) / 3 - 400;
+    const double m = __hiloint2double(hi - 3 * q * (1 << 20), __double2loint(x));
+    const double y = static_cast<double>(exp2f(-0.33333333f * __log2f(static_cast<float>(m))));
+    const double e = fma(-m * y, y * y, 1.0);
+    const double z = fma(y * e, fma(e, 2.0 / 9.0, 1.0 / 3.0), y);
+    return __hiloint2double(__double2hiint(z) - q * (1 << 20), __double2loint(z));
+}
+// log(1 + a/b) for a >= 0, b > 0 (normal): with s = a + b and the power of two nearest
+// s/b taken out, 2 atanh of (s 2^-k - b)/(s 2^-k + b), which is at most 0.2 (the
+// series' remainder is 1e-17 of it there); without a power, a itself stands for s - b.
+__device__ __forceinline__ double log1p_ratio(double a, double b) {
+    const double s = a + b;
+    const int hi = __double2hiint(s), k = (hi - __double2hiint(b) + 0x80000) >> 20;
+    const double sk = __hiloint2double(hi - (k << 20), __double2loint(s));
+    const double w = (k ? sk - b : a) * rcp_newton(sk + b), x = w * w;
+    double p = 1.0 / 21.0;
+    p = fma(p, x, 1.0 / 19.0);
+    p = fma(p, x, 1.0 / 17.0);
+    p = fma(p, x, 1.0 / 15.0);
+    p = fma(p, x, 1.0 / 13.0);
+    p = fma(p, x, 1.0 / 11.0);
+    p = fma(p, x, 1.0 / 9.0);
+    p = fma(p, x, 1.0 / 7.0);
+    p = fma(p, x, 1.0 / 5.0);
+    p = fma(p, x, 1.0 / 3.0);
+    return fma(static_cast<double>(k), 0.69314718055994530942, fma(p * x, w + w, w + w));
+}
+// exp(x) - 1 for 0 <= x < 30: the power of two taken out, the Taylor polynomial of
+// degree 14 of the rest (|r| <= ln 2 / 2, remainder 1e-19).
+__device__ __forceinline__ double expm1_taylor(double x) {
+    const int k = static_cast<int>(static_cast<float>(x) * 1.44269504f + 0.5f);
+    // ln 2 in two parts, the first of 32 bits, whose small multiples are exact (Cody and
+    // Waite's reduction)
+    const double kd = k, r = fma(-kd, 0x1.a39ef35793c76p-33, fma(-kd, 0x1.62e42fee00000p-1, x));
+    double p = 1.0 / 87178291200.0;
+    p = fma(p, r, 1.0 / 6227020800.0);
+    p = fma(p, r, 1.0 / 479001600.0);
+    p = fma(p, r, 1.0 / 39916800.0);
+    p = fma(p, r, 1.0 / 3628800.0);
+    p = fma(p, r, 1.0 / 362880.0);
+    p = fma(p, r, 1.0 / 40320.0);
+    p = fma(p, r, 1.0 / 5040.0);
+    p = fma(p, r, 1.0 / 720.0);
+    p = fma(p, r, 1.0 / 120.0);
+    p = fma(p, r, 1.0 / 24.0);
+    p = fma(p, r, 1.0 / 6.0);
+    p = fma(p, r, 0.5);
+    p = fma(p * r, r, r);
+    const double t = __hiloint2double((1023 + k) << 20, 0);  // 2^k
+    return fma(t, p, t - 1.0);
+}
+#endif
+
 // Device-side counters of one instance (zeroed before use).
 struct Stats {
     double E_pair;             // sum over ordered pairs of n_i n_j phi (self term included)

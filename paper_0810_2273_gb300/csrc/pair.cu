@@ -1030,15 +1030,6 @@ __device__ __forceinline__ void pair_items_f32(const PairLaunch &pl, unsigned ch
 // FP64
 // ---------------------------------------------------------------------------
 
-// 1/x to the last bit or so (x positive and normal): a 20-bit seed and two Newton
-// steps, four FP64 operations instead of a division's nine and its special cases.
-__device__ __forceinline__ double rcp_newton(double x) {
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    y = fma(y, fma(-x, y, 1.0), y);
-    return fma(y, fma(-x, y, 1.0), y);
-}
-
 // The cell of a coordinate x in [0, n): floor(x) in k and x - k, from the low word of x
 // shifted by 1.5 2^52 (rounded down).  False for x outside and for NaN.
 __device__ __forceinline__ bool cell_of(double x, int n, int &k, double &t) {

@@ -37,6 +37,44 @@ __device__ __forceinline__ void pw92_eps(double rs, double &e, double &dedrs) {
     dedrs = -2.0 * A * a1 * lg - pre * dden / (den * (den + 1.0));
 }
 
+// The local quantities of a point of density n: k_F, 1/k_F, 1/n, r_s, eps_c and
+// d eps_c/d r_s.  All of these follow from z = (3 pi^2 n)^(-1/3): k_F = 3 pi^2 n z^2,
+// 1/n = 3 pi^2 z^3, r_s = (9 pi/4)^(1/3) z.  The FP64 pipe bounds the callers, and
+// library cube roots, logarithms and divisions were two thirds of their operations
+// (128 x 112 x 200 slab: semilocal energies 1.54 -> 0.85 ms, q0 with its partials 0.93
+// -> 0.54 ms).  Densities whose powers could leave the normal range take those.
+struct LocalPoint {
+    double kF, ikF, in, rs, ec, dec;
+};
+constexpr double kPlainMin = 1e-40, kPlainMax = 1e40;
+
+__device__ __forceinline__ LocalPoint local_point(double n) {
+    LocalPoint p;
+    if (!(n > kPlainMin && n < kPlainMax)) {
+        p.kF = cbrt(3.0 * kPi * kPi * n);
+        p.ikF = 1.0 / p.kF;
+        p.in = 1.0 / n;
+        p.rs = cbrt(3.0 / (4.0 * kPi * n));
+        pw92_eps(p.rs, p.ec, p.dec);
+        return p;
+    }
+    const double A = 0.031091, a1 = 0.21370;
+    const double b1 = 7.5957, b2 = 3.5876, b3 = 1.6382, b4 = 0.49294;
+    const double t = 3.0 * kPi * kPi, x = t * n, z = rcbrt_newton(x), z2 = z * z;
+    p.kF = x * z2;
+    p.ikF = z;
+    p.in = t * (z2 * z);
+    p.rs = 1.9191582926775128 * z;  // (9 pi / 4)^(1/3)
+    const double irs = rsqrt_newton(p.rs), srs = p.rs * irs;
+    const double den = fma(srs, fma(2.0 * A * b3, p.rs, 2.0 * A * b1), p.rs * fma(2.0 * A * b4, p.rs, 2.0 * A * b2));
+    const double lg = log1p_ratio(1.0, den);
+    const double dden = fma(A * b1, irs, 2.0 * A * b2) + fma(3.0 * A * b3, srs, 4.0 * A * b4 * p.rs);
+    const double pre = fma(-2.0 * A * a1, p.rs, -2.0 * A);
+    p.ec = pre * lg;
+    p.dec = fma(-2.0 * A * a1, lg, -pre * dden * rcp_newton(den * (den + 1.0)));
+    return p;
+}
+
 __device__ __forceinline__ int wrap(int i, int n) {
     i %= n;
     return i < 0 ? i + n : i;
@@ -99,22 +137,17 @@ __global__ void k_grad_q0(int n0, int n1, int n2, const AxisMap am,
             }
             continue;
         }
-        const double kF = cbrt(3.0 * kPi * kPi * nn);
-        const double g2 = gx * gx + gy * gy + gz * gz;
-        const double rs = cbrt(3.0 / (4.0 * kPi * nn));
-        double ec, decdrs;
-        pw92_eps(rs, ec, decdrs);
-        const double inv_kFn2 = 1.0 / (kF * nn * nn);
-        q0[m] = kF - (Zab / 36.0) * g2 * inv_kFn2 - (4.0 * kPi / 3.0) * ec;
-        if (qn) {
-            const double dec_dn = decdrs * (-rs / (3.0 * nn));
-            qn[m] = kF / (3.0 * nn) + (7.0 * Zab / 108.0) * g2 * inv_kFn2 / nn - (4.0 * kPi / 3.0) * dec_dn;
-        }
+        const LocalPoint p = local_point(nn);
+        // g/n keeps 1/n^2 out: G = |g/n|^2
+        const double hx = gx * p.in, hy = gy * p.in, hz = gz * p.in;
+        const double Gz = fma(hx, hx, fma(hy, hy, hz * hz)) * p.ikF;
+        q0[m] = p.kF - (Zab / 36.0) * Gz - (4.0 * kPi / 3.0) * p.ec;
+        if (qn) qn[m] = p.in * fma(4.0 * kPi / 9.0, p.dec * p.rs, fma(7.0 * Zab / 108.0, Gz, p.kF * (1.0 / 3.0)));
         if (qg) {
-            const double f = -(Zab / 18.0) * inv_kFn2;
-            qg[m] = f * gx;
-            qg[N + m] = f * gy;
-            qg[2 * N + m] = f * gz;
+            const double f = -(Zab / 18.0) * (p.ikF * p.in);
+            qg[m] = f * hx;
+            qg[N + m] = f * hy;
+            qg[2 * N + m] = f * hz;
         }
     }
 }
@@ -303,15 +336,11 @@ __global__ void k_tiles_cart(const float4 *__restrict__ p32, const Stats *stats,
 //   t = |g|/(2 k_s n), k_s = (4 k_F/pi)^(1/2), A = (beta/gamma)/(exp(-eps_c/gamma) - 1),
 //   beta = 0.06672455060314922, gamma = (1 - ln 2)/pi^2.
 // Each block sums n eps over its points (fixed grid-stride order, fixed tree);
-// a second kernel adds the block sums in order, so the result is reproducible.
+// a second kernel adds the block sums in a fixed order, so the result is reproducible.
 // ---------------------------------------------------------------------------
 constexpr int kSemiBlocks = 608;  // 4 per SM on 152 SMs
 constexpr int kSemiThreads = 256;
 constexpr int kSemiVals = 6;      // five energies and the point count
-
-__device__ __forceinline__ double gga_fx(double s2, double kappa, double mu) {
-    return 1.0 + kappa - kappa / (1.0 + mu * s2 / kappa);
-}
 
 __global__ void __launch_bounds__(kSemiThreads) k_semilocal(int n0, int n1, int n2, const AxisMap am,
                                                             const double *__restrict__ n,
@@ -319,7 +348,7 @@ __global__ void __launch_bounds__(kSemiThreads) k_semilocal(int n0, int n1, int 
                                                             double *__restrict__ part) {
     const long long N = static_cast<long long>(n0) * n1 * n2;
     const double beta = 0.06672455060314922;
-    const double gamma = (1.0 - log(2.0)) / (kPi * kPi);
+    const double gamma = (1.0 - 0.69314718055994530942) / (kPi * kPi);
     const double mu = beta * kPi * kPi / 3.0;
     double acc[kSemiVals] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
     for (long long m = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x; m < N;
@@ -328,23 +357,26 @@ __global__ void __launch_bounds__(kSemiThreads) k_semilocal(int n0, int n1, int 
         if (!(nn > 0.0)) continue;
         double gx, gy, gz;
         grad_at(m, n0, n1, n2, am, n, gin, gx, gy, gz);
-        const double g2 = gx * gx + gy * gy + gz * gz;
-        const double kF = cbrt(3.0 * kPi * kPi * nn);
-        const double rs = cbrt(3.0 / (4.0 * kPi * nn));
-        double ec, decdrs;
-        pw92_eps(rs, ec, decdrs);
-        const double ex = -3.0 * kF / (4.0 * kPi);
-        const double s2 = g2 / (4.0 * kF * kF * nn * nn);
-        const double ks2 = 4.0 * kF / kPi;
-        const double t2 = g2 / (4.0 * ks2 * nn * nn);
-        const double A = (beta / gamma) / expm1(-ec / gamma);
-        const double At2 = A * t2;
-        const double H = gamma * log1p((beta / gamma) * t2 * (1.0 + At2) / (1.0 + At2 + At2 * At2));
-        acc[0] += nn * ex;
-        acc[1] += nn * ec;
-        acc[2] += nn * ex * gga_fx(s2, 0.804, mu);
-        acc[3] += nn * (ec + H);
-        acc[4] += nn * ex * gga_fx(s2, 1.245, mu);
+        const LocalPoint p = local_point(nn);
+        const double hx = gx * p.in, hy = gy * p.in, hz = gz * p.in;
+        double G = fma(hx, hx, fma(hy, hy, hz * hz));  // |g/n|^2
+        // (F_x and H have reached their limits long before; NaN stays)
+        G = G > 1e100 ? 1e100 : G;
+        const double ex = -3.0 / (4.0 * kPi) * p.kF;
+        const double s2 = 0.25 * G * p.ikF * p.ikF, t2 = (kPi / 16.0) * G * p.ikF;
+        // F_x = 1 + kappa mu s^2/(kappa + mu s^2), both kappas from one reciprocal
+        const double k1 = 0.804, k2 = 1.245, y = mu * s2, e1 = k1 + y, e2 = k2 + y, ie = y * rcp_newton(e1 * e2);
+        // A = (beta/gamma)/E, E = expm1(-eps_c/gamma): the argument of H's logarithm is
+        // v E (E + v)/(E^2 + E v + v^2), v = (beta/gamma) t^2
+        const double E = expm1_taylor(p.ec * (-1.0 / gamma)), v = (beta / gamma) * t2;
+        const double num = v * E * (E + v), dn = fma(E, E, v * (E + v));
+        // (a vanishing eps_c or gradient could make the denominator vanish; H is 0 then)
+        const double H = dn > 1e-280 ? gamma * log1p_ratio(num, dn) : (dn == dn ? 0.0 : dn);
+        acc[0] = fma(nn, ex, acc[0]);
+        acc[1] = fma(nn, p.ec, acc[1]);
+        acc[2] = fma(nn * ex, fma(k1 * ie, e2, 1.0), acc[2]);
+        acc[3] = fma(nn, p.ec + H, acc[3]);
+        acc[4] = fma(nn * ex, fma(k2 * ie, e1, 1.0), acc[4]);
         acc[5] += 1.0;
     }
     __shared__ double red[kSemiVals][kSemiThreads / 32];
@@ -364,12 +396,14 @@ __global__ void __launch_bounds__(kSemiThreads) k_semilocal(int n0, int n1, int 
     }
 }
 
+// Warp w adds value w of the blocks: lanes stride them, then a warp tree.
 __global__ void k_semilocal_sum(const double *__restrict__ part, int nblocks, double *__restrict__ out) {
-    if (threadIdx.x < kSemiVals) {
-        double v = 0.0;
-        for (int b = 0; b < nblocks; ++b) v += part[static_cast<long long>(b) * kSemiVals + threadIdx.x];
-        out[threadIdx.x] = v;
-    }
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    double v = 0.0;
+    for (int b = lane; b < nblocks; b += 32) v += part[static_cast<long long>(b) * kSemiVals + w];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if (lane == 0) out[w] = v;
 }
 
 // The finite-difference gradient alone (Cartesian, 3 planes of N).
@@ -393,7 +427,7 @@ int semilocal_scratch_doubles() { return (kSemiBlocks + 1) * kSemiVals; }
 int launch_semilocal(const int dims[3], const AxisMap &am, const double *n, const double *grad_in,
                      double *scratch, cudaStream_t st) {
     k_semilocal<<<kSemiBlocks, kSemiThreads, 0, st>>>(dims[0], dims[1], dims[2], am, n, grad_in, scratch);
-    k_semilocal_sum<<<1, 32, 0, st>>>(scratch, kSemiBlocks, scratch + kSemiBlocks * kSemiVals);
+    k_semilocal_sum<<<1, 32 * kSemiVals, 0, st>>>(scratch, kSemiBlocks, scratch + kSemiBlocks * kSemiVals);
     count_launches(2);
     VDWDF_CUDA_TRY(cudaGetLastError());
     return VDWDF_OK;
