@@ -640,7 +640,12 @@ __device__ __forceinline__ float dist2(float dx, float dy, float dz, const PairP
 // What lies off the band costs code as well as loads: with one more copy of the step
 // (for tiles whose images all stay inside) the instruction cache no longer held
 // the loop, and the slab took 119 ms.
-template <int MODE, int NT, bool SKEW>
+//
+// OPEN: cells without images or a cutoff.  One image, no masks, tests or counts but in
+// ragged and diagonal tiles.  The general instance against it, ms per pass: molecule
+// 48^3 E + v 48.5 -> 42.2, E 36.0 -> 30.6, binding curve 69.8 -> 58.0, Kr dimer
+// 24 x 18 x 18 E 0.221 -> 0.191.
+template <int MODE, int NT, bool SKEW, bool OPEN>
 __device__ __forceinline__ void pair_items_f32(const PairLaunch &pl, unsigned char *smem_raw,
                                                const unsigned int *s_prefix, const int *s_C,
                                                unsigned int n_items, unsigned int stride, const Table<float> &tb) {
@@ -709,6 +714,10 @@ __device__ __forceinline__ void pair_items_f32(const PairLaunch &pl, unsigned ch
             const int jb = J * kTile;
             const int jl0 = max(0, j_first - jb), jl1 = min(kTile, j_end - jb);
             const bool mine = lane >= jl0 && lane < jl1;
+            const bool diag = (J >> 1) == I;
+            const bool special = diag || ni_act < 64;
+            bool staged = false;
+            int n_cand = 1;
             float ilo[3], ihi[3], jl[3], jh[3];
             {
                 const float4 a0 = __ldg(pp.blo + T0), a1 = __ldg(pp.blo + T1), b0 = __ldg(pp.bhi + T0),
@@ -743,12 +752,18 @@ __device__ __forceinline__ void pair_items_f32(const PairLaunch &pl, unsigned ch
                     nm[a] = max(0, mhi - mlo[a] + 1);
                 }
             }
-            const int n_cand = nm[0] * nm[1] * nm[2];
-            const bool diag = (J >> 1) == I;
-            const bool special = diag || ni_act < 64;
-            bool staged = false;
-            // candidate images in chunks of 32, one per lane
+            if (!OPEN) n_cand = nm[0] * nm[1] * nm[2];
+            // candidate images in chunks of 32, one per lane (an open cell has the one at 0)
             for (int c0 = 0; c0 < n_cand; c0 += 32) {
+                unsigned bal = 1u, jm = mine ? 1u : 0u, jf = 0u;
+                if constexpr (OPEN) {
+                    __syncwarp();  // earlier reads of p, n, js are done
+                    if (mine) {
+                        sw.p[lane] = __ldg(pp.p32 + jb + lane);
+                        sw.n[lane] = __ldg(pp.n32 + jb + lane);
+                    }
+                    __syncwarp();
+                } else {
                 const int t = c0 + lane;
                 bool ok = false;
                 int mm[3] = {0, 0, 0};
@@ -762,7 +777,7 @@ __device__ __forceinline__ void pair_items_f32(const PairLaunch &pl, unsigned ch
                     else
                         ok = !use_cut || box_gap2(ilo, ihi, jl, jh, mm, pp.dims, cull) <= rc2_box;
                 }
-                const unsigned bal = __ballot_sync(0xffffffffu, ok);
+                bal = __ballot_sync(0xffffffffu, ok);
                 if (bal == 0u) continue;
                 __syncwarp();  // earlier reads of img, p, n, js are done
                 if (ok)
@@ -780,7 +795,7 @@ __device__ __forceinline__ void pair_items_f32(const PairLaunch &pl, unsigned ch
                 const int nimg = __popc(bal);
                 // this lane's j point: images that bring the i box within the cutoff (jm), and
                 // those that keep all of it inside (jf; none in ragged or diagonal tiles)
-                unsigned jm = 0u, jf = 0u;
+                jm = 0u;
                 if (mine) {
                     const float4 pj = sw.p[lane];
                     for (int b = 0; b < nimg; ++b) {
@@ -816,16 +831,24 @@ __device__ __forceinline__ void pair_items_f32(const PairLaunch &pl, unsigned ch
                     }
                     if (special) jf = 0u;
                 }
+                }
                 float2 a_acc = f2(0.0f), u_acc = f2(0.0f);
                 float2 cwt = f2(0.0f);
-                unsigned jset = __ballot_sync(0xffffffffu, jm != 0u);
-                while (jset != 0u) {
-                    const int jj = __ffs(jset) - 1;
-                    jset &= jset - 1u;
-                    const unsigned m = __shfl_sync(0xffffffffu, jm, jj);
-                    const unsigned mf = __shfl_sync(0xffffffffu, jf, jj);
-                    evals += static_cast<unsigned>(__popc(m));
-                    cnt_full += static_cast<unsigned>(__popc(mf));
+                if (OPEN) {
+                    evals += static_cast<unsigned>(jl1 - jl0);
+                    if (!special) cnt_full += static_cast<unsigned>(jl1 - jl0);
+                }
+                unsigned jset = OPEN ? 0u : __ballot_sync(0xffffffffu, jm != 0u);
+                for (int jo = jl0; OPEN ? jo < jl1 : jset != 0u; ++jo) {
+                    const int jj = OPEN ? jo : __ffs(jset) - 1;
+                    unsigned m = 1u, mf = special ? 0u : 1u;
+                    if (!OPEN) {
+                        jset &= jset - 1u;
+                        m = __shfl_sync(0xffffffffu, jm, jj);
+                        mf = __shfl_sync(0xffffffffu, jf, jj);
+                        evals += static_cast<unsigned>(__popc(m));
+                        cnt_full += static_cast<unsigned>(__popc(mf));
+                    }
                     const float4 pj = sw.p[jj];
                     const float nj = sw.n[jj];
                     Delta2 dp;
@@ -838,13 +861,17 @@ __device__ __forceinline__ void pair_items_f32(const PairLaunch &pl, unsigned ch
                     float2 Srpt = f2(0.0f), Spu = f2(0.0f);
                     unsigned mfar = 0u;  // images with some pair past the table
                     float2 cw = f2(0.0f);  // partly inside images: those that count, per half
-                    for (unsigned mr = m; mr != 0u;) {
-                        const unsigned bit = mr & (0u - mr);
-                        const float4 sft = sw.img[__ffs(mr) - 1];
-                        mr ^= bit;
+                    unsigned mr = m;
+                    do {
+                        const unsigned bit = OPEN ? 1u : mr & (0u - mr);
                         // integers: every sum is exact
-                        const float2 dx = add2(xi, f2(sft.x - pj.x)), dy = add2(yi, f2(sft.y - pj.y)),
-                                     dz = add2(zi, f2(sft.z - pj.z));
+                        float2 dx = sub2(xi, f2(pj.x)), dy = sub2(yi, f2(pj.y)), dz = sub2(zi, f2(pj.z));
+                        if (!OPEN) {
+                            const float4 sft = sw.img[__ffs(mr) - 1];
+                            mr ^= bit;
+                            dx = add2(xi, f2(sft.x - pj.x)), dy = add2(yi, f2(sft.y - pj.y)),
+                            dz = add2(zi, f2(sft.z - pj.z));
+                        }
                         float2 r2 = mul2(H2, mul2(dz, dz));
                         r2 = fma2(H1, mul2(dy, dy), r2);
                         r2 = fma2(H0, mul2(dx, dx), r2);
@@ -857,9 +884,9 @@ __device__ __forceinline__ void pair_items_f32(const PairLaunch &pl, unsigned ch
                         float2 tD = mul2(rr, dp.sqcD);
                         float2 w = f2(1.0f);  // 0 in a half that does not count
                         uint32_t l0a = c0a, l1a = c1a;
-                        if ((mf & bit) == 0u) {
+                        if (OPEN ? special : (mf & bit) == 0u) {
                             bool in0 = true, in1 = true;
-                            if (use_cut) {
+                            if (!OPEN && use_cut) {
                                 in0 = !beyond<SKEW>(r2.x, dx.x, dy.x, dz.x, cut);
                                 in1 = !beyond<SKEW>(r2.y, dx.y, dy.y, dz.y, cut);
                             }
@@ -912,12 +939,12 @@ __device__ __forceinline__ void pair_items_f32(const PairLaunch &pl, unsigned ch
                             if (__any_sync(0xffffffffu, (w.x != 0.0f && !(tex && on0)) || (w.y != 0.0f && !(tex && on1))))
                                 mfar |= bit;
                         }
-                    }
+                    } while (!OPEN && mr != 0u);
                     // ordered pairs: two for every inside evaluation (once for i, once for j), less
                     // the one of a self-image taken off above
                     cwt = add2(cwt, cw);
                     if (cl0 || cl1) {
-                        const float nf = static_cast<float>(__popc(mf));
+                        const float nf = OPEN ? (special ? 0.0f : 1.0f) : static_cast<float>(__popc(mf));
                         nclamp += 2u * static_cast<unsigned>((cl0 ? nf + cw.x : 0.0f) + (cl1 ? nf + cw.y : 0.0f));
                     }
                     if (POT) {
@@ -929,8 +956,8 @@ __device__ __forceinline__ void pair_items_f32(const PairLaunch &pl, unsigned ch
                     // the halves past the table (once more from the geometry, so that the loop above
                     // keeps nothing for them in registers)
                     while (mfar != 0u) {
-                        const float4 sft = sw.img[__ffs(mfar) - 1];
-                        const bool part = (mf & mfar & (0u - mfar)) == 0u;
+                        const float4 sft = OPEN ? make_float4(0.f, 0.f, 0.f, 0.f) : sw.img[__ffs(mfar) - 1];
+                        const bool part = OPEN ? special : (mf & mfar & (0u - mfar)) == 0u;
                         mfar &= mfar - 1u;
 #pragma unroll
                         for (int h = 0; h < 2; ++h) {
@@ -942,7 +969,7 @@ __device__ __forceinline__ void pair_items_f32(const PairLaunch &pl, unsigned ch
                             const bool on = tD >= 0.0f && tD <= K.tDmax;
                             if ((tex && on) || !(r2 > 0.0f)) continue;
                             if (part && (!(h ? act1 : act0) || (diag && jb + jj < (h ? i1 : i0)) ||
-                                         (use_cut && beyond<SKEW>(r2, dx, dy, dz, cut))))
+                                         (!OPEN && use_cut && beyond<SKEW>(r2, dx, dy, dz, cut))))
                                 continue;
                             float phi, rd = 0.0f, rd2 = 0.0f;
                             if (on) {  // (only with a table too large for a texture)
@@ -1226,7 +1253,7 @@ struct Warp64 {
 // whose warps hold a lane past the table), the pipe 88 % busy as before.  ms per pass,
 // 24 x 42 x 60 monolayer E + v 453 -> 274 and E 242 -> 143, hexagonal 20 x 20 x 50
 // 93 -> 47, slab 32 x 28 x 50 185 -> 138, open dimer 31 x 23 x 19 E 16.7 -> 14.0.
-template <typename R, int MODE, int NT, bool SKEW>
+template <typename R, int MODE, int NT, bool SKEW, bool OPEN = false>
 __global__ void __launch_bounds__(NT, 1) k_pair(const __grid_constant__ PairLaunch pl) {
     constexpr bool POT = (MODE == 1);
     constexpr int NW = NT / 32;
@@ -1264,7 +1291,7 @@ __global__ void __launch_bounds__(NT, 1) k_pair(const __grid_constant__ PairLaun
     const unsigned int stride = max(1u, sh.item_stride);
     const unsigned int n_items = min((s_prefix[pl.ninst] + stride - 1u) / stride, sh.item_limit);
     if constexpr (sizeof(R) == 4) {
-        pair_items_f32<MODE, NT, SKEW>(pl, smem_raw, s_prefix, s_C, n_items, stride, tb);
+        pair_items_f32<MODE, NT, SKEW, OPEN>(pl, smem_raw, s_prefix, s_C, n_items, stride, tb);
         return;
     } else {
     const Consts<double> &K = sh.k64;
@@ -1736,9 +1763,9 @@ __global__ void k_kernel_eval(const PairShared sh, int64_t npts, const double *r
     }
 }
 
-template <typename R, int MODE, int NT, bool SKEW>
+template <typename R, int MODE, int NT, bool SKEW, bool OPEN = false>
 int launch_one(const PairLaunch &pl, int nctas, size_t smem, cudaStream_t st) {
-    auto kern = k_pair<R, MODE, NT, SKEW>;
+    auto kern = k_pair<R, MODE, NT, SKEW, OPEN>;
     VDWDF_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         static_cast<int>(smem)));
     kern<<<nctas, NT, smem, st>>>(pl);
@@ -1750,9 +1777,20 @@ int launch_one(const PairLaunch &pl, int nctas, size_t smem, cudaStream_t st) {
 template <typename R, int MODE>
 int launch_nt(int threads, bool skew, const PairLaunch &pl, int nctas, size_t smem, cudaStream_t st) {
     if constexpr (sizeof(R) == 4)
-        if (threads == 640)
+        if (threads == 640) {
+            // cells with neither images nor a cutoff: the instance without either
+            // (13-17 % faster, see pair_items_f32)
+            bool open = true;
+            for (int k = 0; k < pl.ninst; ++k) {
+                const PairParams &p = pl.inst[k];
+                open = open && !p.use_cut && p.M[0] == 0 && p.M[1] == 0 && p.M[2] == 0;
+            }
+            if (open)
+                return skew ? launch_one<R, MODE, 640, true, true>(pl, nctas, smem, st)
+                            : launch_one<R, MODE, 640, false, true>(pl, nctas, smem, st);
             return skew ? launch_one<R, MODE, 640, true>(pl, nctas, smem, st)
                         : launch_one<R, MODE, 640, false>(pl, nctas, smem, st);
+        }
     if (skew) {
         if (threads == 448) return launch_one<R, MODE, 448, true>(pl, nctas, smem, st);
         return threads == 384 ? launch_one<R, MODE, 384, true>(pl, nctas, smem, st)

@@ -155,3 +155,15 @@ def test_orthogonal_beside_skewed_in_a_batch(V, gtable, precision, tol):
     for n, g, p, e in zip(ns, geo, per, E):
         one, _ = V.energy(n, g, p, 1e-6, 6.0, gtable, precision)
         assert abs(e - one) <= tol * abs(one)
+
+
+@pytest.mark.parametrize("active", [1, 33, 64, 65, 129])
+def test_skewed_open_cell(V, oracle_mod, gtable, oracle_spline, active):
+    """A skewed cell without images or a cutoff (its own instance of the FP32 kernel), and
+    the same with a cutoff beyond every distance (the general one)."""
+    cell = CELLS["skew"][0]
+    n = _density((9, 8, 7), cell, active)
+    s = np.sort(n, axis=None)[::-1]
+    n_cut = 0.5 * (s[active - 1] + s[active])
+    for r_cut in (0.0, 60.0):
+        _check(V, oracle_mod, gtable, oracle_spline, n, cell, (False, False, False), n_cut, r_cut)
