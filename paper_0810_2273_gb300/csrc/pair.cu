@@ -476,6 +476,12 @@ __device__ __forceinline__ void count_item(Stats *s, unsigned long long cnt, uns
 // pipe otherwise idles.  Random stencils cost 3.1 SM clocks per shared load (bank
 // conflicts) and 22 per gather, side by side: 49.7 clocks for sixteen loads, 42.0
 // for twelve and one gather (448 threads on an SM, measured on random cells).
+// Energy mode has less arithmetic to hide the loads behind: there the shared pipe is
+// 89 % busy, and one of the two halves takes a second block from the texture, the same
+// rows' first and second columns, which levels the two pipes (20 loads and 3 gathers
+// for both halves).  Energies: dimer of 41^2 x 75 points 0.193 -> 0.183 ms, 36 x 63 x 90
+// monolayer 78.0 -> 75.6 ms, 36 x 36 x 100 hexagonal cell 49.1 -> 47.2 ms.  With the
+// potential nothing is won: issue bounds it.
 __device__ __forceinline__ float4 tex_block(unsigned long long tex, float x, float y) {
     return tex2Dgather<float4>(static_cast<cudaTextureObject_t>(tex), x, y, 0);
 }
@@ -512,13 +518,18 @@ __device__ __forceinline__ void band_pair2(unsigned long long tex, uint32_t rs, 
                                            uint32_t a1, float2 fl, const float2 wd[4], const float2 dwd[4],
                                            float2 &p, float2 &pt, float2 &pu) {
     const float4 g0 = tex_block(tex, fl.x, fk.x + 3.0f), g1 = tex_block(tex, fl.y, fk.y + 3.0f);
+    float4 h0;  // (energy mode) the first half's first and second columns
+    if (!POT) h0 = tex_block(tex, fl.x - 2.0f, fk.x + 3.0f);
     float2 r[4], dr[4];
 #pragma unroll
     for (int m = 0; m < 4; ++m) {
         float2 c[4];
 #pragma unroll
         for (int n = 0; n < 4; ++n) {
-            if (m < 2 || n < 2)
+            if (!POT && m >= 2 && n < 2)
+                c[n] = make_float2(m == 2 ? (n == 0 ? h0.w : h0.z) : (n == 0 ? h0.x : h0.y),
+                                   lds32(a1 + m * rs + 4u * n));
+            else if (m < 2 || n < 2)
                 c[n] = make_float2(lds32(a0 + m * rs + 4u * n), lds32(a1 + m * rs + 4u * n));
             else if (m == 2)
                 c[n] = n == 2 ? make_float2(g0.w, g1.w) : make_float2(g0.z, g1.z);
