@@ -142,6 +142,17 @@ __device__ __forceinline__ void bdw2(float2 t, float2 d[4]) {
     d[2] = mul2(s, fma2(s, f2(-9.0f), f2(12.0f)));
     d[3] = mul2(mul2(t, t), f2(3.0f));
 }
+// The last three weights and derivative weights (not times 6), for sums over the
+// differences from the first coefficient.
+__device__ __forceinline__ void bw_diff2(float2 t, float2 w[4], float2 d[4]) {
+    const float2 t2 = mul2(t, t), h = f2(0.5f);
+    w[1] = fma2(t2, fma2(h, t, f2(-1.0f)), f2(2.0f / 3.0f));
+    w[2] = fma2(t, fma2(t, fma2(t, f2(-0.5f), h), h), f2(1.0f / 6.0f));
+    w[3] = mul2(mul2(t, f2(1.0f / 6.0f)), t2);
+    d[1] = mul2(t, fma2(t, f2(1.5f), f2(-2.0f)));
+    d[2] = fma2(t, fma2(t, f2(-1.5f), f2(1.0f)), h);
+    d[3] = mul2(t2, h);
+}
 
 // The delta-derivative weights sum to zero, so sum_n dwd[n] c[n] is taken as
 // sum_{n>=1} dwd[n] (c[n] - c[0]): neighbouring coefficients differ little and
@@ -246,7 +257,7 @@ __device__ __forceinline__ void delta_part(R qi, R qj, const Consts<R> &K, Delta
 struct Delta2 {
     float2 sqcD;          // (q_i + q_j) cD
     float2 b1, sb;        // r dphi/dd1 = a + b1 pu, r dphi/dd2 = a + (b1 - 2 sb) pu
-    float2 wd[4], dwd[4]; // dwd[0] is not used
+    float2 wd[4], dwd[4]; // E + v: bw_diff2's (no [0]), else bw2's
     float2 fl;            // the delta cells' third columns, l + 2, as texture coordinates
     uint32_t l0, l1;
 };
@@ -266,15 +277,20 @@ __device__ __forceinline__ void delta_part2(float2 qi, float qj, const Consts<fl
     d.l0 = b0 - 0x4B400000u;
     d.l1 = b1 - 0x4B400000u;
     d.fl = make_float2(f.x + 3.0f, f.y + 3.0f);
-    bw2(u, d.wd);
-    if (POT) bdw2(u, d.dwd);
+    if (POT)
+        bw_diff2(u, d.wd, d.dwd);
+    else
+        bw2(u, d.wd);
     if (cl0 || cl1) {
         // past the last node the weights continue linearly: + e w'(u), and the derivative
         // weights sum to zero
         float2 dw[4];
-        bdw2(u, dw);
+        if (POT)
+            dw[1] = d.dwd[1], dw[2] = d.dwd[2], dw[3] = d.dwd[3];
+        else
+            bdw2(u, dw);
         const float2 e = make_float2(cl0 ? fabsf(td0.x) - td.x : 0.0f, cl1 ? fabsf(td0.y) - td.y : 0.0f);
-        d.wd[0] = sub2(d.wd[0], mul2(e, add2(dw[1], add2(dw[2], dw[3]))));
+        if (!POT) d.wd[0] = sub2(d.wd[0], mul2(e, add2(dw[1], add2(dw[2], dw[3]))));
 #pragma unroll
         for (int n = 1; n < 4; ++n) d.wd[n] = fma2(e, dw[n], d.wd[n]);
     }
@@ -486,29 +502,44 @@ __device__ __forceinline__ float4 tex_block(unsigned long long tex, float x, flo
     return tex2Dgather<float4>(static_cast<cudaTextureObject_t>(tex), x, y, 0);
 }
 
-// One row of the stencil: row = sum_n wd[n] c[n], and with POT the delta derivative
-// from exact coefficient differences (see combine): fma(c0, -1, c_n) is c_n - c0 with
-// one rounding.
+// One row of the stencil: row = sum_n wd[n] c[n], with POT (weights that sum to one,
+// 1/6 of the others) from the differences c[n] - c[0], which the delta derivative needs
+// for its accuracy in any case (see combine).
 template <bool POT>
 __device__ __forceinline__ void row2(const float2 c[4], const float2 wd[4], const float2 dwd[4], float2 &row,
                                      float2 &drow) {
-    row = fma2(wd[3], c[3], fma2(wd[2], c[2], fma2(wd[1], c[1], mul2(wd[0], c[0]))));
-    if (POT)
-        drow = fma2(dwd[3], sub2(c[3], c[0]), fma2(dwd[2], sub2(c[2], c[0]), mul2(dwd[1], sub2(c[1], c[0]))));
+    if (POT) {
+        const float2 d1 = sub2(c[1], c[0]), d2 = sub2(c[2], c[0]), d3 = sub2(c[3], c[0]);
+        row = fma2(wd[3], d3, fma2(wd[2], d2, fma2(wd[1], d1, c[0])));
+        drow = fma2(dwd[3], d3, fma2(dwd[2], d2, mul2(dwd[1], d1)));
+    } else {
+        row = fma2(wd[3], c[3], fma2(wd[2], c[2], fma2(wd[1], c[1], mul2(wd[0], c[0]))));
+    }
 }
 
-// Six times the cubic B-spline through four neighbours r at offset t of their middle
-// cell, in powers of t, and (DER) a third of six times its t-derivative.  The
-// differences of neighbours stand in for the eight weight polynomials: as many
-// operations, but one constant instead of nine (each a register pair to fill).
-template <bool DER>
-__device__ __forceinline__ float2 spline2(const float2 r[4], float2 t, float2 t3, float2 &der) {
-    const float2 u0 = sub2(r[1], r[0]), u1 = sub2(r[2], r[1]), u2 = sub2(r[3], r[2]);
-    const float2 v = sub2(u1, u0), x = sub2(sub2(u2, u1), v), y = add2(u0, u1);
-    // 6 r1 + v + 3 t y + 3 t^2 v + t^3 x, and y + 2 t v + t^2 x
-    const float2 z = fma2(t, v, y);
-    if (DER) der = fma2(t, fma2(t, x, v), z);
-    return fma2(f2(3.0f), fma2(t, z, add2(r[1], r[1])), fma2(t3, x, v));
+// Six times the cubic B-spline of the rows r at offset t of their middle cell, and
+// (POT) a third of six times its t-derivative and six times the spline of dr.  With
+// three results the weights pay (25 operations a half against 28 from powers of t and
+// the differences of neighbours), with one the differences do (14 against 16).
+// E + v with these weights and with row2's differences, against neither: 36 x 63 x 90
+// monolayer 102.2 -> 100.2 ms.
+template <bool POT>
+__device__ __forceinline__ void rows2(const float2 r[4], const float2 dr[4], float2 t, float2 &p, float2 &pt,
+                                      float2 &pu) {
+    if (POT) {
+        const float2 s = sub2(f2(1.0f), t), t2 = mul2(t, t), s2 = mul2(s, s), w0 = mul2(s2, s), w3 = mul2(t2, t);
+        const float2 w1 = fma2(t2, fma2(t, f2(3.0f), f2(-6.0f)), f2(4.0f)),
+                     w2 = fma2(s2, fma2(s, f2(3.0f), f2(-6.0f)), f2(4.0f));
+        p = fma2(w3, r[3], fma2(w2, r[2], fma2(w1, r[1], mul2(w0, r[0]))));
+        pu = fma2(w3, dr[3], fma2(w2, dr[2], fma2(w1, dr[1], mul2(w0, dr[0]))));
+        const float2 c1 = fma2(add2(t, t), s, f2(1.0f));
+        pt = fma2(t2, sub2(r[3], r[2]), fma2(c1, sub2(r[2], r[1]), mul2(s2, sub2(r[1], r[0]))));
+    } else {
+        // 6 r1 + v + 3 t y + 3 t^2 v + t^3 x
+        const float2 u0 = sub2(r[1], r[0]), u1 = sub2(r[2], r[1]), u2 = sub2(r[3], r[2]);
+        const float2 v = sub2(u1, u0), x = sub2(sub2(u2, u1), v), y = add2(u0, u1), z = fma2(t, v, y);
+        p = fma2(f2(3.0f), fma2(t, z, add2(r[1], r[1])), fma2(mul2(mul2(t, t), t), x, v));
+    }
 }
 
 // Both halves in the resident band: t the offsets in their D cells (fk: the cells'
@@ -538,10 +569,7 @@ __device__ __forceinline__ void band_pair2(unsigned long long tex, uint32_t rs, 
         }
         row2<POT>(c, wd, dwd, r[m], dr[m]);
     }
-    const float2 t3 = mul2(mul2(t, t), t);
-    p = spline2<POT>(r, t, t3, pt);
-    float2 unused;
-    if (POT) pu = spline2<false>(dr, t, t3, unused);
+    rows2<POT>(r, dr, t, p, pt, pu);
 }
 
 // Rows k, k + 1 (y0 = k + 1) of one half's stencil: from the band where the half is in
@@ -583,10 +611,7 @@ __device__ __forceinline__ void table_pair2(unsigned long long tex, uint32_t rs,
         row2<POT>(ca, wd, dwd, r[2 * h], dr[2 * h]);
         row2<POT>(cb, wd, dwd, r[2 * h + 1], dr[2 * h + 1]);
     }
-    const float2 t3 = mul2(mul2(t, t), t);
-    p = spline2<POT>(r, t, t3, pt);
-    float2 unused;
-    if (POT) pu = spline2<false>(dr, t, t3, unused);
+    rows2<POT>(r, dr, t, p, pt, pu);
 }
 
 // Warp sums of two values: the total of v0 ends in lanes 0-15, that of v1 in lanes
@@ -661,11 +686,17 @@ __device__ __forceinline__ void pair_items_f32(const PairLaunch &pl, unsigned ch
                                                const unsigned int *s_prefix, const int *s_C,
                                                unsigned int n_items, unsigned int stride, const Table<float> &tb) {
     constexpr bool POT = (MODE == 1);
+    constexpr float kUnit = POT ? 6.0f : 1.0f;  // bw_diff2's weights lack this factor
     const int warp = threadIdx.x >> 5;
     int lane = threadIdx.x & 31;
     asm volatile("" : "+r"(lane));  // kept, not read from the special register again
     const bool hi = (lane & 16) != 0;
-    Warp32 &sw = reinterpret_cast<Warp32 *>(smem_raw)[warp];
+    // the warp's shared memory by an address that stays in a register: otherwise it is
+    // formed again from the thread index at each use (E + v: molecule 48^3 42.2 -> 40.5 ms,
+    // slab 48 x 42 x 75 51.4 -> 49.9, monolayer 36 x 63 x 90 102.2 -> 100.2)
+    uint32_t sw_addr = static_cast<uint32_t>(__cvta_generic_to_shared(reinterpret_cast<Warp32 *>(smem_raw) + warp));
+    asm volatile("" : "+r"(sw_addr));
+    Warp32 &sw = *reinterpret_cast<Warp32 *>(__cvta_shared_to_generic(sw_addr));
     const PairShared &sh = pl.sh;
     const Consts<float> &K = sh.k32;
     const unsigned long long tex = sh.tex32;
@@ -893,7 +924,7 @@ __device__ __forceinline__ void pair_items_f32(const PairLaunch &pl, unsigned ch
                         }
                         float2 rr = mul2(r2, make_float2(rsqrt_ftz(r2.x), rsqrt_ftz(r2.y)));
                         float2 tD = mul2(rr, dp.sqcD);
-                        float2 w = f2(1.0f);  // 0 in a half that does not count
+                        float2 w = f2(kUnit);  // 0 in a half that does not count
                         uint32_t l0a = c0a, l1a = c1a;
                         if (OPEN ? special : (mf & bit) == 0u) {
                             bool in0 = true, in1 = true;
@@ -910,8 +941,8 @@ __device__ __forceinline__ void pair_items_f32(const PairLaunch &pl, unsigned ch
                                 in1 = in1 && act1 && (!diag || jb + jj >= i1);
                                 cnt -= (in0 && diag && jb + jj == i0 ? 1u : 0u) + (in1 && diag && jb + jj == i1 ? 1u : 0u);
                             }
-                            w = make_float2(in0 ? 1.0f : 0.0f, in1 ? 1.0f : 0.0f);
-                            cw = add2(cw, w);
+                            w = make_float2(in0 ? kUnit : 0.0f, in1 ? kUnit : 0.0f);
+                            cw = add2(cw, make_float2(in0 ? 1.0f : 0.0f, in1 ? 1.0f : 0.0f));
                             // an idle half reads the band's first cell (one address for all)
                             if (!in0) tD.x = band_lo, l0a = tb.s;
                             if (!in1) tD.y = band_lo, l1a = tb.s;
@@ -942,8 +973,8 @@ __device__ __forceinline__ void pair_items_f32(const PairLaunch &pl, unsigned ch
                                                  dp.fl, dp.wd, dp.dwd, p, pt, pu);
                                 A2 = fma2(wt, p, A2);
                                 if (POT) {
-                                    Srpt = fma2(make_float2(wt.x == 0.0f ? 0.0f : rr.x, wt.y == 0.0f ? 0.0f : rr.y), pt,
-                                                Srpt);
+                                    Srpt = fma2(make_float2(wt.x == 0.0f ? 0.0f : kUnit * rr.x,
+                                                            wt.y == 0.0f ? 0.0f : kUnit * rr.y), pt, Srpt);
                                     Spu = fma2(wt, pu, Spu);
                                 }
                             }
@@ -959,7 +990,7 @@ __device__ __forceinline__ void pair_items_f32(const PairLaunch &pl, unsigned ch
                         nclamp += 2u * static_cast<unsigned>((cl0 ? nf + cw.x : 0.0f) + (cl1 ? nf + cw.y : 0.0f));
                     }
                     if (POT) {
-                        const float2 a = mul2(Srpt, f2(3.0f * K.cD));  // spline2 gives a third of the derivative
+                        const float2 a = mul2(Srpt, f2(3.0f * K.cD));  // rows2 gives a third of the derivative
                         const float2 u = fma2(Spu, dp.b1, a), v = mul2(Spu, dp.sb);
                         u_acc = fma2(f2(nj), u, u_acc);
                         V2 = sub2(sub2(u, v), v);
