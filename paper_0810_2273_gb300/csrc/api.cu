@@ -696,8 +696,9 @@ Launch choose_launch(int precision, bool pot, const vdwdf_tuning *tu, const vdwd
     Launch ln;
     const int S = t->nd + 2;
     // Default shape.  FP32 640: that kernel is bound by instruction issue, and 20 warps
-    // of 96 registers keep the schedulers 84 % busy (E + v on the 36 x 63 x 90 monolayer
-    // 102.7 ms against 111.9 with 16 warps of 128).  FP64 is bound by the FP64 pipe, and
+    // of 96 registers keep the schedulers 81 % busy (E + v on the 36 x 63 x 90 monolayer
+    // 102.7 ms against 111.9 with 16 warps of 128; energy with 24 warps of 80 within 1.5 %
+    // there, and 6 % slower on the Kr dimer).  FP64 is bound by the FP64 pipe, and
     // few warps are enough: E + v with 256 threads (384 on skewed cells) 274.5 ms on the
     // 24 x 42 x 60 monolayer against 281.7 with 512; energy 143.3 with 512 against 144.7.
     ln.threads = precision == VDWDF_FP32 ? 640 : (!pot ? 512 : (skew ? 384 : 256));

@@ -495,8 +495,8 @@ __device__ __forceinline__ void count_item(Stats *s, unsigned long long cnt, uns
 // Energy mode has less arithmetic to hide the loads behind: there the shared pipe is
 // 89 % busy, and one of the two halves takes a second block from the texture, the same
 // rows' first and second columns, which levels the two pipes (20 loads and 3 gathers
-// for both halves).  Energies: dimer of 41^2 x 75 points 0.193 -> 0.183 ms, 36 x 63 x 90
-// monolayer 78.0 -> 75.6 ms, 36 x 36 x 100 hexagonal cell 49.1 -> 47.2 ms.  With the
+// for both halves).  Energies: Kr dimer 24 x 18 x 18 0.193 -> 0.183 ms, 36 x 63 x 90
+// monolayer 78.0 -> 75.6 ms, 36 x 36 x 90 hexagonal cell 49.1 -> 47.2 ms.  With the
 // potential nothing is won: issue bounds it.
 __device__ __forceinline__ float4 tex_block(unsigned long long tex, float x, float y) {
     return tex2Dgather<float4>(static_cast<cudaTextureObject_t>(tex), x, y, 0);
@@ -666,19 +666,19 @@ __device__ __forceinline__ float dist2(float dx, float dy, float dz, const PairP
 // that keeps the whole i box inside the cutoff (most of them) needs no test, weight
 // or count per lane.
 //
-// Bound by instruction issue: 350 instructions a step (a j point's image against 64
-// i points), 217 of them FP32 arithmetic, with the schedulers 84 % busy and the
-// shared-memory pipe 68 % (36 x 63 x 90 monolayer, E + v).  The kernel before this
-// one (a lane's halves held two j points, 14 warps of 128 registers, packed
-// arithmetic) against this one, ms per pass, E + v / E:
-//   monolayer 36 x 63 x 90  123.0 / 99.7 -> 102.7 / 78.5   slab 48 x 42 x 75  63.2 / - -> 51.4 / 39.9
-//   hexagonal 36 x 36 x 90   74.4 / 62.6 ->  60.9 / 49.2   molecule 48^3      58.0 / - -> 48.2 / -
+// Bound by instruction issue: 334 instructions a step (a j point's image against 64
+// i points), 199 of them FP32 arithmetic, with the schedulers 81 % busy and the
+// shared-memory pipe 73 % (24 x 42 x 60 monolayer, E + v; energy 238 instructions, 73 %
+// and 79 %).  The kernel before this one (a lane's halves held two j points, 14 warps of
+// 128 registers, packed arithmetic) against this one, ms per pass, E + v / E:
+//   monolayer 36 x 63 x 90  123.0 / 99.7 -> 98.1 / 75.2    slab 48 x 42 x 75  63.2 / - -> 49.7 / -
+//   hexagonal 36 x 36 x 90      - / 62.6 ->    - / 46.9    molecule 48^3      58.0 / - -> 39.7 / 30.2
 // What lies off the band costs code as well as loads: with one more copy of the step
 // (for tiles whose images all stay inside) the instruction cache no longer held
 // the loop, and the slab took 119 ms.
 //
 // OPEN: cells without images or a cutoff.  One image, no masks, tests or counts but in
-// ragged and diagonal tiles.  The general instance against it, ms per pass: molecule
+// ragged and diagonal tiles.  The general instance against it when it came, ms per pass: molecule
 // 48^3 E + v 48.5 -> 42.2, E 36.0 -> 30.6, binding curve 69.8 -> 58.0, Kr dimer
 // 24 x 18 x 18 E 0.221 -> 0.191.
 template <int MODE, int NT, bool SKEW, bool OPEN>
@@ -1818,21 +1818,24 @@ int launch_one(const PairLaunch &pl, int nctas, size_t smem, cudaStream_t st) {
 
 template <typename R, int MODE>
 int launch_nt(int threads, bool skew, const PairLaunch &pl, int nctas, size_t smem, cudaStream_t st) {
-    if constexpr (sizeof(R) == 4)
-        if (threads == 640) {
-            // cells with neither images nor a cutoff: the instance without either
-            // (13-17 % faster, see pair_items_f32)
-            bool open = true;
-            for (int k = 0; k < pl.ninst; ++k) {
-                const PairParams &p = pl.inst[k];
-                open = open && !p.use_cut && p.M[0] == 0 && p.M[1] == 0 && p.M[2] == 0;
-            }
-            if (open)
-                return skew ? launch_one<R, MODE, 640, true, true>(pl, nctas, smem, st)
-                            : launch_one<R, MODE, 640, false, true>(pl, nctas, smem, st);
+    if constexpr (sizeof(R) == 4) {
+        // cells with neither images nor a cutoff: the instance without either (13-17 %
+        // faster, see pair_items_f32), at the default's threads and, so that a tuned shape
+        // can have it as well, at 512 on orthogonal cells (binding curve with the shape tuned
+        // on the batch 72.6 -> 57.7 ms, default 54.8)
+        bool open = threads == 640 || (threads == 512 && !skew);
+        for (int k = 0; k < pl.ninst; ++k) {
+            const PairParams &p = pl.inst[k];
+            open = open && !p.use_cut && p.M[0] == 0 && p.M[1] == 0 && p.M[2] == 0;
+        }
+        if (open && threads == 512) return launch_one<R, MODE, 512, false, true>(pl, nctas, smem, st);
+        if (open)
+            return skew ? launch_one<R, MODE, 640, true, true>(pl, nctas, smem, st)
+                        : launch_one<R, MODE, 640, false, true>(pl, nctas, smem, st);
+        if (threads == 640)
             return skew ? launch_one<R, MODE, 640, true>(pl, nctas, smem, st)
                         : launch_one<R, MODE, 640, false>(pl, nctas, smem, st);
-        }
+    }
     if (skew) {
         if (threads == 448) return launch_one<R, MODE, 448, true>(pl, nctas, smem, st);
         return threads == 384 ? launch_one<R, MODE, 384, true>(pl, nctas, smem, st)

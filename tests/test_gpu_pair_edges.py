@@ -167,3 +167,14 @@ def test_skewed_open_cell(V, oracle_mod, gtable, oracle_spline, active):
     n_cut = 0.5 * (s[active - 1] + s[active])
     for r_cut in (0.0, 60.0):
         _check(V, oracle_mod, gtable, oracle_spline, n, cell, (False, False, False), n_cut, r_cut)
+
+
+@pytest.mark.parametrize("active", [1, 33, 64, 65, 129])
+def test_open_cell_tuned_threads(V, oracle_mod, gtable, oracle_spline, active):
+    """An open orthogonal cell at the thread count that has an instance for such cells
+    besides the default's."""
+    cell, periodic, r_cut = CELLS["open"]
+    n = _density((9, 8, 7), cell, active)
+    s = np.sort(n, axis=None)[::-1]
+    _check(V, oracle_mod, gtable, oracle_spline, n, cell, periodic, 0.5 * (s[active - 1] + s[active]), r_cut,
+           tuning={"threads": 512, "smem_row0": -1})
