@@ -1276,36 +1276,13 @@ struct Warp64 {
     double js[2][kTile];
 };
 
-// MODE 0: energy (unordered pairs), MODE 1: potential (A, U per point).
-//
-// Per work item the warp holds an i tile (lane = i point; two of them in FP32,
-// pair_items_f32).  For each j tile it lists the images whose shifted i box comes
-// within the cutoff of the j box, then each lane marks, for its own j point, which
-// of those images bring the i box within the cutoff of that point.  The pair loop
-// runs over j points (broadcast) and, inside, over the marked images: the delta part
-// of a pair is computed once for all its images.
-//
-// The FP64 instances are bound by the FP64 pipe (1.7 lanes an SM and clock, 1/73 of
-// FP32), so what need not run on it does not: r comes from a table over index
-// displacements (k_r_table; it also holds the cutoff test), the D cell's cubic from
-// a table of polynomials instead of weights and rows (spline64), cells and signs from
-// integer operations on the bits.  Rare cases (past the table, the last delta node)
-// stand behind votes: behind a lane's branch the compiler ran them for all, predicated.
-// FP64 operations per evaluation 136 -> 89 (16 x 28 x 40 monolayer, E + v, a third of
-// whose warps hold a lane past the table), the pipe 88 % busy as before.  ms per pass,
-// 24 x 42 x 60 monolayer E + v 453 -> 274 and E 242 -> 143, hexagonal 20 x 20 x 50
-// 93 -> 47, slab 32 x 28 x 50 185 -> 138, open dimer 31 x 23 x 19 E 16.7 -> 14.0.
-template <typename R, int MODE, int NT, bool SKEW, bool OPEN = false>
-__global__ void __launch_bounds__(NT, 1) k_pair(const __grid_constant__ PairLaunch pl) {
-    constexpr bool POT = (MODE == 1);
-    constexpr int NW = NT / 32;
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    __shared__ unsigned int s_prefix[kMaxInst + 1];
-    __shared__ int s_C[kMaxInst];
-
+// What every CTA does first: the table, with the resident band staged (FP32), the first
+// item of each instance and its chunks.  The band starts behind the warps' parts (NW).
+template <typename R, int NW>
+__device__ __forceinline__ void pair_begin(const PairLaunch &pl, unsigned char *smem_raw, unsigned int *s_prefix,
+                                           int *s_C, Table<R> &tb) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const PairShared &sh = pl.sh;
-    Table<R> tb;
     make_table<R>(sh, tb);
     if constexpr (sizeof(R) == 4) {
         float *band = reinterpret_cast<float *>(smem_raw + sizeof(Warp32) * NW);
@@ -1329,11 +1306,44 @@ __global__ void __launch_bounds__(NT, 1) k_pair(const __grid_constant__ PairLaun
         s_prefix[pl.ninst] = acc;
     }
     __syncthreads();  // the only block barrier: table band and item counts ready
+}
+
+// MODE 0: energy (unordered pairs), MODE 1: potential (A, U per point).
+//
+// Per work item the warp holds an i tile (lane = i point; two of them in FP32,
+// pair_items_f32).  For each j tile it lists the images whose shifted i box comes
+// within the cutoff of the j box, then each lane marks, for its own j point, which
+// of those images bring the i box within the cutoff of that point.  The pair loop
+// runs over j points (broadcast) and, inside, over the marked images: the delta part
+// of a pair is computed once for all its images.
+//
+// The FP64 instances are bound by the FP64 pipe (1.7 lanes an SM and clock, 1/73 of
+// FP32), so what need not run on it does not: r comes from a table over index
+// displacements (k_r_table; it also holds the cutoff test), the D cell's cubic from
+// a table of polynomials instead of weights and rows (spline64), cells and signs from
+// integer operations on the bits.  Rare cases (past the table, the last delta node)
+// stand behind votes: behind a lane's branch the compiler ran them for all, predicated.
+// FP64 operations per evaluation 136 -> 89 (16 x 28 x 40 monolayer, E + v, a third of
+// whose warps hold a lane past the table), the pipe 88 % busy as before.  ms per pass,
+// 24 x 42 x 60 monolayer E + v 453 -> 274 and E 242 -> 143, hexagonal 20 x 20 x 50
+// 93 -> 47, slab 32 x 28 x 50 185 -> 138, open dimer 31 x 23 x 19 E 16.7 -> 14.0.
+template <typename R, int MODE, int NT, bool SKEW>
+__global__ void __launch_bounds__(NT, 1) k_pair(const __grid_constant__ PairLaunch pl) {
+    constexpr bool POT = (MODE == 1);
+    constexpr int NW = NT / 32;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ unsigned int s_prefix[kMaxInst + 1];
+    __shared__ int s_C[kMaxInst];
+
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const PairShared &sh = pl.sh;
+    Table<R> tb;
+    pair_begin<R, NW>(pl, smem_raw, s_prefix, s_C, tb);
     // autotuning samples every item_stride-th item (item * stride < the total)
     const unsigned int stride = max(1u, sh.item_stride);
     const unsigned int n_items = min((s_prefix[pl.ninst] + stride - 1u) / stride, sh.item_limit);
     if constexpr (sizeof(R) == 4) {
-        pair_items_f32<MODE, NT, SKEW, OPEN>(pl, smem_raw, s_prefix, s_C, n_items, stride, tb);
+        pair_items_f32<MODE, NT, SKEW, false>(pl, smem_raw, s_prefix, s_C, n_items, stride, tb);
         return;
     } else {
     const Consts<double> &K = sh.k64;
@@ -1596,6 +1606,19 @@ __global__ void __launch_bounds__(NT, 1) k_pair(const __grid_constant__ PairLaun
     }
 }
 
+// Cells without images or a cutoff (FP32; see pair_items_f32).
+template <int MODE, int NT, bool SKEW>
+__global__ void __launch_bounds__(NT, 1) k_pair_open(const __grid_constant__ PairLaunch pl) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ unsigned int s_prefix[kMaxInst + 1];
+    __shared__ int s_C[kMaxInst];
+    Table<float> tb;
+    pair_begin<float, NT / 32>(pl, smem_raw, s_prefix, s_C, tb);
+    const unsigned int stride = max(1u, pl.sh.item_stride);
+    const unsigned int n_items = min((s_prefix[pl.ninst] + stride - 1u) / stride, pl.sh.item_limit);
+    pair_items_f32<MODE, NT, SKEW, true>(pl, smem_raw, s_prefix, s_C, n_items, stride, tb);
+}
+
 // Per D cell k and delta column l the cubic in t (times 1, as the coefficients / 36 give
 // it) through rows k .. k + 3 of the bicubic coefficients: poly[(k S + l) 4 ...].
 __global__ void k_table_poly(const double *__restrict__ c, long long n, int S, double *__restrict__ poly) {
@@ -1807,7 +1830,11 @@ __global__ void k_kernel_eval(const PairShared sh, int64_t npts, const double *r
 
 template <typename R, int MODE, int NT, bool SKEW, bool OPEN = false>
 int launch_one(const PairLaunch &pl, int nctas, size_t smem, cudaStream_t st) {
-    auto kern = k_pair<R, MODE, NT, SKEW, OPEN>;
+    void (*kern)(PairLaunch) = nullptr;
+    if constexpr (OPEN)
+        kern = k_pair_open<MODE, NT, SKEW>;
+    else
+        kern = k_pair<R, MODE, NT, SKEW>;
     VDWDF_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                         static_cast<int>(smem)));
     kern<<<nctas, NT, smem, st>>>(pl);
