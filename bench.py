@@ -272,7 +272,7 @@ def run_gpu(args):
         tails.append(V.far_tail(n, w["lengths"], w["periodic"], w["n_cut"], w["r_cut"]))
     tail = {"T_hartree": tails[-1]["T"], "E_plus_T_hartree": results[-1][0] + tails[-1]["T"],
             "ms_per_call": float(np.median([t["ms"] for t in tails[1:]])), "nodes": tails[-1]["nodes"],
-            "planes": tails[-1]["planes"], "bound": "fp64 (one exp per active point and quadrature node)"}
+            "planes": tails[-1]["planes"], "bound": "fp64 (per active point three exps, moments, a square per node)"}
     # the same at a 30 bohr cutoff (FP32 energy): E + T should hardly move
     E30, _ = V.energy(n, w["lengths"], w["periodic"], w["n_cut"], 30.0, T, precision="fp32")
     T30 = V.far_tail(n, w["lengths"], w["periodic"], w["n_cut"], 30.0)["T"]
@@ -342,7 +342,7 @@ def run_gpu(args):
         "semilocal": {"ms_per_call": semi_t, "points": int(n.numel()),
                       "points_per_s": n.numel() / (semi_t * 1e-3),
                       "hbm_gbs": 8.0 * n.numel() / (semi_t * 1e-3) / 1e9,
-                      "bound": "fp64 (per-point cbrt, log, expm1 at GB300's FP64 rate)",
+                      "bound": "fp64 (per-point cube root, log, expm1 series at GB300's FP64 rate)",
                       "E_hartree": {k: semi[k] for k in ("Ex_lda", "Ec_lda", "Ex_pbe", "Ec_pbe", "Ex_revpbe")},
                       "eq3_needed_number": semi["Ec_lda"] - semi["Ec_pbe"] + results[-1][0]},
         "far_tail": tail,
@@ -468,7 +468,7 @@ def run_workloads(V, inputs, T, dev, flush, sms, fp64_peak):
             e["fp64_64x56x100"] = rate(d["f64_regrid"], None, ops)
             e["fp32_over_fp64"] = e["fp32_64x56x100"]["pairs_per_s"] / e["fp64_64x56x100"]["pairs_per_s"]
             e["rel_err_fp32_vs_fp64"] = abs(d["f32_regrid"][2] - d["f64_regrid"][2]) / abs(d["f64_regrid"][2])
-            e["fp64_note"] = "the FP64 E + v pass at full size takes about 11 min; ratio on the 64x56x100 regrid"
+            e["fp64_note"] = "the FP64 E + v pass at full size takes about 8 min; ratio on the 64x56x100 regrid"
         out[key] = e
     return out
 
