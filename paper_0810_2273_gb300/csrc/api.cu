@@ -297,6 +297,7 @@ struct Geom {
     long long N;
     int M[3];
     int rtm[3];         // FP64: largest |index displacement| that can lie inside the cutoff
+    bool rtab;          // FP64: ... which a table can hold along every axis
     double rc;
     bool use_cut;
     double B[9];        // reciprocal rows: B_a . M_b = delta_ab
@@ -387,6 +388,7 @@ int check_cut(double n_cut, double r_cut, Geom &G) {
     if (any_per && !(r_cut > 0.0)) return VDWDF_EINVAL;
     G.use_cut = r_cut > 0.0;
     G.rc = G.use_cut ? r_cut : 0.0;
+    G.rtab = true;
     for (int a = 0; a < 3; ++a) {
         // every image L with |r_i - r_j + L| <= r_cut has |m_a| <= r_cut |B_a| + 1
         const double bl = std::sqrt(G.B[3 * a] * G.B[3 * a] + G.B[3 * a + 1] * G.B[3 * a + 1] +
@@ -397,6 +399,9 @@ int check_cut(double n_cut, double r_cut, Geom &G) {
         // r_cut spans r_cut |B_a| N_a cells along a; without images the grid bounds it too
         const double cells = std::floor(G.rc * bl * G.dims[a] * (1.0 + 1e-9)) + 1.0;
         const double most = G.per[a] ? cells : (G.use_cut ? std::min<double>(cells, G.dims[a] - 1) : G.dims[a] - 1);
+        // (the product of three extents up to a million stays within 64 bits; a table for
+        // fewer displacements than occur would lose pairs)
+        G.rtab = G.rtab && most <= 1e6;
         G.rtm[a] = static_cast<int>(std::min(most, 1e6));
     }
     return VDWDF_OK;
@@ -437,7 +442,7 @@ struct Work {
 // table, so that the grids it takes do not depend on the cutoff)
 size_t layout(const Geom &G, int nb, bool pot, bool fp64, Work *w, unsigned char *base, bool alloc_free = false) {
     Carve c;
-    const bool rtab = fp64 && !alloc_free && r_table_entries(G.rtm, G.skew) <= kMaxRTable;
+    const bool rtab = fp64 && !alloc_free && G.rtab && r_table_entries(G.rtm, G.skew) <= kMaxRTable;
     const size_t N = static_cast<size_t>(G.N);
     const size_t tiles = (N + kTile - 1) / kTile;
     const size_t o_q0 = c.take<double>(N);
