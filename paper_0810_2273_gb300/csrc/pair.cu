@@ -1181,13 +1181,17 @@ __device__ __forceinline__ void spline64(const double *poly, int S, int k, doubl
 }
 
 // past_part in FP64 with one reciprocal (of eq. (17)'s denominator times tD) in place
-// of five divisions.  y = q_i q_j and s2 = q_i^2 + q_j^2.
+// of five divisions.  y = q_i q_j and s2 = q_i^2 + q_j^2.  False, and nothing written,
+// where that product (27 (q r)^7 at equal q) is not within 2^-500 .. 2^501: past_part
+// takes such pairs, whose divisions by an infinity give the 0 that they contribute.
 template <bool POT>
-__device__ __forceinline__ void past_part64(double r, double tD, double qi, double qj, const Consts<double> &K,
+__device__ __forceinline__ bool past_part64(double r, double tD, double qi, double qj, const Consts<double> &K,
                                             const double *rho_c, double &phi, double &rd, double &rd2) {
     const double r2 = r * r, r6 = r2 * r2 * r2, y = qi * qj, s2 = fma(qi, qi, qj * qj);
-    const double z = r6 * (y * y), X = z * s2;
-    const double w = rcp_newton(X * tD);
+    const double z = r6 * (y * y), X = z * s2, XtD = X * tD;
+    // (by the exponent, off the FP64 pipe)
+    if (static_cast<unsigned>(__double2hiint(XtD) - ((1023 - 500) << 20)) >= (1001u << 20)) return false;
+    const double w = rcp_newton(XtD);
     const double inv = w * tD, itD = w * X;  // 1/X, 1/tD
     const double p17 = -K.C * inv;
     const bool i_small = qi < qj;
@@ -1222,6 +1226,7 @@ __device__ __forceinline__ void past_part64(double r, double tD, double qi, doub
         rd = fma(t, fma(qi, is2, qj * iy), p17 * (i_small ? ramp - sl : ramp));
         rd2 = fma(t, fma(qj, is2, qi * iy), p17 * (i_small ? ramp : ramp - sl));
     }
+    return true;
 }
 
 // FP64 warp sums of two values (as warp_sum2).
@@ -1535,13 +1540,12 @@ __global__ void __launch_bounds__(NT, 1) k_pair(const __grid_constant__ PairLaun
                             t = end ? 1.0 : (on ? t : 0.0);
                             if (in && !(on && poly)) {
                                 double phi, rd = 0.0, rd2 = 0.0;
-                                if (on) {
-                                    // a table too large for polynomials: from its coefficients
+                                if (on || !past_part64<POT>(r, tD, qi, qj, K, tb.rho, phi, rd, rd2)) {
+                                    // a table too large for polynomials, from its coefficients, or a
+                                    // pair past it that past_part64 leaves
                                     Delta<double> dd;
                                     delta_part<POT, double>(qi, qj, K, dd);
                                     dist_part<POT, double>(r, r * r, qi, qj, 1.0 / qi, qi * qi, dd, K, tb, phi, rd, rd2);
-                                } else {
-                                    past_part64<POT>(r, tD, qi, qj, K, tb.rho, phi, rd, rd2);
                                 }
                                 A += phi;
                                 if (POT) {
