@@ -51,6 +51,7 @@ constexpr double kPlainMin = 1e-40, kPlainMax = 1e40;
 __device__ __forceinline__ LocalPoint local_point(double n) {
     LocalPoint p;
     if (!(n > kPlainMin && n < kPlainMax)) {
+        n = n < 1e-300 ? 1e-300 : n;  // (1/n and r_s would overflow; such a point weighs nothing)
         p.kF = cbrt(3.0 * kPi * kPi * n);
         p.ikF = 1.0 / p.kF;
         p.in = 1.0 / n;
@@ -342,6 +343,15 @@ constexpr int kSemiBlocks = 608;  // 4 per SM on 152 SMs
 constexpr int kSemiThreads = 256;
 constexpr int kSemiVals = 6;      // five energies and the point count
 
+// x >= 0 cut to 2^332 (1e100), an infinity too; NaN stays.  F_x and H have reached
+// their limits in y and v long before, and what they multiply them into stays finite
+// (E is at most 1e103).  By the exponent, off the FP64 pipe.
+__device__ __forceinline__ double cap_limit(double x) {
+    constexpr int top = (1023 + 332) << 20;
+    const int hi = __double2hiint(x);
+    return hi >= top && hi <= 0x7FF00000 ? __hiloint2double(top, 0) : x;
+}
+
 __global__ void __launch_bounds__(kSemiThreads) k_semilocal(int n0, int n1, int n2, const AxisMap am,
                                                             const double *__restrict__ n,
                                                             const double *__restrict__ gin,
@@ -359,16 +369,14 @@ __global__ void __launch_bounds__(kSemiThreads) k_semilocal(int n0, int n1, int 
         grad_at(m, n0, n1, n2, am, n, gin, gx, gy, gz);
         const LocalPoint p = local_point(nn);
         const double hx = gx * p.in, hy = gy * p.in, hz = gz * p.in;
-        double G = fma(hx, hx, fma(hy, hy, hz * hz));  // |g/n|^2
-        // (F_x and H have reached their limits long before; NaN stays)
-        G = G > 1e100 ? 1e100 : G;
+        const double G = fma(hx, hx, fma(hy, hy, hz * hz));  // |g/n|^2
         const double ex = -3.0 / (4.0 * kPi) * p.kF;
         const double s2 = 0.25 * G * p.ikF * p.ikF, t2 = (kPi / 16.0) * G * p.ikF;
         // F_x = 1 + kappa mu s^2/(kappa + mu s^2), both kappas from one reciprocal
-        const double k1 = 0.804, k2 = 1.245, y = mu * s2, e1 = k1 + y, e2 = k2 + y, ie = y * rcp_newton(e1 * e2);
+        const double k1 = 0.804, k2 = 1.245, y = cap_limit(mu * s2), e1 = k1 + y, e2 = k2 + y, ie = y * rcp_newton(e1 * e2);
         // A = (beta/gamma)/E, E = expm1(-eps_c/gamma): the argument of H's logarithm is
         // v E (E + v)/(E^2 + E v + v^2), v = (beta/gamma) t^2
-        const double E = expm1_taylor(p.ec * (-1.0 / gamma)), v = (beta / gamma) * t2;
+        const double E = expm1_taylor(p.ec * (-1.0 / gamma)), v = cap_limit((beta / gamma) * t2);
         const double num = v * E * (E + v), dn = fma(E, E, v * (E + v));
         // (a vanishing eps_c or gradient could make the denominator vanish; H is 0 then)
         const double H = dn > 1e-280 ? gamma * log1p_ratio(num, dn) : (dn == dn ? 0.0 : dn);
