@@ -33,7 +33,9 @@
  *    and freed on it before return; the library owns it.
  *  - Fault injection for tests (host side only; no device fault is caused):
  *    with the environment variable VDWDF_FAIL_ALLOC=1 every scratch
- *    allocation fails (VDWDF_EALLOC); with VDWDF_MAX_ITERS=k the persistent
+ *    allocation fails (VDWDF_EALLOC); with VDWDF_FAIL_ALLOC=2 a table's
+ *    polynomials and texture cannot be had, which the sums go without (the
+ *    same results to their precision, slower); with VDWDF_MAX_ITERS=k the persistent
  *    pair kernels stop after k work items per CTA, as their iteration guard
  *    does, and the call returns VDWDF_ETIMEOUT.  The next call without them
  *    works as before.
@@ -464,6 +466,10 @@ int vdwdf_diag_voxel_potential(const vdwdf_grid *grid, const double *n_dev, doub
  *    is, used there once by vdwdf_energy, vdwdf_potential,
  *    vdwdf_energy_batched or vdwdf_kernel_eval (npts >= 1), because making it
  *    resident allocates.  Otherwise the call returns VDWDF_ENOTABLE.
+ *    FP64 sums are faster with polynomials of the table beside it.  Tables of
+ *    up to 2^18 cells (8 MB of polynomials; 400 x 200 nodes take 2.6 MB) have
+ *    them once resident, larger ones from their first FP64 sum by vdwdf_energy,
+ *    vdwdf_potential or vdwdf_energy_batched on.
  *  - Overlap: calls overlapping in time would race on the one scratch array.
  *    The library therefore holds a process-wide lock for the whole call, and
  *    the call synchronises its stream before every return that follows its

@@ -33,9 +33,11 @@ struct vdwdf_table {
     struct Dev {
         double *d64 = nullptr;
         float *d32 = nullptr;
-        double *poly = nullptr;         // per cell cubics of d64 (NULL: the table is too large)
+        // copies that the sums are faster with, and go without
+        double *poly = nullptr;         // per cell cubics of d64 (NULL: none, see want_poly)
+        bool poly_tried = false;
         cudaArray_t arr = nullptr;      // the bicubic block of coef32 for texture gathers
-        cudaTextureObject_t tex = 0;    // 0: the table exceeds the texture limits
+        cudaTextureObject_t tex = 0;    // 0: the table exceeds the texture limits, or none could be had
     };
     std::map<int, Dev> dev;  // device id -> copies
 };
@@ -49,12 +51,17 @@ std::atomic<unsigned long long> g_table_gen{0};  // generation ids of tables
 
 // Fault injection for tests, on the host only (no device fault is ever caused):
 //   VDWDF_FAIL_ALLOC=1  every scratch allocation of a call fails (VDWDF_EALLOC);
+//   VDWDF_FAIL_ALLOC=2  the copies of a table that the sums can go without fail;
 //   VDWDF_MAX_ITERS=k   the persistent pair kernels stop after k work items per
 //                       CTA, as their iteration guard would, so the call returns
 //                       VDWDF_ETIMEOUT.
 bool fail_alloc_requested() {
     const char *e = std::getenv("VDWDF_FAIL_ALLOC");
     return e && e[0] == '1';
+}
+bool fail_optional_requested() {
+    const char *e = std::getenv("VDWDF_FAIL_ALLOC");
+    return e && e[0] == '2';
 }
 unsigned int max_iters_override(unsigned int v) {
     const char *e = std::getenv("VDWDF_MAX_ITERS");
@@ -126,6 +133,7 @@ constexpr double kPi = 3.14159265358979323846;
 constexpr int kMaxImages = 64;
 constexpr long long kMaxRTable = 1LL << 23;  // entries of the FP64 path's displacement table (64 MB)
 constexpr long long kMaxPoly = 1LL << 22;    // cells of a table kept as polynomials (128 MB)
+constexpr long long kSmallPoly = 1LL << 18;  // ... with the first call of any kind (8 MB)
 
 // Device layout of the coefficients: (nD + 2) x (nd + 2) bicubic coefficients / 36,
 // then nd + 2 coefficients / 6 of the beyond-table normalisation rho(delta).
@@ -158,15 +166,20 @@ struct TableDev {
 };
 
 // The bicubic block of the FP32 coefficients as a texture (exact fetches of single
-// values); none when an axis exceeds the device's limit for gathers.
+// values); none when an axis exceeds the device's limit for gathers or it cannot be had
+// (the FP32 sums then read the band and the global coefficients).
 int make_texture(const vdwdf_table *t, int dev, vdwdf_table::Dev &d) {
     const int S = t->nd + 2, rows = t->nD + 2;
     int wmax = 0, hmax = 0;
     VDWDF_CUDA_TRY(cudaDeviceGetAttribute(&wmax, cudaDevAttrMaxTexture2DGatherWidth, dev));
     VDWDF_CUDA_TRY(cudaDeviceGetAttribute(&hmax, cudaDevAttrMaxTexture2DGatherHeight, dev));
-    if (S > wmax || rows > hmax) return VDWDF_OK;
+    if (S > wmax || rows > hmax || fail_optional_requested()) return VDWDF_OK;
     const cudaChannelFormatDesc cd = cudaCreateChannelDesc<float>();
-    if (cudaMallocArray(&d.arr, &cd, S, rows, cudaArrayTextureGather) != cudaSuccess) return VDWDF_EALLOC;
+    if (cudaMallocArray(&d.arr, &cd, S, rows, cudaArrayTextureGather) != cudaSuccess) {
+        cudaGetLastError();  // (not an error of the next launch)
+        d.arr = nullptr;
+        return VDWDF_OK;
+    }
     VDWDF_CUDA_TRY(cudaMemcpy2DToArray(d.arr, 0, 0, t->coef32.data(), sizeof(float) * S, sizeof(float) * S, rows,
                                        cudaMemcpyHostToDevice));
     cudaResourceDesc rd;
@@ -180,6 +193,28 @@ int make_texture(const vdwdf_table *t, int dev, vdwdf_table::Dev &d) {
     td.readMode = cudaReadModeElementType;
     VDWDF_CUDA_TRY(cudaCreateTextureObject(&d.tex, &rd, &td, nullptr));
     return VDWDF_OK;
+}
+
+// The polynomials of the FP64 sums, once per device; none for tables of more than
+// kMaxPoly cells, or when they cannot be had (the sums then read the coefficients).
+int make_poly(const vdwdf_table *t, vdwdf_table::Dev &d) {
+    const int S = t->nd + 2;
+    const long long cells = static_cast<long long>(t->nD - 1) * S;
+    if (d.poly_tried) return VDWDF_OK;
+    d.poly_tried = true;
+    if (cells > kMaxPoly || fail_optional_requested()) return VDWDF_OK;
+    if (cudaMalloc(&d.poly, static_cast<size_t>(cells) * 4 * sizeof(double)) != cudaSuccess) {
+        cudaGetLastError();
+        d.poly = nullptr;
+        return VDWDF_OK;
+    }
+    int rc = launch_table_poly(d.d64, t->nD, S, d.poly);
+    if (rc == VDWDF_OK && cudaStreamSynchronize(nullptr) != cudaSuccess) rc = VDWDF_ECUDA;
+    if (rc) {
+        cudaFree(d.poly);
+        d.poly = nullptr;
+    }
+    return rc;
 }
 
 void free_copies(vdwdf_table::Dev &d) {
@@ -200,7 +235,11 @@ TableDev view_of(const vdwdf_table::Dev &d) {
     return v;
 }
 
-int table_on_device(const vdwdf_table *tc, TableDev *out) {
+// The copies of a table on the current device, made by the first call that needs them.
+// want_poly: the call is an FP64 pair sum (which waits for its stream, so that an
+// allocation is in order).  Small tables have their polynomials from the first call of any
+// kind, so that vdwdf_energy_noalloc finds them; others do not cost an FP32 caller 128 MB.
+int table_on_device(const vdwdf_table *tc, TableDev *out, bool want_poly = false) {
     vdwdf_table *t = const_cast<vdwdf_table *>(tc);
     int dev = 0;
     VDWDF_CUDA_TRY(cudaGetDevice(&dev));
@@ -214,13 +253,9 @@ int table_on_device(const vdwdf_table *tc, TableDev *out) {
             if (cudaMalloc(&d.d32, n * sizeof(float)) != cudaSuccess) return VDWDF_EALLOC;
             VDWDF_CUDA_TRY(cudaMemcpy(d.d64, t->coef64.data(), n * sizeof(double), cudaMemcpyHostToDevice));
             VDWDF_CUDA_TRY(cudaMemcpy(d.d32, t->coef32.data(), n * sizeof(float), cudaMemcpyHostToDevice));
-            const int S = t->nd + 2;
-            if (static_cast<long long>(t->nD - 1) * S <= kMaxPoly) {
-                if (cudaMalloc(&d.poly, static_cast<size_t>(t->nD - 1) * S * 4 * sizeof(double)) != cudaSuccess)
-                    return VDWDF_EALLOC;
-                const int rc = launch_table_poly(d.d64, t->nD, S, d.poly);
+            if (static_cast<long long>(t->nD - 1) * (t->nd + 2) <= kSmallPoly) {
+                const int rc = make_poly(t, d);
                 if (rc) return rc;
-                VDWDF_CUDA_TRY(cudaStreamSynchronize(nullptr));
             }
             return make_texture(t, dev, d);
         };
@@ -230,6 +265,10 @@ int table_on_device(const vdwdf_table *tc, TableDev *out) {
             return rc;
         }
         it = t->dev.emplace(dev, d).first;
+    }
+    if (want_poly) {
+        const int rc = make_poly(t, it->second);
+        if (rc) return rc;
     }
     *out = view_of(it->second);
     return VDWDF_OK;
@@ -803,7 +842,7 @@ int run_single(const vdwdf_grid *grid, const double *n_dev, const double *grad_d
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const long long launches0 = g_launches.load();
     TableDev td;
-    rc = table_on_device(table, &td);
+    rc = table_on_device(table, &td, precision == VDWDF_FP64);
     if (rc) return rc;
     int *order = nullptr, nb = 0;
     rc = brick_order(G.dims, &order, &nb);
@@ -1455,7 +1494,7 @@ int diag_voxel(const vdwdf_grid *grid, const double *n_dev, const double *grad_d
 int autotune_one(const Geom &G, const double *n_dev, double n_cut, const vdwdf_table *table, int precision,
                  vdwdf_tuning *best, cudaStream_t st) {
     TableDev td;
-    int rc = table_on_device(table, &td);
+    int rc = table_on_device(table, &td, precision == VDWDF_FP64);
     if (rc) return rc;
     int *order = nullptr, nb = 0;
     rc = brick_order(G.dims, &order, &nb);
@@ -1804,7 +1843,7 @@ int vdwdf_energy_batched(int ninst, const vdwdf_grid *grids, const double *const
     const bool tune_auto = tuning && tuning->threads == VDWDF_TUNE_AUTO;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     TableDev td;
-    int rc = table_on_device(table, &td);
+    int rc = table_on_device(table, &td, precision == VDWDF_FP64);
     if (rc) return rc;
     int dev = 0;
     VDWDF_CUDA_TRY(cudaGetDevice(&dev));
