@@ -29,8 +29,11 @@
  *    device work of a call is ordered on that stream.  Calls that return
  *    host results (vdwdf_result, E_out) synchronise that stream before
  *    returning; the others return without waiting.
- *  - Scratch device memory is taken with cudaMallocAsync on the call's stream
- *    and freed on it before return; the library owns it.
+ *  - Scratch device memory is taken stream-ordered on the call's stream and
+ *    freed on it before return; the library owns it.  Calls that synchronise
+ *    take it from a memory pool of the library's own, which keeps up to 64 MB
+ *    per device between calls while a table lives and nothing otherwise; the
+ *    others from the device's default pool.
  *  - Fault injection for tests (host side only; no device fault is caused):
  *    with the environment variable VDWDF_FAIL_ALLOC=1 every scratch
  *    allocation fails (VDWDF_EALLOC); with VDWDF_FAIL_ALLOC=2 a table's

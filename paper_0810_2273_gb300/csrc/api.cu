@@ -74,7 +74,8 @@ unsigned int max_iters_override(unsigned int v) {
 // the device's default pool gives its memory back at every synchronisation, and
 // mapping it again took half of a small call (Kr dimer 24 x 18 x 18, E FP32: 533 us of
 // which the pair pass is 220, against 343 with the pool).  Trimmed to nothing
-// when the last table is freed.
+// when the last table is freed, and while none lives at the end of each call that takes
+// none (semilocal energies, far fields).
 constexpr unsigned long long kPoolKeep = 64ull << 20;
 std::mutex g_pool_mu;
 std::map<int, cudaMemPool_t> g_pools;
@@ -110,6 +111,11 @@ cudaError_t scratch_pool(cudaMemPool_t *pool) {
 void trim_pools() {
     std::lock_guard<std::mutex> lk(g_pool_mu);
     for (auto &kv : g_pools) cudaMemPoolTrimTo(kv.second, 0);
+}
+
+// At the end of a call without a table, its scratch freed on st.
+void give_back(cudaStream_t st) {
+    if (g_tables.load() == 0 && cudaStreamSynchronize(st) == cudaSuccess) trim_pools();
 }
 
 // A call's scratch, with the fault-injection hook: from the library's pool (freed with
@@ -1314,6 +1320,7 @@ int vdwdf_semilocal(const vdwdf_grid *grid, const double *n_dev, const double *g
         rc = VDWDF_ECUDA;
     cudaFreeAsync(scratch, st);
     if (rc == VDWDF_OK && cudaStreamSynchronize(st) != cudaSuccess) rc = VDWDF_ECUDA;
+    give_back(st);
     if (rc) return rc;
     std::memset(out, 0, sizeof(*out));
     out->Ex_lda = G.dV * sums[0];
@@ -1781,6 +1788,7 @@ int vdwdf_far_tail(const vdwdf_grid *grid, const double *n_dev, const double *gr
     if (lbase) cudaFreeAsync(lbase, st);
     cudaFreeAsync(base, st);
     if (rc == VDWDF_OK && cudaStreamSynchronize(st) != cudaSuccess) rc = VDWDF_ECUDA;
+    give_back(st);
     if (rc) return rc;
     std::memset(out, 0, sizeof(*out));
     out->T = T;

@@ -1,7 +1,13 @@
 """What the library keeps on the device, and calls that go without an optional part of
-it: the FP64 polynomials and the texture copy of a table."""
+it: the FP64 polynomials and the texture copy of a table, the scratch pool of calls
+without a table."""
+import subprocess
+import sys
+
 import numpy as np
 import pytest
+
+from conftest import ROOT
 
 pytestmark = pytest.mark.gpu
 
@@ -84,3 +90,38 @@ def test_calls_without_the_optional_table_copies(V, oracle_mod, oracle_table, or
     assert np.max(np.abs(vg.cpu().numpy() - v)) <= 10 * tol * np.max(np.abs(v))
     monkeypatch.delenv("VDWDF_FAIL_ALLOC")
     table.free()
+
+
+CHILD = """
+import torch
+import numpy as np
+import paper_0810_2273_gb300 as V
+def free():
+    torch.cuda.synchronize()
+    return torch.cuda.mem_get_info(0)[0]
+n = torch.full((120, 120, 120), 0.05, dtype=torch.float64, device="cuda:0")
+table = V.Table.from_nodes(np.linspace(1.0, 0.1, 24).reshape(6, 4), 12.0)
+calls = (lambda: V.semilocal(n, (60.0,) * 3, (1, 1, 1), gradient="spectral"),
+         lambda: V.far_tail(n, (60.0,) * 3, (1, 1, 1), 1e-6, 8.0, want_v=True),
+         lambda: V.far_tail(n, (60.0,) * 3, (1, 0, 0), 1e-6, 8.0))
+for call in calls:
+    call()
+with_table = free()
+table.free()
+without = free()
+print(without - with_table)
+for call in calls:
+    for _ in range(2):
+        call()
+        print(without - free())
+"""
+
+
+def test_scratch_is_given_back_without_tables():
+    """Semilocal energies and far fields, which take no table, keep no device memory
+    when they return while no table lives (in a process of its own)."""
+    out = subprocess.run([sys.executable, "-c", CHILD], capture_output=True, text=True, cwd=ROOT, timeout=600)
+    assert out.returncode == 0, out.stderr[-2000:]
+    kept = [int(x) for x in out.stdout.split()]
+    assert kept[0] >= 32 << 20  # what the calls kept while the table lived
+    assert kept[1:] == [0] * 6, kept
