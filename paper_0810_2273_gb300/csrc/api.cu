@@ -1843,11 +1843,15 @@ int vdwdf_energy_batched(int ninst, const vdwdf_grid *grids, const double *const
         rc = check_tuning(tuning, geo[k].skew, true);
         if (rc) return rc;
     }
-    // one launch runs its instances with or without the cross terms: beside a skewed
-    // cell the orthogonal ones run as skewed cells too (their cross terms are 0)
-    bool any_skew = false;
-    for (const Geom &g : geo) any_skew = any_skew || g.skew;
-    for (Geom &g : geo) g.skew = any_skew;
+    // one launch (kMaxInst instances) runs its instances with or without the cross terms:
+    // beside a skewed cell in it the orthogonal ones run as skewed cells too (their cross
+    // terms are 0)
+    for (int k0 = 0; k0 < ninst; k0 += kMaxInst) {
+        const int k1 = std::min(ninst, k0 + kMaxInst);
+        bool any_skew = false;
+        for (int k = k0; k < k1; ++k) any_skew = any_skew || geo[k].skew;
+        for (int k = k0; k < k1; ++k) geo[k].skew = any_skew;
+    }
     const bool tune_auto = tuning && tuning->threads == VDWDF_TUNE_AUTO;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
     TableDev td;
