@@ -138,6 +138,7 @@ cudaError_t scratch_malloc(void **p, size_t bytes) {
 constexpr double kPi = 3.14159265358979323846;
 constexpr int kMaxImages = 64;
 constexpr long long kMaxRTable = 1LL << 23;  // entries of the FP64 path's displacement table (64 MB)
+constexpr long long kMaxBatchRTable = 1LL << 27;  // ... of all instances of a batch (1 GB)
 constexpr long long kMaxPoly = 1LL << 22;    // cells of a table kept as polynomials (128 MB)
 constexpr long long kSmallPoly = 1LL << 18;  // ... with the first call of any kind (8 MB)
 
@@ -1851,6 +1852,17 @@ int vdwdf_energy_batched(int ninst, const vdwdf_grid *grids, const double *const
         bool any_skew = false;
         for (int k = k0; k < k1; ++k) any_skew = any_skew || geo[k].skew;
         for (int k = k0; k < k1; ++k) geo[k].skew = any_skew;
+    }
+    // FP64: a plan keeps its instances' distance tables; past the bound the others'
+    // distances are computed
+    if (precision == VDWDF_FP64) {
+        long long held = 0;
+        for (Geom &g : geo) {
+            const long long e = r_table_entries(g.rtm, g.skew);
+            if (!g.rtab || e > kMaxRTable) continue;
+            g.rtab = held + e <= kMaxBatchRTable;
+            if (g.rtab) held += e;
+        }
     }
     const bool tune_auto = tuning && tuning->threads == VDWDF_TUNE_AUTO;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);

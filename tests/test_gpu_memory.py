@@ -1,6 +1,6 @@
 """What the library keeps on the device, and calls that go without an optional part of
 it: the FP64 polynomials and the texture copy of a table, the scratch pool of calls
-without a table."""
+without a table, the distance tables of a large batch."""
 import subprocess
 import sys
 
@@ -125,3 +125,23 @@ def test_scratch_is_given_back_without_tables():
     kept = [int(x) for x in out.stdout.split()]
     assert kept[0] >= 32 << 20  # what the calls kept while the table lived
     assert kept[1:] == [0] * 6, kept
+
+
+def test_large_fp64_batch_bounds_its_distance_tables(V, oracle_mod, oracle_table, oracle_spline):
+    """Two hundred cells of two active points under a long cutoff, whose tables of
+    distances (55 MB each) would take 11 GB: the batch takes them for as many as fit
+    its bound and computes the others' distances; all energies agree."""
+    table = V.Table.from_nodes(oracle_table, 30.0)
+    base = np.zeros(DIMS)
+    base[2, 3, 4], base[5, 6, 1] = 0.3, 0.2
+    ns = [_t(base * (1.0 + 0.001 * k)) for k in range(200)]
+    per, rc = (True, True, True), 105.0
+    V.energy_batched(ns[:1], [L], [per], 1e-6, 20.0, table, "fp64")
+    free0 = _free()
+    E, r = V.energy_batched(ns, [L] * 200, [per] * 200, 1e-6, rc, table, "fp64")
+    assert free0 - _free() < 2 << 30
+    for k in (0, 18, 19, 199):
+        e = oracle_mod.Problem(base * (1.0 + 0.001 * k), L, per, 1e-6, rc, oracle_spline).energy()
+        assert abs(E[k] - e["E"]) <= 1e-10 * abs(e["E"])
+    assert r["pairs"] == 200 * e["pairs"]
+    table.free()
