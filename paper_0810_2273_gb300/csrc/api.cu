@@ -9,6 +9,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <cfloat>
 #include <cmath>
 #include <cstdio>
 #include <cstdlib>
@@ -611,7 +612,15 @@ void fill_params(const Geom &G, const Work &w, PairParams &pp) {
     for (int a = 0; a < 3; ++a) {
         pp.h2[a] = G.met[a];
         pp.g2x[a] = 2.0 * G.met[3 + a];
+        // FP32: r^2 of any displacement is a normal number, as the kernel's reciprocal root
+        // needs; where the spacing is raised for it (below 1.1e-19), D is 0 to FP32 and the
+        // cutoff is left to the FP64 recheck
         pp.h2f[a] = static_cast<float>(pp.h2[a]);
+        if (pp.h2f[a] < FLT_MIN) {
+            pp.h2f[a] = FLT_MIN;
+            pp.cut_lo = -1.0f;
+            pp.cut_hi = FLT_MAX;
+        }
         pp.g2f[a] = static_cast<float>(pp.g2x[a]);
         pp.dims[a] = G.dims[a];
         pp.M[a] = G.M[a];
