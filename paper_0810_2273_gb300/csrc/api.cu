@@ -609,6 +609,19 @@ void fill_params(const Geom &G, const Work &w, PairParams &pp) {
     pp.cut_hi = rc2f * (1.0f + 1e-5f);
     pp.box_out = rc2f * 1.0002f + 1e-6f;
     pp.box_in = rc2f * 0.9998f - 1e-6f;
+    if (G.skew && G.use_cut) {
+        // Cartesian boxes in FP32: a gap collects at most eleven roundings of sums as large
+        // as the cell with its images.  Where these are more than half of the margins (a
+        // cell of more than about 70 cutoffs), the margins grow by them
+        double span = 0.0;
+        for (int a = 0; a < 3; ++a) span += G.L[a] * (G.M[a] + 1);
+        const double eps = std::ldexp(12.0 * span, -24);
+        if (eps > 0.5e-4 * G.rc) {
+            const double far = G.rc + eps, near = std::max(0.0, G.rc - eps);
+            pp.box_out = static_cast<float>(far * far) * 1.0002f + 1e-6f;
+            pp.box_in = static_cast<float>(near * near) * 0.9998f - 1e-6f;
+        }
+    }
     for (int a = 0; a < 3; ++a) {
         pp.h2[a] = G.met[a];
         pp.g2x[a] = 2.0 * G.met[3 + a];
