@@ -154,7 +154,7 @@ typedef struct {
                                  other fields are ignored) */
 typedef struct {
     int32_t threads;      /* threads per CTA: 256, 384, 448, 512 or 1024 (0 = default:
-                             FP32 640, which only the default takes; FP64 512,
+                             FP32 640, which has no other name; FP64 512,
                              for E + v 256, or 384 on skewed cells);
                              skewed cells take 384, 448 or 512; VDWDF_TUNE_AUTO in
                              vdwdf_energy_batched                                    */
@@ -491,9 +491,10 @@ int vdwdf_energy_noalloc(const vdwdf_grid *grid, const double *n_dev, const doub
  * path, on every k-th work item: about 16 items per warp slot spread over the
  * whole pair triangle) and write the fastest to *best: the one with the most
  * pair evaluations per millisecond of its second timed run.  The shape
- * is the fastest of those that a tuning can name.  The FP32 default (640
- * threads) is not one of them and measured faster on every workload, in
- * vdwdf_energy, vdwdf_potential and the batched path. */
+ * is the fastest of eight with 256 to 1024 threads.  The FP32 default (640
+ * threads; a NULL tuning, or threads = 0) is not one of them and measured
+ * faster on every workload, in vdwdf_energy, vdwdf_potential and the batched
+ * path: take it unless a measurement of your own says otherwise. */
 int vdwdf_autotune(const vdwdf_grid *grid, const double *n_dev, double n_cut, double r_cut,
                    const vdwdf_table *table, int precision, vdwdf_tuning *best,
                    void *cuda_stream);

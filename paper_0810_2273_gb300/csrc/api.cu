@@ -745,8 +745,8 @@ void fill_shared(const vdwdf_table *t, const TableDev &td, const Launch &ln,
 // A caller's launch shape: VDWDF_EINVAL outside the documented values,
 // VDWDF_EUNSUPPORTED for a thread count the skewed kernel is not built for.
 // The autotuner's candidate launch shapes (threads, items per warp slot, shared
-// band rows, band start): shapes that a caller's tuning can name.  The FP32 default
-// (640 threads) is not among them.
+// band rows, band start).  The FP32 default (640 threads, which a tuning takes as
+// threads = 0) is not among them; it is faster (see vdwdf_autotune).
 constexpr int kTuneCount = 8;
 constexpr vdwdf_tuning kTuneCandidates[kTuneCount] = {
     {256, 256, 0, -1}, {384, 256, 0, -1}, {448, 256, 0, -1}, {512, 256, 0, -1},

@@ -71,7 +71,7 @@ __device__ __forceinline__ double log1p_ratio(double a, double b) {
     p = fma(p, x, 1.0 / 3.0);
     return fma(static_cast<double>(k), 0.69314718055994530942, fma(p * x, w + w, w + w));
 }
-// exp(x) - 1 for 0 <= x < 30: the power of two taken out, the Taylor polynomial of
+// exp(x) - 1 for 0 <= x < 700 (237 at the largest density): the power of two taken out, the Taylor polynomial of
 // degree 14 of the rest (|r| <= ln 2 / 2, remainder 1e-19).
 __device__ __forceinline__ double expm1_taylor(double x) {
     const int k = static_cast<int>(static_cast<float>(x) * 1.44269504f + 0.5f);
@@ -129,7 +129,7 @@ struct CellRows {
 // Per-instance inputs of the pair kernel.
 struct PairParams {
     double h2[3];        // metric in index units, diagonal: |M_a|^2 / N_a^2
-    float h2f[3], g2f[3];  // h2 and g2x in FP32
+    float h2f[3], g2f[3];  // h2 (no less than the smallest normal number) and g2x in FP32
     double g2x[3];       // 2 x off-diagonal metric (01, 02, 12): r^2 = sum h2_a d_a^2
                          //   + g2x[0] d_0 d_1 + g2x[1] d_0 d_2 + g2x[2] d_1 d_2
     float cull_h2[3];    // culling metric: h2 on orthogonal cells, the smallest
@@ -171,7 +171,8 @@ struct LoopConsts {
 struct PairShared {
     const double *tab64;  // (nD + 2) x (nd + 2) B-spline coefficients / 36, D outer,
     const float *tab32;   // then nd + 2 coefficients / 6 of rho(delta) (beyond-table factor)
-    const double *poly64; // per D cell and delta column of tab64 its cubic in the cell (NULL: none)
+    const double *poly64; // per D cell and delta column of tab64 its cubic in the cell (NULL: none,
+                          // the sums then read tab64)
     int S;                // row stride (nd + 2)
     int nD, nd;
     double cD, cd;        // tD = r (q_i + q_j) cD,  td = |q_i - q_j|/(q_i + q_j) cd
@@ -184,8 +185,8 @@ struct PairShared {
                           // ks0 < 0: ks0 is inst[0].stats->band_row0 (set by launch_band_choose)
     unsigned long long tex32; // the bicubic coefficients of tab32 as a 2D texture (rows along D) for
                           // gathers; 0 when the table is too large for one
-    int itile, jpts;      // i points and j points per work item (j: a multiple of 8 in FP32, of
-                          // kTile in FP64)
+    int itile, jpts;      // i points and j points per work item (j: a multiple of kTile, or 16 in
+                          // FP32)
     unsigned int item_limit;  // process at most item_limit items (autotuning) ...
     unsigned int item_stride; // ... taking every item_stride-th one (1: all in order)
     unsigned int max_iters;   // cap on the work loop of one CTA
